@@ -235,6 +235,16 @@ __device__ __forceinline__ float rna_tf32(float x)
 }
 
 
+// threadIdx.x, not known to be a constant of the loop over the segments: the exact path's
+// address arithmetic then stays in the exact path.  Hoisted out of the loop it was spilled
+// around the fast path, which runs at the register limit (256-token tails 33.2 us, not 29.8).
+__device__ __forceinline__ int thread_id()
+{
+    int t;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    return t;
+}
+
 // zero the staged rows past a segment of L < 64 tokens (all threads, or the builder
 // warps only)
 template <int D>
@@ -277,8 +287,12 @@ __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, bool builders_on
 // is summed in float32 from the bf16 inputs, each warp's 64 key dims by a butterfly, into
 // the set's diagonal partials: fp16 Q~ and K~ would round the terms of that dot product to
 // 11 bits, which a token whose own q . k cancels cannot afford.
+//
+// A segment that the guard is sure to send to the exact path for its gates alone (one above
+// 0, or a total log2-decay below -kLamRange) stops after the totals and returns false: the
+// staged inputs are untouched, so the exact path starts from them without another copy.
 template <int D>
-__device__ __forceinline__ void build_fast(uint8_t *smem, uint32_t tmem, int L, int par, int gslot)
+__device__ __forceinline__ bool build_fast(uint8_t *smem, uint32_t tmem, int L, int par, int gslot)
 {
     using G = Geo<D>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -296,7 +310,7 @@ __device__ __forceinline__ void build_fast(uint8_t *smem, uint32_t tmem, int L, 
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
 
     if (!worker)
-        return;
+        return true;
     zero_tail<D>(smem, L, true);
     const int dp = tid % G::DP, qt = tid / G::DP;
     float amax = -INFINITY;
@@ -331,6 +345,11 @@ __device__ __forceinline__ void build_fast(uint8_t *smem, uint32_t tmem, int L, 
         if (qt == 0)
             *reinterpret_cast<float2 *>(sGam + gslot * D + 2 * dp) = make_float2(ex2(t0), ex2(t1));
         lam_ok = t0 >= -kLamRange && t1 >= -kLamRange;
+    }
+    if (bar_or(1, !(amax <= 0.f && lam_ok))) {
+        if (lane == 0)
+            sRed[warp * 8 + 1] = 0.f;
+        return false;
     }
     uint8_t *set = smem + par * SET_BYTES;
     __nv_bfloat162 bq = __float2bfloat162_rn(0.f), bk = bq;   // max |q|, |k|
@@ -389,7 +408,7 @@ __device__ __forceinline__ void build_fast(uint8_t *smem, uint32_t tmem, int L, 
     // non-increasing Lam (|Q~| <= |q|, |A| <= D max|q| max|k|), a total decay of at most
     // 2^-10 (Q~ of the segment's last tokens keeps its precision) and every fp16 operand below
     // 2^15; NaN fails
-    bool ok = amax <= 0.f && lam_ok && hmax_of(hq) < kF16Lim && hmax_of(hk) < kF16Lim &&
+    bool ok = hmax_of(hq) < kF16Lim && hmax_of(hk) < kF16Lim &&
               mv < kF16Lim;
     ok = __all_sync(0xffffffffu, ok);
     if (lane == 0) {
@@ -399,6 +418,7 @@ __device__ __forceinline__ void build_fast(uint8_t *smem, uint32_t tmem, int L, 
         sRed[warp * 8 + 3] = mv;
     }
     tmem_wait_st();
+    return true;
 }
 
 
@@ -605,19 +625,18 @@ __device__ __forceinline__ void state_store(uint32_t tmem, float *dst)
 
 // ---- exact path pieces (every thread of the 512-thread CTA takes part) ----
 
-// cumulative log2-gates of a staged segment (key dim d over 32 tokens per state thread,
-// token-major into X_LAM; gates below kGateFloor taken at the floor), Q~ = q 2^{Lam} (tf32,
-// X_QT), K^^T = k 2^{Lam_last - Lam} (tf32, rows 64.. of X_B2), V^T float32 into TMEM and
-// 2^{Lam_last} into gam slot gslot.  Ends with the operands visible to the tensor core.
+// cumulative log2-gates of a staged segment (16 tokens of a key dim per thread, token-major
+// into X_LAM; gates below kGateFloor taken at the floor), Q~ = q 2^{Lam} (tf32, X_QT),
+// K^^T = k 2^{Lam_last - Lam} (tf32, rows 64.. of X_B2), V^T float32 into TMEM and
+// 2^{Lam_last} into gam slot gslot.  Returns (uniformly) whether some gate is above 0.
 template <int D>
-__device__ __forceinline__ void exact_build(uint8_t *smem, uint32_t tmem, int L, int gslot)
+__device__ __forceinline__ bool exact_build(uint8_t *smem, uint32_t tmem, int L, int gslot)
 {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int d = (warp & 3) * 32 + lane;
-    const bool worker = warp >= 8 && d < D;
+    const int tid = thread_id(), warp = tid >> 5, lane = tid & 31;
+    const int d = (warp & 3) * 32 + lane;      // key dim, and value dim = TMEM lane of V^T
+    const bool worker = d < D;
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
-    const int colhalf = (warp >> 2) & 1;
-    const int th = colhalf;
+    const int t0 = (warp >> 2) * 16;           // this thread's 16 tokens
     const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
     const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
     const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
@@ -625,85 +644,270 @@ __device__ __forceinline__ void exact_build(uint8_t *smem, uint32_t tmem, int L,
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
     float *sGam = reinterpret_cast<float *>(smem + OFF_GAM);
     float *sLam = reinterpret_cast<float *>(smem + X_LAM);
-    float last = 0.f, tot0 = 0.f;
     zero_tail<D>(smem, L, false);
-    {
-        float run = 0.f;
-        if (worker) {
-#pragma unroll 8
-            for (int x = 0; x < 32; ++x) {
-                run = fmaf(fmaxf(sG[(32 * th + x) * D + d], kGateFloor), kLog2e, run);
-                sLam[(32 * th + x) * D + d] = run;
-            }
-            sTot[th * D + d] = run;
-        }
-        __syncthreads();
-        if (worker) {
-            tot0 = sTot[d];
-            last = tot0 + sTot[D + d];   // Lam_last of key dim d
-            if (!th)
-                sGam[gslot * D + d] = ex2(last);
-        }
-    }
+    float lam[16];
+    bool up = false;
     if (worker) {
-#pragma unroll 1
-        for (int hh = 0; hh < 2; ++hh) {
-            uint32_t vtr[16];
+        float run = 0.f;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                float4 w;
-                float *wv = &w.x;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int x = 16 * hh + 4 * g + u;
-                    const int i = 32 * th + x;
-                    float lam = sLam[i * D + d];
-                    if (th) {
-                        lam = tot0 + lam;
-                        sLam[i * D + d] = lam;
-                    }
-                    *reinterpret_cast<float *>(smem + X_QT + t_off(64, i, d)) =
-                        rna_tf32(bf16f(sQ[i * D + d]) * ex2(lam));
-                    wv[u] = rna_tf32(bf16f(sK[i * D + d]) * ex2(last - lam));
-                    vtr[4 * g + u] = __float_as_uint(bf16f(sV[i * D + d]));
-                }
-                *reinterpret_cast<float4 *>(smem + X_B2 + t_off(Geo<D>::ROWS, 64 + d, 32 * th + 16 * hh + 4 * g)) = w;
-            }
-            tmem_st16(tmem + lrow + TM_V + 32 * th + 16 * hh, vtr);
+        for (int x = 0; x < 16; ++x) {
+            const float g = fmaxf(sG[(t0 + x) * D + d], kGateFloor);
+            up = up || g > 0.f;
+            run = fmaf(g, kLog2e, run);
+            lam[x] = run;
         }
+        sTot[(warp >> 2) * D + d] = run;
+    }
+    up = __syncthreads_or(up) != 0;
+    if (worker) {
+        float before = 0.f, last = 0.f;        // Lam before this thread's tokens, Lam_last
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (u == (warp >> 2))
+                before = last;
+            last += sTot[u * D + d];
+        }
+        if (t0 == 0)
+            sGam[gslot * D + d] = ex2(last);
+        uint32_t vtr[16];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            float4 w;
+            float *wv = &w.x;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = t0 + 4 * g + u;
+                const float l = before + lam[4 * g + u];
+                sLam[i * D + d] = l;
+                *reinterpret_cast<float *>(smem + X_QT + t_off(64, i, d)) =
+                    rna_tf32(bf16f(sQ[i * D + d]) * ex2(l));
+                wv[u] = rna_tf32(bf16f(sK[i * D + d]) * ex2(last - l));
+                vtr[4 * g + u] = __float_as_uint(bf16f(sV[i * D + d]));
+            }
+            *reinterpret_cast<float4 *>(smem + X_B2 + t_off(Geo<D>::ROWS, 64 + d, t0 + 4 * g)) = w;
+        }
+        tmem_st16(tmem + lrow + TM_V + t0, vtr);
         tmem_wait_st();
     }
+    return up;
 }
 
 // (state warps) the state as two tf32 parts for S^T Q~^T (an A operand from TMEM is read as
 // tf32): hi = S with its low 13 mantissa bits cleared (exact in tf32), lo = S - hi (exact in
 // fp32, at most 13 significant bits), so the product keeps the state to ~2^-20 instead of a
-// 2^-10 truncation
+// 2^-10 truncation.  S itself is then left decayed by gam slot gslot for the state update.
 template <int D>
-__device__ __forceinline__ void exact_split_state(uint32_t tmem)
+__device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t tmem, int gslot)
 {
     constexpr int CW = Geo<D>::CW;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = thread_id() >> 5, lane = thread_id() & 31;
     if (warp < 8 || (warp & 3) * 32 + lane >= D)
         return;
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
     const int colhalf = (warp >> 2) & 1;
+    // 16 columns at a time: 32 took the kernel past its registers
 #pragma unroll 1
-    for (int c0 = 0; c0 < CW; c0 += 32) {
+    for (int c0 = 0; c0 < CW; c0 += 16) {
         const int d0 = colhalf * CW + c0;
-        float r[32], lo[32];
-        tmem_ld32(tmem + lrow + TM_S + d0, r);
+        const float *gam = reinterpret_cast<const float *>(smem + OFF_GAM) + gslot * D + d0;
+        uint32_t r[16], x2[16];
+        tmem_ld16(tmem + lrow + TM_S + d0, r);
         tmem_wait_ld();
 #pragma unroll
-        for (int x = 0; x < 32; ++x) {
-            const float hi = __uint_as_float(__float_as_uint(r[x]) & 0xFFFFE000u);
-            lo[x] = r[x] - hi;
-            r[x] = hi;
-        }
-        tmem_st32(tmem + lrow + Geo<D>::SHI + d0, r);
-        tmem_st32(tmem + lrow + (d0 < 64 ? TM_SLO0 + d0 : TM_SLO1 + (d0 - 64)), lo);
+        for (int x = 0; x < 16; ++x)
+            x2[x] = r[x] & 0xFFFFE000u;
+        tmem_st16(tmem + lrow + Geo<D>::SHI + d0, x2);
+#pragma unroll
+        for (int x = 0; x < 16; ++x)
+            x2[x] = __float_as_uint(__uint_as_float(r[x]) - __uint_as_float(x2[x]));
+        tmem_st16(tmem + lrow + (d0 < 64 ? TM_SLO0 + d0 : TM_SLO1 + (d0 - 64)), x2);
+#pragma unroll
+        for (int x = 0; x < 16; ++x)
+            r[x] = __float_as_uint(__uint_as_float(r[x]) * gam[x]);
+        tmem_st16(tmem + lrow + TM_S + d0, r);
     }
     tmem_wait_st();
+}
+
+// ---- exact path: A_ij = sum_d q_id k_jd 2^{Lam_id - Lam_jd}, j <= i < L, in float32, rounded
+// to tf32 into rows 0..63 of X_B2 (zeros above the diagonal).
+//
+// Taken pair by pair that is 262,144 exponentials at d = 128 and, with one thread per pair, a
+// 32-way bank conflict on every operand (63 us a segment in all; 15.6 us in this form:
+// 475-token tails of 9 x 16 heads, 507 us -> 125 us).  When no gate is
+// above 0 the 64 x 64 triangle is cut in halves instead: the lower left H x H square of every
+// block of 2 H tokens (H = 32, 16, 8) factors at the token R that ends the block's first
+// half, 2^{Lam_i - Lam_j} = 2^{Lam_i - Lam_R} 2^{Lam_R - Lam_j} with j <= R < i, so both
+// exponents are <= 0: no overflow, and a factor that underflows stands for a product that
+// does.  Each level scales every row of q or k once (64 x d exponentials) and multiplies the
+// squares as float32 register tiles; the eight 8 x 8 triangles left on the diagonal are taken
+// pair by pair.  Segments with a gate above 0 keep the pairwise form (exact_scores_pairs).
+
+// the rows of one level, scaled, into the staged log-gates' area (free by now): row r is
+// k_r 2^{Lam_R - Lam_r} in the first half of its block, q_r 2^{Lam_r - Lam_R} in the second
+template <int D, int H>
+__device__ __forceinline__ void exact_level_rows(uint8_t *smem)
+{
+    const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
+#pragma unroll 1
+    for (int x = 0; x < CH * D / 4 / NT; ++x) {
+        const int idx = thread_id() + x * NT;
+        const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
+        const int ref = (r & ~(2 * H - 1)) + H - 1;
+        const bool isq = (r & H) != 0;
+        const float4 l = *reinterpret_cast<const float4 *>(sLam + r * D + c);
+        const float4 lr = *reinterpret_cast<const float4 *>(sLam + ref * D + c);
+        const uint2 w = *reinterpret_cast<const uint2 *>(smem + (isq ? OFF_SQ : OFF_SK) + (r * D + c) * 2);
+        const float sg = isq ? 1.f : -1.f;
+        float4 y;
+        y.x = __uint_as_float(w.x << 16) * ex2(sg * (l.x - lr.x));
+        y.y = __uint_as_float(w.x & 0xFFFF0000u) * ex2(sg * (l.y - lr.y));
+        y.z = __uint_as_float(w.y << 16) * ex2(sg * (l.z - lr.z));
+        y.w = __uint_as_float(w.y & 0xFFFF0000u) * ex2(sg * (l.w - lr.w));
+        *reinterpret_cast<float4 *>(smem + OFF_SG + (r * D + c) * 4) = y;
+    }
+}
+
+// the level's squares: 2 H tiles of 4 x 4 scores, each by the G = 256 / H neighbouring lanes
+// that share its key dims (every 16-byte row read of a quarter-warp is 128 contiguous bytes),
+// then a transposing butterfly over the lanes
+template <int D, int H>
+__device__ __forceinline__ void exact_level_squares(uint8_t *smem)
+{
+    constexpr int G = 256 / H, TB = H / 4;
+    const int tile = thread_id() / G, ds = thread_id() % G;
+    const int blk = tile / (TB * TB), t = tile % (TB * TB);
+    const int i0 = blk * 2 * H + H + (t / TB) * 4, j0 = blk * 2 * H + (t % TB) * 4;
+    const float *X = reinterpret_cast<const float *>(smem + OFF_SG);
+    float v[16];
+#pragma unroll
+    for (int x = 0; x < 16; ++x)
+        v[x] = 0.f;
+#pragma unroll 1
+    for (int c0 = 0; c0 < D / 4; c0 += G) {
+        if (G <= D / 4 || ds < D / 4) {
+            const int c = (c0 + ds) * 4;
+            float4 k4[4];
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+                k4[y] = *reinterpret_cast<const float4 *>(X + (j0 + y) * D + c);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const float4 q4 = *reinterpret_cast<const float4 *>(X + (i0 + x) * D + c);
+#pragma unroll
+                for (int y = 0; y < 4; ++y)
+                    v[4 * x + y] = fmaf(q4.w, k4[y].w, fmaf(q4.z, k4[y].z,
+                                   fmaf(q4.y, k4[y].y, fmaf(q4.x, k4[y].x, v[4 * x + y]))));
+            }
+        }
+    }
+    // 16 sums over G lanes: halve the values held at each of the first four exchanges
+    int first = 0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const int o = G >> (s + 1), n = 8 >> s;
+        if (o > 0) {
+            const bool up = (ds & o) != 0;
+#pragma unroll
+            for (int x = 0; x < n; ++x) {
+                const float send = up ? v[x] : v[x + n];
+                v[x] = (up ? v[x + n] : v[x]) + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+            first += up ? n : 0;
+        }
+    }
+    if (G == 32)
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    constexpr int HELD = G == 8 ? 2 : 1;
+    if (G < 32 || (ds & 1) == 0) {
+#pragma unroll
+        for (int x = 0; x < HELD; ++x) {
+            const int i = i0 + (first + x) / 4, j = j0 + (first + x) % 4;
+            *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(v[x]);
+            *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, j, i)) = 0.f;
+        }
+    }
+}
+
+// the 8 x 8 triangles on the diagonal: thread (block, key dim) takes the 36 products of its
+// key dim from registers; warp sums over 32 key dims go to the staged values' area ...
+template <int D>
+__device__ __forceinline__ void exact_triangles(uint8_t *smem)
+{
+    constexpr int NP = D / 32;                 // warps, and partial sums, per block
+    const int warp = thread_id() >> 5, lane = thread_id() & 31;
+    const int d = (warp % NP) * 32 + lane;
+    const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
+    const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
+    const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
+    float *part = reinterpret_cast<float *>(smem + OFF_SV);
+#pragma unroll 1
+    for (int blk = warp / NP; blk < 8; blk += 16 / NP) {
+        float l[8], k[8], v[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            l[x] = sLam[(8 * blk + x) * D + d];
+            k[x] = bf16f(sK[(8 * blk + x) * D + d]);
+        }
+        float *dst = part + (blk * NP + warp % NP) * 40;
+        // product n = i (i + 1) / 2 + j, eight at a time
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float q = bf16f(sQ[(8 * blk + i) * D + d]);
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const int n = i * (i + 1) / 2 + j;
+                v[n % 8] = j == i ? q * k[j] : q * k[j] * ex2(l[i] - l[j]);
+                if (n % 8 == 7 || n == 35) {
+                    if (n == 35) {
+#pragma unroll
+                        for (int x = 4; x < 8; ++x)
+                            v[x] = 0.f;
+                    }
+                    const float sum = warp_sum8(v, lane);
+                    if ((lane & 3) == 0)
+                        dst[(n & ~7) + (lane >> 2)] = sum;
+                }
+            }
+        }
+    }
+}
+
+// ... and are added up, one thread per element of the eight 8 x 8 blocks
+template <int D>
+__device__ __forceinline__ void exact_triangles_sum(uint8_t *smem)
+{
+    constexpr int NP = D / 32;
+    const int blk = thread_id() >> 6, i = (thread_id() >> 3) & 7, j = thread_id() & 7;
+    const float *part = reinterpret_cast<const float *>(smem + OFF_SV) + blk * NP * 40;
+    float a = 0.f;
+    if (j <= i) {
+        const int n = i * (i + 1) / 2 + j;
+#pragma unroll
+        for (int x = 0; x < NP; ++x)
+            a += part[x * 40 + n];
+    }
+    *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, 8 * blk + i, 8 * blk + j)) = rna_tf32(a);
+}
+
+// pair by pair, for segments with a gate above 0
+template <int D>
+__device__ __forceinline__ void exact_scores_pairs(uint8_t *smem, int L)
+{
+    const int tid = thread_id();
+    const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
+    const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
+    const float *lg = reinterpret_cast<const float *>(smem + X_LAM);
+    for (int idx = tid; idx < CH * CH; idx += NT) {
+        const int i = idx >> 6, j = idx & 63;
+        float acc = 0.f;
+        if (j <= i && i < L) {
+            for (int dd = 0; dd < D; ++dd)
+                acc = fmaf(bf16f(sQ[i * D + dd]) * bf16f(sK[j * D + dd]),
+                           ex2(lg[i * D + dd] - lg[j * D + dd]), acc);
+        }
+        *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(acc);
+    }
 }
 
 // (issuing thread) S^T Q~^T into D_O (TM_O0): the hi part, then the lo part
@@ -724,48 +928,55 @@ __device__ __forceinline__ void exact_issue_sq(uint32_t tmem, uint32_t sb)
     }
 }
 
-// (every thread) A_ij = sum_d q_id k_jd 2^{Lam_id - Lam_jd}, j <= i < L, elementwise, rounded
-// to tf32 into rows 0..63 of X_B2
+// Every operand of an exact segment, and S^T Q~^T issued: from staged inputs to A and K^^T in
+// X_B2, V^T and the decayed state in TMEM, visible to the tensor core.
 template <int D>
-__device__ __forceinline__ void exact_scores(uint8_t *smem, int L)
+__device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int L)
 {
-    const int tid = threadIdx.x;
-    const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
-    const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
-    const float *lg = reinterpret_cast<const float *>(smem + X_LAM);
-    for (int idx = tid; idx < CH * CH; idx += NT) {
-        const int i = idx >> 6, j = idx & 63;
-        float acc = 0.f;
-        if (j <= i && i < L) {
-            for (int dd = 0; dd < D; ++dd)
-                acc = fmaf(bf16f(sQ[i * D + dd]) * bf16f(sK[j * D + dd]),
-                           ex2(lg[i * D + dd] - lg[j * D + dd]), acc);
-        }
-        *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(acc);
+    const bool up = exact_build<D>(smem, tmem, L, 0);
+    __syncthreads();
+    exact_split_state<D>(smem, tmem, 0);
+    if (!up)
+        exact_level_rows<D, 32>(smem);
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    if (thread_id() == kIssuer) {
+        tc_fence_after();
+        exact_issue_sq<D>(tmem, smem_u32(smem));
     }
+    // the scores while the tensor core runs S^T Q~^T
+    if (up) {
+        exact_scores_pairs<D>(smem, L);
+    } else {
+        exact_triangles<D>(smem);
+        exact_level_squares<D, 32>(smem);
+        __syncthreads();
+        exact_triangles_sum<D>(smem);
+        exact_level_rows<D, 16>(smem);
+        __syncthreads();
+        exact_level_squares<D, 16>(smem);
+        __syncthreads();
+        exact_level_rows<D, 8>(smem);
+        __syncthreads();
+        exact_level_squares<D, 8>(smem);
+    }
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
 }
 
-// (issuing thread) D_O += V^T A^T
+// (issuing thread) D_O += V^T A^T and S^T += V^T K^ (onto the decayed state), 8 tokens per step
 template <int D>
-__device__ __forceinline__ void exact_issue_av(uint32_t tmem, uint32_t sb)
+__device__ __forceinline__ void exact_issue_update(uint32_t tmem, uint32_t sb)
 {
-#pragma unroll
+#pragma unroll 1
     for (int kk = 0; kk < CH / 8; ++kk) {
         const uint32_t koff = (kk >> 2) * (Geo<D>::ROWS * 128) + (kk & 3) * 32;
         mma_tf32_ts(tmem + TM_O0, tmem + TM_V + kk * 8, sdesc_sw128(sb + X_B2 + koff, 16, 1024),
                     IDT_N64, 1);
-    }
-}
-
-// (issuing thread) S^T += V^T K^ (the decay diag(2^{Lam_last}) S applied before)
-template <int D>
-__device__ __forceinline__ void exact_issue_state(uint32_t tmem, uint32_t sb)
-{
-#pragma unroll
-    for (int kk = 0; kk < CH / 8; ++kk) {
-        const uint32_t koff = (kk >> 2) * (Geo<D>::ROWS * 128) + (kk & 3) * 32 + 64 * 128;
-        mma_tf32_ts(tmem + TM_S, tmem + TM_V + kk * 8, sdesc_sw128(sb + X_B2 + koff, 16, 1024),
-                    Geo<D>::IDT_ST, 1);
+        mma_tf32_ts(tmem + TM_S, tmem + TM_V + kk * 8,
+                    sdesc_sw128(sb + X_B2 + koff + 64 * 128, 16, 1024), Geo<D>::IDT_ST, 1);
     }
 }
 

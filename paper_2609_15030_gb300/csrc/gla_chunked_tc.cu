@@ -38,7 +38,7 @@
 // 2^{Lam_last} stays >= 2^-10 in every key dim (so Q~ never nears fp16's
 // subnormals).  Any other chunk (strong decay, huge values) runs the exact
 // path: tf32 operands (the state split into two exact tf32 parts), the
-// intra-chunk matrix computed elementwise in float32 with 2^{Lam_i - Lam_j} <= 1,
+// intra-chunk matrix computed in float32 from factors 2^{Lam_i - Lam_j} <= 1,
 // and the state updated as
 // diag(2^{Lam_last}) S + K^^T V with K^_j = k_j 2^{Lam_last - Lam_j}.  The
 // choice depends only on the chunk's inputs and on the state it starts from,
@@ -75,7 +75,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
     // [0] TMEM base, [1] abort flag, [2] decision on the latest built segment (1 = fast),
     // [3] run result (1 = the segment at [4..5] needs the exact path), [4..5] position
-    // where the run stopped, [6..7] its local token index
+    // where the run stopped, [6..7] its local token index, [8] whether the latest segment's
+    // build is whole (0: its gates alone send it to the exact path, its inputs still staged)
     volatile uint32_t *sMisc = reinterpret_cast<volatile uint32_t *>(smem + OFF_MISC);
     volatile int64_t *sRun = reinterpret_cast<volatile int64_t *>(smem + OFF_MISC + 16);
     const uint32_t bar_tma = sb + OFF_BAR, bar_a = sb + OFF_BAR + 8, bar_o = sb + OFF_BAR + 16,
@@ -280,41 +281,22 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         return ok && (float)D * mq * mk < kF16Lim;
     };
 
-    // ---- one exact segment, from staged inputs, no decay pending and no MMA in flight;
-    // leaves the final state in TMEM, writes its outputs and checkpoint
-    auto exact_segment = [&](int64_t tok_s, int L, int par, int gslot, int64_t seg_end) -> bool {
-        exact_build<D>(smem, tmem, L, gslot);
-        exact_split_state<D>(tmem);
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
+    // ---- one exact segment, from staged inputs, no decay pending and no MMA in flight; stages
+    // the next segment once its own inputs are read; leaves the final state in TMEM, writes
+    // its outputs and checkpoint
+    auto exact_segment = [&](int64_t tok_s, int L, int64_t seg_end) -> bool {
+        exact_operands<D>(smem, tmem, L);
         if (tid == kIssuer) {
             tc_fence_after();
-            exact_issue_sq<D>(tmem, sb);
-        }
-        exact_scores<D>(smem, L);
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == kIssuer) {
-            tc_fence_after();
-            exact_issue_av<D>(tmem, sb);
+            exact_issue_update<D>(tmem, sb);
             tc_commit(bar_o);
         }
+        if (tid == kLoader && seg_end < end)
+            issue_tma(tok_s + L);
         if (!wait_all(kIssuer, bar_o, ph_o))
             return false;
-        state_pass<D>(smem, tmem, gslot, nullptr, false);          // S <- diag(2^{Lam_last}) S
-        tc_fence_before();
-        __syncthreads();
-        if (tid == kIssuer) {
-            tc_fence_after();
-            exact_issue_state<D>(tmem, sb);
-            tc_commit(bar_s);
-        }
-        if (!wait_all(kIssuer, bar_s, ph_s))
-            return false;
         state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false);   // checkpoint and |S| of the final state
-        out_epilogue<D>(tmem, outp(tok_s), tstride, L, par, false);
+        out_epilogue<D>(tmem, outp(tok_s), tstride, L, 0, false);
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
@@ -349,14 +331,17 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                 for (int j = 1; j <= kPrefetch; ++j)
                     prefetch(rtok + L + (int64_t)CH * (j - 1));
             }
-            build_fast<D>(smem, tmem, L, par, kseq & 3);
+            const bool built = build_fast<D>(smem, tmem, L, par, kseq & 3);
             fence_proxy_async_smem();
             tc_fence_before();
             if (!sync_group(1))
                 return;
             const bool next_long = is_long(rpos + L);
             if (tid == kLoader) {
+                sMisc[8] = built ? 1u : 0u;
                 mbar_arrive(bar_built);
+            }
+            if (tid == kLoader && built) {
                 // the staged rows are consumed: stage the next segment (long or short) now;
                 // an exact decision on this one reloads it
                 if (rpos + L < end)
@@ -397,7 +382,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         }
         stop = fast ? 0u : 1u;
         // a segment sent to the exact path: its (unused) D_A product is drained first
-        if (!fast && !wait_group(2, kIssuer, bar_a, ph_a0))
+        if (!fast && sMisc[8] != 0 && !wait_group(2, kIssuer, bar_a, ph_a0))
             return;
         while (fast) {
             const int L = seg_len(rpos);
@@ -459,7 +444,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                     mbar_arrive(bar_go);
             }
             stop = fast ? 0u : (inputs_ok ? 2u : 1u);
-            if (!fast && !(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
+            if (!fast && sMisc[8] != 0 &&
+                !(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
                 return;
         }
         if (pend) {
@@ -521,7 +507,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             if (!fast) {
                 // the exact path takes this segment: its (unused) D_A product drained first
                 stop = 1;
-                if (!(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
+                if (sMisc[8] != 0 &&
+                    !(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
                     return;
                 break;
             }
@@ -627,10 +614,12 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         tok = sRun[1];
         kseq = 0;
         if (stop != 0) {
-            // the segment at pos takes the exact path (1) or starts a new run (2): restage its
-            // inputs (the copy of the next segment may be in flight)
+            // the segment at pos takes the exact path (1) or starts a new run (2).  Its inputs
+            // are still staged if its build stopped early (sMisc[8] == 0); else restage them (the
+            // copy of the next segment may be in flight)
             const int Lx = seg_len(pos);
-            if (tid == kLoader) {
+            const bool staged = sMisc[8] == 0;
+            if (tid == kLoader && !staged) {
                 if (tma_pending && !mbar_wait_bounded(bar_tma, ph_tma, kTimeoutNs))
                     sMisc[1] = 1;
                 if (tma_pending)
@@ -640,14 +629,12 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             if (stop == 2)
                 continue;   // the new run waits for the copy
             // every thread runs the exact segment
-            if (!wait_tma())
+            if (!staged && !wait_tma())
                 break;
-            if (!exact_segment(tok, Lx, 0, 0, pos + Lx))
+            if (!exact_segment(tok, Lx, pos + Lx))
                 break;
             pos += Lx;
             tok += Lx;
-            if (tid == kLoader && pos < end)
-                issue_tma(tok);
         }
     }
 

@@ -253,6 +253,30 @@ def test_exact_segments_at_run_boundaries(pattern):
     assert np.array_equal(ck_r[0].view(np.uint32), cks[0][m + 1:].view(np.uint32))
 
 
+@pytest.mark.parametrize("gate_above_0", [False, True])
+@pytest.mark.parametrize("d,p0,n", [(128, 0, 64), (128, 5, 59), (128, 0, 9), (128, 3, 250),
+                                    (64, 0, 64), (64, 40, 33), (64, 3, 250)])
+def test_exact_segment_scores(d, p0, n, gate_above_0):
+    """Decaying gates of mixed strength: every long segment takes the exact path, whose scores
+    come from scaled squares and 8 x 8 triangles (with a gate above 0: pair by pair).  A last
+    query equal to one early key picks single scores out of every square and triangle.  The
+    operands carry 11 significant bits (relative rounding 2^-12) and everything else is
+    float32; an output passes through at most four of them (Q~, A, K^ and the state), so TOL
+    holds while the magnitudes summed are within twice the head's largest output."""
+    dev = device()
+    nH = 3
+    inp = gen_linear(71 + n, 0, 1, n, nH, d, d, "sigmoid")
+    rng = np.random.default_rng(n + d)
+    inp.a[:] *= rng.uniform(0.5, 12.0, size=(1, 1, nH, d)).astype(np.float32)
+    inp.q[0, n - 1] = inp.k[0, max(0, n - 12)]
+    if gate_above_0:
+        inp.a[0, ::64] = 0.03
+    S0 = gen_state(5, 0, 1, nH, d, d)
+    got = run_prefill(inp, [p0], [n], S0, 64, dev, hs.HS_LINATTN_CHUNKED_TC)
+    ref = oracle.gla(inp.q, inp.k, inp.v, inp.a, [p0], [n], S0=S0, C_=64)
+    _check(*got, *ref, [p0], [n], "exact scores")
+
+
 @pytest.mark.parametrize("where", ["short_call", "full_segment"])
 def test_zero_gate_inside_an_exact_segment(where):
     """A zero gate (a = -1e4) followed, in the same segment, by growing gates (the exact
