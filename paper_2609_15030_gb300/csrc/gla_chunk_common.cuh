@@ -105,7 +105,7 @@ struct Geo {
     static constexpr uint32_t O1 = TM_S + D;      // D_O of odd chunks, right of S^T
     static constexpr uint32_t SHI = TM_S + D;     // exact path: hi part of S^T
     static constexpr uint32_t IDF_ST = idesc_f16(128, D, 1);       // S^T += V^T K~ (K~ read MN-major)
-    static constexpr uint32_t IDT_ST = idesc_tf32(128, D, 0, 0);   // exact: S^T += V^T K^
+    static constexpr uint32_t IDT_UP = idesc_tf32(128, 64 + D, 0, 0);   // exact: [D_O | S^T] update
     static constexpr uint32_t STAGE = 3 * CH * D * 2 + CH * D * 4;  // staged q, k, v, log-gates
 };
 
@@ -625,21 +625,26 @@ __device__ __forceinline__ void state_store(uint32_t tmem, float *dst)
 
 // ---- exact path pieces (every thread of the 512-thread CTA takes part) ----
 
-// cumulative log2-gates of a staged segment (16 tokens of a key dim per thread, token-major
-// into X_LAM; gates below kGateFloor taken at the floor), Q~ = q 2^{Lam} (tf32, X_QT),
-// K^^T = k 2^{Lam_last - Lam} (tf32, rows 64.. of X_B2), V^T float32 into TMEM and
-// 2^{Lam_last} into gam slot gslot.  Returns (uniformly) whether some gate is above 0.
+// element (token, key dim) of X_LAM, in floats: token-major, the 16-byte chunks of odd tokens
+// swapped in pairs so that the fragment loads of exact_square (16 bytes from each of two
+// neighbouring rows per quarter-warp) meet no bank twice
 template <int D>
-__device__ __forceinline__ bool exact_build(uint8_t *smem, uint32_t tmem, int L, int gslot)
+__device__ __forceinline__ int lam_at(int row, int d)
+{
+    return row * D + (d ^ ((row & 1) << 2));
+}
+
+// cumulative log2-gates of a staged segment (16 tokens of a key dim per thread, into X_LAM;
+// gates below kGateFloor taken at the floor), Q~ = q 2^{Lam} (tf32, X_QT) and 2^{Lam_last} into
+// gam slot 0.  Returns (uniformly) whether some gate is above 0.
+template <int D>
+__device__ __forceinline__ bool exact_decay(uint8_t *smem, int L)
 {
     const int tid = thread_id(), warp = tid >> 5, lane = tid & 31;
-    const int d = (warp & 3) * 32 + lane;      // key dim, and value dim = TMEM lane of V^T
+    const int d = (warp & 3) * 32 + lane;
     const bool worker = d < D;
-    const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
     const int t0 = (warp >> 2) * 16;           // this thread's 16 tokens
     const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
-    const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
-    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
     const float *sG = reinterpret_cast<const float *>(smem + OFF_SG);
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
     float *sGam = reinterpret_cast<float *>(smem + OFF_GAM);
@@ -668,7 +673,33 @@ __device__ __forceinline__ bool exact_build(uint8_t *smem, uint32_t tmem, int L,
             last += sTot[u * D + d];
         }
         if (t0 == 0)
-            sGam[gslot * D + d] = ex2(last);
+            sGam[d] = ex2(last);
+#pragma unroll
+        for (int x = 0; x < 16; ++x) {
+            const float l = before + lam[x];
+            sLam[lam_at<D>(t0 + x, d)] = l;
+            *reinterpret_cast<float *>(smem + X_QT + t_off(64, t0 + x, d)) =
+                rna_tf32(bf16f(sQ[(t0 + x) * D + d]) * ex2(l));
+        }
+    }
+    return up;
+}
+
+// (builder warps) K^^T = k 2^{Lam_last - Lam} (tf32, rows 64.. of X_B2) and V^T float32 into TMEM
+template <int D>
+__device__ __forceinline__ void exact_keys_values(uint8_t *smem, uint32_t tmem)
+{
+    const int warp = thread_id() >> 5, lane = thread_id() & 31;
+    const int d = (warp & 3) * 32 + lane;      // key dim, and value dim = TMEM lane of V^T
+    if (warp >= 8 || d >= D)
+        return;
+    const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
+    const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
+    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
+    const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
+    const float last = sLam[lam_at<D>(CH - 1, d)];
+#pragma unroll 1
+    for (int t0 = (warp >> 2) * 32; t0 < (warp >> 2) * 32 + 32; t0 += 16) {
         uint32_t vtr[16];
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
@@ -677,27 +708,22 @@ __device__ __forceinline__ bool exact_build(uint8_t *smem, uint32_t tmem, int L,
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int i = t0 + 4 * g + u;
-                const float l = before + lam[4 * g + u];
-                sLam[i * D + d] = l;
-                *reinterpret_cast<float *>(smem + X_QT + t_off(64, i, d)) =
-                    rna_tf32(bf16f(sQ[i * D + d]) * ex2(l));
-                wv[u] = rna_tf32(bf16f(sK[i * D + d]) * ex2(last - l));
+                wv[u] = rna_tf32(bf16f(sK[i * D + d]) * ex2(last - sLam[lam_at<D>(i, d)]));
                 vtr[4 * g + u] = __float_as_uint(bf16f(sV[i * D + d]));
             }
             *reinterpret_cast<float4 *>(smem + X_B2 + t_off(Geo<D>::ROWS, 64 + d, t0 + 4 * g)) = w;
         }
         tmem_st16(tmem + lrow + TM_V + t0, vtr);
-        tmem_wait_st();
     }
-    return up;
+    tmem_wait_st();
 }
 
 // (state warps) the state as two tf32 parts for S^T Q~^T (an A operand from TMEM is read as
 // tf32): hi = S with its low 13 mantissa bits cleared (exact in tf32), lo = S - hi (exact in
 // fp32, at most 13 significant bits), so the product keeps the state to ~2^-20 instead of a
-// 2^-10 truncation.  S itself is then left decayed by gam slot gslot for the state update.
+// 2^-10 truncation.  S itself is then left decayed by gam slot 0 for the state update.
 template <int D>
-__device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t tmem, int gslot)
+__device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t tmem)
 {
     constexpr int CW = Geo<D>::CW;
     const int warp = thread_id() >> 5, lane = thread_id() & 31;
@@ -709,7 +735,7 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 #pragma unroll 1
     for (int c0 = 0; c0 < CW; c0 += 16) {
         const int d0 = colhalf * CW + c0;
-        const float *gam = reinterpret_cast<const float *>(smem + OFF_GAM) + gslot * D + d0;
+        const float *gam = reinterpret_cast<const float *>(smem + OFF_GAM) + d0;
         uint32_t r[16], x2[16];
         tmem_ld16(tmem + lrow + TM_S + d0, r);
         tmem_wait_ld();
@@ -733,161 +759,294 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 // to tf32 into rows 0..63 of X_B2 (zeros above the diagonal).
 //
 // Taken pair by pair that is 262,144 exponentials at d = 128 and, with one thread per pair, a
-// 32-way bank conflict on every operand (63 us a segment in all; 15.6 us in this form:
-// 475-token tails of 9 x 16 heads, 507 us -> 125 us).  When no gate is
-// above 0 the 64 x 64 triangle is cut in halves instead: the lower left H x H square of every
-// block of 2 H tokens (H = 32, 16, 8) factors at the token R that ends the block's first
-// half, 2^{Lam_i - Lam_j} = 2^{Lam_i - Lam_R} 2^{Lam_R - Lam_j} with j <= R < i, so both
-// exponents are <= 0: no overflow, and a factor that underflows stands for a product that
-// does.  Each level scales every row of q or k once (64 x d exponentials) and multiplies the
-// squares as float32 register tiles; the eight 8 x 8 triangles left on the diagonal are taken
-// pair by pair.  Segments with a gate above 0 keep the pairwise form (exact_scores_pairs).
+// 32-way bank conflict on every operand.  When no gate is above 0 the 64 x 64 triangle is cut
+// in halves instead: the lower left H x H square of every block of 2 H tokens (H = 32, 16, 8)
+// factors at the token R that ends the block's first half, 2^{Lam_i - Lam_j} =
+// 2^{Lam_i - Lam_R} 2^{Lam_R - Lam_j} with j <= R < i, so both exponents are <= 0: no overflow,
+// and a factor that underflows stands for a product that does.  The factors are formed in
+// registers as matrix fragments and split into two tf32 parts each, so that a product keeps
+// ~2^-21 (three tf32 products, float32 sums).  The eight 8 x 8 triangles left on the diagonal
+// are taken pair by pair.  The tasks (one warp each, drawn from a shared counter, the long ones
+// first) are halves of the key dims of four 16 x 16 units (a square of H = 16, or two of H = 8),
+// quarters of those of each half of the 32 x 32 square, and 64 key dims of a triangle.  Meanwhile the
+// issuing thread's warp feeds S^T Q~^T to the tensor core, about 6 k cycles of dependent products,
+// which the tasks about fill.  Segments with a gate above 0 keep the pairwise form
+// (exact_scores_pairs).
 
-// the rows of one level, scaled, into the staged log-gates' area (free by now): row r is
-// k_r 2^{Lam_R - Lam_r} in the first half of its block, q_r 2^{Lam_r - Lam_R} in the second
-template <int D, int H>
-__device__ __forceinline__ void exact_level_rows(uint8_t *smem)
+// a 16 x 16 unit's rows: query rows r0.. and r1.. (8 each), key rows c0.. and c1.., and the
+// tokens R that (r0, c0) and (r1, c1) factor at; units 2 and 3 hold two squares of H = 8, in
+// the quadrants (r0, c0) and (r1, c1)
+struct SquareUnit {
+    int r0, r1, c0, c1, ref0, ref1;
+};
+
+__device__ __forceinline__ SquareUnit square_unit(int u)
+{
+    SquareUnit m;
+    m.c0 = 32 * (u & 1);
+    m.r0 = m.c0 + (u < 2 ? 16 : 8);
+    m.c1 = m.c0 + (u < 2 ? 8 : 16);
+    m.r1 = m.c0 + 24;
+    m.ref0 = m.c0 + (u < 2 ? 15 : 7);
+    m.ref1 = m.c0 + (u < 2 ? 15 : 23);
+    return m;
+}
+
+// partial sums of the tasks, in the staged log-gates' area (free by then)
+constexpr uint32_t X_P32 = OFF_SG;             // 32 x 32 square [4 quarters][32][32]     16 KiB
+constexpr uint32_t X_P16 = OFF_SG + 16384;     // units [4][2 halves][16][16]              8 KiB
+constexpr uint32_t X_PTR = OFF_SG + 24576;     // triangles [8][d / 64][40]              2.5 KiB
+
+// four factors x 2^{+-(l - lr)} of one row (key dims kk..kk+3), x in bf16, lr given
+template <int D, int SIGN>
+__device__ __forceinline__ void factors4(const uint8_t *smem, uint32_t off, int row, const float4 &r,
+                                         int kk, float *y)
 {
     const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
-#pragma unroll 1
-    for (int x = 0; x < CH * D / 4 / NT; ++x) {
-        const int idx = thread_id() + x * NT;
-        const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
-        const int ref = (r & ~(2 * H - 1)) + H - 1;
-        const bool isq = (r & H) != 0;
-        const float4 l = *reinterpret_cast<const float4 *>(sLam + r * D + c);
-        const float4 lr = *reinterpret_cast<const float4 *>(sLam + ref * D + c);
-        const uint2 w = *reinterpret_cast<const uint2 *>(smem + (isq ? OFF_SQ : OFF_SK) + (r * D + c) * 2);
-        const float sg = isq ? 1.f : -1.f;
-        float4 y;
-        y.x = __uint_as_float(w.x << 16) * ex2(sg * (l.x - lr.x));
-        y.y = __uint_as_float(w.x & 0xFFFF0000u) * ex2(sg * (l.y - lr.y));
-        y.z = __uint_as_float(w.y << 16) * ex2(sg * (l.z - lr.z));
-        y.w = __uint_as_float(w.y & 0xFFFF0000u) * ex2(sg * (l.w - lr.w));
-        *reinterpret_cast<float4 *>(smem + OFF_SG + (r * D + c) * 4) = y;
-    }
+    const uint2 w = *reinterpret_cast<const uint2 *>(smem + off + (row * D + kk) * 2);
+    const float4 l = *reinterpret_cast<const float4 *>(sLam + lam_at<D>(row, kk));
+    const float s = (float)SIGN;
+    y[0] = __uint_as_float(w.x << 16) * ex2(s * (l.x - r.x));
+    y[1] = __uint_as_float(w.x & 0xFFFF0000u) * ex2(s * (l.y - r.y));
+    y[2] = __uint_as_float(w.y << 16) * ex2(s * (l.z - r.z));
+    y[3] = __uint_as_float(w.y & 0xFFFF0000u) * ex2(s * (l.w - r.w));
 }
 
-// the level's squares: 2 H tiles of 4 x 4 scores, each by the G = 256 / H neighbouring lanes
-// that share its key dims (every 16-byte row read of a quarter-warp is 128 contiguous bytes),
-// then a transposing butterfly over the lanes
-template <int D, int H>
-__device__ __forceinline__ void exact_level_squares(uint8_t *smem)
-{
-    constexpr int G = 256 / H, TB = H / 4;
-    const int tile = thread_id() / G, ds = thread_id() % G;
-    const int blk = tile / (TB * TB), t = tile % (TB * TB);
-    const int i0 = blk * 2 * H + H + (t / TB) * 4, j0 = blk * 2 * H + (t % TB) * 4;
-    const float *X = reinterpret_cast<const float *>(smem + OFF_SG);
-    float v[16];
-#pragma unroll
-    for (int x = 0; x < 16; ++x)
-        v[x] = 0.f;
-#pragma unroll 1
-    for (int c0 = 0; c0 < D / 4; c0 += G) {
-        if (G <= D / 4 || ds < D / 4) {
-            const int c = (c0 + ds) * 4;
-            float4 k4[4];
-#pragma unroll
-            for (int y = 0; y < 4; ++y)
-                k4[y] = *reinterpret_cast<const float4 *>(X + (j0 + y) * D + c);
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const float4 q4 = *reinterpret_cast<const float4 *>(X + (i0 + x) * D + c);
-#pragma unroll
-                for (int y = 0; y < 4; ++y)
-                    v[4 * x + y] = fmaf(q4.w, k4[y].w, fmaf(q4.z, k4[y].z,
-                                   fmaf(q4.y, k4[y].y, fmaf(q4.x, k4[y].x, v[4 * x + y]))));
-            }
-        }
-    }
-    // 16 sums over G lanes: halve the values held at each of the first four exchanges
-    int first = 0;
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int o = G >> (s + 1), n = 8 >> s;
-        if (o > 0) {
-            const bool up = (ds & o) != 0;
-#pragma unroll
-            for (int x = 0; x < n; ++x) {
-                const float send = up ? v[x] : v[x + n];
-                v[x] = (up ? v[x + n] : v[x]) + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-            first += up ? n : 0;
-        }
-    }
-    if (G == 32)
-        v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-    constexpr int HELD = G == 8 ? 2 : 1;
-    if (G < 32 || (ds & 1) == 0) {
-#pragma unroll
-        for (int x = 0; x < HELD; ++x) {
-            const int i = i0 + (first + x) / 4, j = j0 + (first + x) % 4;
-            *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(v[x]);
-            *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, j, i)) = 0.f;
-        }
-    }
-}
-
-// the 8 x 8 triangles on the diagonal: thread (block, key dim) takes the 36 products of its
-// key dim from registers; warp sums over 32 key dims go to the staged values' area ...
 template <int D>
-__device__ __forceinline__ void exact_triangles(uint8_t *smem)
+__device__ __forceinline__ float4 lam4(const uint8_t *smem, int row, int kk)
 {
-    constexpr int NP = D / 32;                 // warps, and partial sums, per block
-    const int warp = thread_id() >> 5, lane = thread_id() & 31;
-    const int d = (warp % NP) * 32 + lane;
-    const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
-    const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
-    const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
-    float *part = reinterpret_cast<float *>(smem + OFF_SV);
-#pragma unroll 1
-    for (int blk = warp / NP; blk < 8; blk += 16 / NP) {
-        float l[8], k[8], v[8];
+    return *reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(smem + X_LAM) +
+                                             lam_at<D>(row, kk));
+}
+
+// MT x NT tiles of 16 x 8 scores += fragments a (rows g and g + 8 of each tile) and b, each four
+// consecutive key dims per lane: a k step of the products takes two of them (any assignment
+// of key dims to k will do, as long as both operands share it)
+template <int MT, int NT8>
+__device__ __forceinline__ void squares_mma(float (&acc)[MT][NT8][4], const float (&a)[2 * MT][4],
+                                            const float (&b)[NT8][4])
+{
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            l[x] = sLam[(8 * blk + x) * D + d];
-            k[x] = bf16f(sK[(8 * blk + x) * D + d]);
+    for (int x = 0; x < 4; x += 2) {
+        uint32_t bh[NT8][2], bl[NT8][2];
+#pragma unroll
+        for (int n = 0; n < NT8; ++n) {
+            split_tf32(b[n][x], bh[n][0], bl[n][0]);
+            split_tf32(b[n][x + 1], bh[n][1], bl[n][1]);
         }
-        float *dst = part + (blk * NP + warp % NP) * 40;
-        // product n = i (i + 1) / 2 + j, eight at a time
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float q = bf16f(sQ[(8 * blk + i) * D + d]);
+        for (int m = 0; m < MT; ++m) {
+            uint32_t ah[4], al[4];
+            split_tf32(a[2 * m][x], ah[0], al[0]);
+            split_tf32(a[2 * m + 1][x], ah[1], al[1]);
+            split_tf32(a[2 * m][x + 1], ah[2], al[2]);
+            split_tf32(a[2 * m + 1][x + 1], ah[3], al[3]);
 #pragma unroll
-            for (int j = 0; j <= i; ++j) {
-                const int n = i * (i + 1) / 2 + j;
-                v[n % 8] = j == i ? q * k[j] : q * k[j] * ex2(l[i] - l[j]);
-                if (n % 8 == 7 || n == 35) {
-                    if (n == 35) {
+            for (int n = 0; n < NT8; ++n)
+                mma_m16n8k8_tf32(acc[m][n], al, bh[n]);
 #pragma unroll
-                        for (int x = 4; x < 8; ++x)
-                            v[x] = 0.f;
-                    }
-                    const float sum = warp_sum8(v, lane);
-                    if ((lane & 3) == 0)
-                        dst[(n & ~7) + (lane >> 2)] = sum;
+            for (int n = 0; n < NT8; ++n)
+                mma_m16n8k8_tf32(acc[m][n], ah, bl[n]);
+#pragma unroll
+            for (int n = 0; n < NT8; ++n)
+                mma_m16n8k8_tf32(acc[m][n], ah, bh[n]);
+        }
+    }
+}
+
+// (one warp) a quarter of the key dims of one half (queries 32 + 16 mh..) of the 32 x 32 square
+// (queries 32..63, keys 0..31, factored at token 31)
+template <int D>
+__device__ __forceinline__ void exact_square32(uint8_t *smem, int mh, int quarter)
+{
+    const int lane = thread_id() & 31, g = lane >> 2, t = lane & 3;
+    float acc[1][4][4] = {};
+#pragma unroll 1
+    for (int k0 = quarter * (D / 4); k0 < (quarter + 1) * (D / 4); k0 += 16) {
+        const int kk = k0 + 4 * t;
+        const float4 r = lam4<D>(smem, 31, kk);
+        float a[2][4], b[4][4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+            factors4<D, 1>(smem, OFF_SQ, 32 + 16 * mh + 8 * x + g, r, kk, a[x]);
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            factors4<D, -1>(smem, OFF_SK, 8 * x + g, r, kk, b[x]);
+        squares_mma<1, 4>(acc, a, b);
+    }
+    float *dst = reinterpret_cast<float *>(smem + X_P32) + quarter * 1024 + (16 * mh + g) * 32 + 2 * t;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        *reinterpret_cast<float2 *>(dst + 8 * n) = make_float2(acc[0][n][0], acc[0][n][1]);
+        *reinterpret_cast<float2 *>(dst + 8 * 32 + 8 * n) = make_float2(acc[0][n][2], acc[0][n][3]);
+    }
+}
+
+// (one warp) half of unit u's key dims
+template <int D>
+__device__ __forceinline__ void exact_square16(uint8_t *smem, int u, int half)
+{
+    const int lane = thread_id() & 31, g = lane >> 2, t = lane & 3;
+    const SquareUnit m = square_unit(u);
+    float acc[1][2][4] = {};
+#pragma unroll 1
+    for (int k0 = half * (D / 2); k0 < (half + 1) * (D / 2); k0 += 32) {
+        float a[2][2][4], b[2][2][4];
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const int kk = k0 + 16 * y + 4 * t;
+            const float4 ra = lam4<D>(smem, m.ref0, kk), rb = lam4<D>(smem, m.ref1, kk);
+            factors4<D, 1>(smem, OFF_SQ, m.r0 + g, ra, kk, a[y][0]);
+            factors4<D, 1>(smem, OFF_SQ, m.r1 + g, rb, kk, a[y][1]);
+            factors4<D, -1>(smem, OFF_SK, m.c0 + g, ra, kk, b[y][0]);
+            factors4<D, -1>(smem, OFF_SK, m.c1 + g, rb, kk, b[y][1]);
+        }
+        squares_mma<1, 2>(acc, a[0], b[0]);
+        squares_mma<1, 2>(acc, a[1], b[1]);
+    }
+    float *dst = reinterpret_cast<float *>(smem + X_P16) + (2 * u + half) * 256;
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+        float *p = dst + g * 16 + 8 * n + 2 * t;
+        *reinterpret_cast<float2 *>(p) = make_float2(acc[0][n][0], acc[0][n][1]);
+        *reinterpret_cast<float2 *>(p + 8 * 16) = make_float2(acc[0][n][2], acc[0][n][3]);
+    }
+}
+
+// (one warp) the 8 x 8 triangle of tokens 8 blk.. over 64 key dims (part `part`), two per lane:
+// 36 products each, then warp sums into X_PTR
+template <int D>
+__device__ __forceinline__ void exact_triangle(uint8_t *smem, int blk, int part)
+{
+    const int lane = thread_id() & 31, d = part * 64 + 2 * lane;
+    const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
+    float *dst = reinterpret_cast<float *>(smem + X_PTR) + (blk * (D / 64) + part) * 40;
+    float2 l[8];
+    uint32_t k[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        l[x] = *reinterpret_cast<const float2 *>(sLam + lam_at<D>(8 * blk + x, d));
+        k[x] = *reinterpret_cast<const uint32_t *>(smem + OFF_SK + ((8 * blk + x) * D + d) * 2);
+    }
+    float v[8];
+    // product n = i (i + 1) / 2 + j, eight at a time
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t w = *reinterpret_cast<const uint32_t *>(smem + OFF_SQ + ((8 * blk + i) * D + d) * 2);
+        const float2 q = make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+#pragma unroll
+        for (int j = 0; j <= i; ++j) {
+            const int n = i * (i + 1) / 2 + j;
+            const float k0 = __uint_as_float(k[j] << 16), k1 = __uint_as_float(k[j] & 0xFFFF0000u);
+            v[n % 8] = j == i ? fmaf(q.y, k1, q.x * k0)
+                              : fmaf(q.y * k1, ex2(l[i].y - l[j].y), q.x * k0 * ex2(l[i].x - l[j].x));
+            if (n % 8 == 7 || n == 35) {
+                if (n == 35) {
+#pragma unroll
+                    for (int x = 4; x < 8; ++x)
+                        v[x] = 0.f;
                 }
+                const float sum = warp_sum8(v, lane);
+                if ((lane & 3) == 0)
+                    dst[(n & ~7) + (lane >> 2)] = sum;
             }
         }
     }
 }
 
-// ... and are added up, one thread per element of the eight 8 x 8 blocks
+constexpr int kSquareTasks = 8 + 8;
+
+// (one warp) the task-th of kSquareTasks + 8 (D / 64) score tasks
 template <int D>
-__device__ __forceinline__ void exact_triangles_sum(uint8_t *smem)
+__device__ __forceinline__ void exact_task(uint8_t *smem, int task)
 {
-    constexpr int NP = D / 32;
-    const int blk = thread_id() >> 6, i = (thread_id() >> 3) & 7, j = thread_id() & 7;
-    const float *part = reinterpret_cast<const float *>(smem + OFF_SV) + blk * NP * 40;
-    float a = 0.f;
-    if (j <= i) {
-        const int n = i * (i + 1) / 2 + j;
+    if (task < 8)
+        exact_square16<D>(smem, task >> 1, task & 1);
+    else if (task < kSquareTasks)
+        exact_square32<D>(smem, task & 1, (task - 8) >> 1);
+    else
+        exact_triangle<D>(smem, (task - kSquareTasks) / (D / 64), (task - kSquareTasks) % (D / 64));
+}
+
+// (builder warps) whether the gates of a staged segment alone send it to the exact path: the
+// first step of build_fast, with its arithmetic and its verdict (uniform over the builders)
+template <int D>
+__device__ __forceinline__ bool gates_exact(uint8_t *smem, int L)
+{
+    using G = Geo<D>;
+    const int tid = thread_id(), dp = tid % G::DP, qt = tid / G::DP;
+    const float *sG = reinterpret_cast<const float *>(smem + OFF_SG);
+    float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
+    zero_tail<D>(smem, L, true);
+    float amax = -INFINITY, r0 = 0.f, r1 = 0.f;
 #pragma unroll
-        for (int x = 0; x < NP; ++x)
-            a += part[x * 40 + n];
+    for (int x = 0; x < G::TPG; ++x) {
+        const float2 a = *reinterpret_cast<const float2 *>(sG + (G::TPG * qt + x) * D + 2 * dp);
+        amax = fmaxf(amax, fmaxf(a.x, a.y));
+        r0 = fmaf(a.x, kLog2e, r0);
+        r1 = fmaf(a.y, kLog2e, r1);
     }
-    *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, 8 * blk + i, 8 * blk + j)) = rna_tf32(a);
+    *reinterpret_cast<float2 *>(sTot + qt * D + 2 * dp) = make_float2(r0, r1);
+    bar_builders();
+    float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+    for (int u = 0; u < G::NQ; ++u) {
+        const float2 t = *reinterpret_cast<const float2 *>(sTot + u * D + 2 * dp);
+        t0 += t.x;
+        t1 += t.y;
+    }
+    return bar_or(1, !(amax <= 0.f && t0 >= -kLamRange && t1 >= -kLamRange));
+}
+
+// (builder warps) zeros above the diagonal, in 16-byte pieces; pieces that cross the diagonal
+// belong to the triangles
+template <int D>
+__device__ __forceinline__ void exact_zeros(uint8_t *smem)
+{
+#pragma unroll
+    for (int x = 0; x < CH * CH / 4 / NB; ++x) {
+        const int e = thread_id() + x * NB;
+        const int i = e >> 4, j = (e & 15) * 4;
+        if (j > i)
+            *reinterpret_cast<float4 *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) =
+                make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+// the partial sums added up: every score on and below the diagonal, and the triangles' zeros
+template <int D>
+__device__ __forceinline__ void exact_scores_sum(uint8_t *smem)
+{
+    const int tid = thread_id();
+    auto put = [&](int i, int j, float a) {
+        *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(a);
+    };
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int e = tid + x * NT;
+        const float *src = reinterpret_cast<const float *>(smem + X_P32) + e;
+        put(32 + (e >> 5), e & 31, (src[0] + src[1024]) + (src[2048] + src[3072]));
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int e = tid + x * NT, u = e >> 8, r = (e >> 4) & 15, c = e & 15;
+        const float *src = reinterpret_cast<const float *>(smem + X_P16) + 2 * u * 256 + (e & 255);
+        const SquareUnit m = square_unit(u);
+        if (u < 2 || (r >> 3) == (c >> 3))
+            put(r < 8 ? m.r0 + r : m.r1 + r - 8, c < 8 ? m.c0 + c : m.c1 + c - 8, src[0] + src[256]);
+    }
+    {
+        constexpr int NP = D / 64;
+        const int blk = tid >> 6, i = (tid >> 3) & 7, j = tid & 7, n = i * (i + 1) / 2 + j;
+        const float *src = reinterpret_cast<const float *>(smem + X_PTR) + blk * NP * 40;
+        float a = 0.f;
+        if (j <= i) {
+#pragma unroll
+            for (int x = 0; x < NP; ++x)
+                a += src[x * 40 + n];
+        }
+        put(8 * blk + i, 8 * blk + j, a);
+    }
 }
 
 // pair by pair, for segments with a gate above 0
@@ -904,7 +1063,7 @@ __device__ __forceinline__ void exact_scores_pairs(uint8_t *smem, int L)
         if (j <= i && i < L) {
             for (int dd = 0; dd < D; ++dd)
                 acc = fmaf(bf16f(sQ[i * D + dd]) * bf16f(sK[j * D + dd]),
-                           ex2(lg[i * D + dd] - lg[j * D + dd]), acc);
+                           ex2(lg[lam_at<D>(i, dd)] - lg[lam_at<D>(j, dd)]), acc);
         }
         *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(acc);
     }
@@ -929,54 +1088,63 @@ __device__ __forceinline__ void exact_issue_sq(uint32_t tmem, uint32_t sb)
 }
 
 // Every operand of an exact segment, and S^T Q~^T issued: from staged inputs to A and K^^T in
-// X_B2, V^T and the decayed state in TMEM, visible to the tensor core.
+// X_B2, V^T and the decayed state in TMEM, visible to the tensor core.  `next` is a word of
+// shared memory (the task counter).  The state warps split the state and start S^T Q~^T while
+// the builders form K^ and V^T; then both draw score tasks.
 template <int D>
-__device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int L)
+__device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int L, int *next)
 {
-    const bool up = exact_build<D>(smem, tmem, L, 0);
-    __syncthreads();
-    exact_split_state<D>(smem, tmem, 0);
-    if (!up)
-        exact_level_rows<D, 32>(smem);
+    constexpr int TASKS = kSquareTasks + 8 * (D / 64);
+    if (thread_id() == 0)
+        *next = 0;
+    const bool up = exact_decay<D>(smem, L);
     fence_proxy_async_smem();
-    tc_fence_before();
     __syncthreads();
-    if (thread_id() == kIssuer) {
-        tc_fence_after();
-        exact_issue_sq<D>(tmem, smem_u32(smem));
+    if (thread_id() < NB) {
+        if (!up)
+            exact_zeros<D>(smem);
+        exact_keys_values<D>(smem, tmem);
+    } else {
+        exact_split_state<D>(smem, tmem);
+        tc_fence_before();
+        bar_staters();
+        if (thread_id() == kIssuer) {
+            tc_fence_after();
+            exact_issue_sq<D>(tmem, smem_u32(smem));
+        }
+        __syncwarp();
     }
-    // the scores while the tensor core runs S^T Q~^T
     if (up) {
         exact_scores_pairs<D>(smem, L);
     } else {
-        exact_triangles<D>(smem);
-        exact_level_squares<D, 32>(smem);
+        while (true) {
+            int task = 0;
+            if ((thread_id() & 31) == 0)
+                task = atomicAdd(next, 1);
+            task = __shfl_sync(0xffffffffu, task, 0);
+            if (task >= TASKS)
+                break;
+            exact_task<D>(smem, task);
+        }
         __syncthreads();
-        exact_triangles_sum<D>(smem);
-        exact_level_rows<D, 16>(smem);
-        __syncthreads();
-        exact_level_squares<D, 16>(smem);
-        __syncthreads();
-        exact_level_rows<D, 8>(smem);
-        __syncthreads();
-        exact_level_squares<D, 8>(smem);
+        exact_scores_sum<D>(smem);
     }
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
 }
 
-// (issuing thread) D_O += V^T A^T and S^T += V^T K^ (onto the decayed state), 8 tokens per step
+// (issuing thread) [D_O | S^T] += V^T [A ; K^^T]^T (S^T decayed before), 8 tokens per step: one
+// accumulator of N = 64 + D columns, since D_O (TM_O0) and S^T (TM_S) are adjacent
 template <int D>
 __device__ __forceinline__ void exact_issue_update(uint32_t tmem, uint32_t sb)
 {
+    static_assert(TM_S == TM_O0 + 64, "D_O and S^T adjacent");
 #pragma unroll 1
     for (int kk = 0; kk < CH / 8; ++kk) {
         const uint32_t koff = (kk >> 2) * (Geo<D>::ROWS * 128) + (kk & 3) * 32;
         mma_tf32_ts(tmem + TM_O0, tmem + TM_V + kk * 8, sdesc_sw128(sb + X_B2 + koff, 16, 1024),
-                    IDT_N64, 1);
-        mma_tf32_ts(tmem + TM_S, tmem + TM_V + kk * 8,
-                    sdesc_sw128(sb + X_B2 + koff + 64 * 128, 16, 1024), Geo<D>::IDT_ST, 1);
+                    Geo<D>::IDT_UP, 1);
     }
 }
 
@@ -987,7 +1155,7 @@ template <int D>
 __device__ __forceinline__ void fast_issue_scores(uint32_t tmem, uint32_t sb, int par)
 {
     const uint32_t setb = sb + (uint32_t)par * SET_BYTES;
-#pragma unroll 1
+#pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         const uint32_t koff = (kk >> 2) * 8192 + (kk & 3) * 32;
         mma_f16_ss(tmem + (par ? TM_A1 : TM_A0), sdesc_sw128(setb + S_QH + koff, 16, 1024),
@@ -1000,7 +1168,7 @@ template <int D>
 __device__ __forceinline__ void fast_issue_sq(uint32_t tmem, uint32_t sb, int par)
 {
     const uint32_t setb = sb + (uint32_t)par * SET_BYTES;
-#pragma unroll 1
+#pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         const uint32_t koff = (kk >> 2) * 8192 + (kk & 3) * 32;
         mma_f16_ts(tmem + (par ? Geo<D>::O1 : TM_O0), tmem + TM_SH + kk * 8,
@@ -1018,7 +1186,7 @@ __device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, in
 {
     const uint32_t setb = sb + (uint32_t)par * SET_BYTES;
     const uint32_t vt = tmem + TM_V + 32 * par;
-#pragma unroll 1
+#pragma unroll
     for (int kk = 0; kk < CH / 16; ++kk) {
         mma_f16_ts(tmem + (par ? Geo<D>::O1 : TM_O0), vt + kk * 8,
                    sdesc_sw128(setb + S_AH + kk * 32, 16, 1024), IDF_N64, 1);

@@ -74,11 +74,11 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     const uint32_t sb = smem_u32(smem);
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
     // [0] TMEM base, [1] abort flag, [2] decision on the latest built segment (1 = fast),
-    // [3] run result (1 = the segment at [4..5] needs the exact path), [4..5] position
-    // where the run stopped, [6..7] its local token index, [8] whether the latest segment's
-    // build is whole (0: its gates alone send it to the exact path, its inputs still staged)
+    // [3] run result (1 = the segment at [4] needs the exact path), [4] token index where the
+    // run stopped, [8] whether the latest segment's
+    // build is whole (0: its gates alone send it to the exact path, its inputs still staged),
+    // [9] an exact segment's look ahead, [10] its task counter
     volatile uint32_t *sMisc = reinterpret_cast<volatile uint32_t *>(smem + OFF_MISC);
-    volatile int64_t *sRun = reinterpret_cast<volatile int64_t *>(smem + OFF_MISC + 16);
     const uint32_t bar_tma = sb + OFF_BAR, bar_a = sb + OFF_BAR + 8, bar_o = sb + OFF_BAR + 16,
                    bar_s = sb + OFF_BAR + 24, bar_built = sb + OFF_BAR + 32,
                    bar_go = sb + OFF_BAR + 40, bar_ld = sb + OFF_BAR + 48,
@@ -90,10 +90,9 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     const int n = p.n_tokens[b];
     if (n <= 0)
         return;
-    const int64_t pos0 = p.pos0[b];
-    const int64_t end = pos0 + n;
+    // positions are token indexes of this call (32 bits); the chunk grid is `off` tokens ahead
+    const int off = p.off[b];
     const int64_t tstride = (int64_t)p.n_heads * D;   // elements between consecutive tokens
-    const int C = p.ckpt_interval;
 
     if (tid == 0) {
         mbar_init(bar_tma, 1);
@@ -135,11 +134,11 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     uint32_t ph_a0 = 0, ph_a1 = 0;   // D_A products of even / odd segments (bar_a, bar_a1)
     bool aborted = false;
 
-    // L2 prefetch of the 64 tokens from local position t (if any are this problem's)
-    auto prefetch = [&](int64_t t) {
-        if (t >= n)
+    // L2 prefetch of the 64 tokens `ahead` tokens past token t (if any are this problem's)
+    auto prefetch = [&](int t, int ahead) {
+        if (n - t <= ahead)
             return;
-        const int32_t y = (int32_t)((int64_t)p.row0[b] + t);
+        const int32_t y = p.row0[b] + t + ahead;
         const int32_t x = h * D;
         tma_prefetch_2d(&maps.q, x, y);
         tma_prefetch_2d(&maps.k, x, y);
@@ -149,18 +148,21 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // (loader) staged inputs of the segment at local position tok_local; segments after
     // the first start on the 64-token grid, so the segment kPrefetch ahead starts at
     // tok_local + 64 * kPrefetch and is requested into L2 now
-    auto issue_tma = [&](int64_t tok_local) {
-        const int32_t y = (int32_t)((int64_t)p.row0[b] + tok_local);
+    auto copy_inputs = [&](int tok_local) {
+        const int32_t y = p.row0[b] + tok_local;
         const int32_t x = h * D;
         mbar_arrive_expect_tx(bar_tma, Geo<D>::STAGE);
+        tma_load_2d(sb + OFF_SG, &maps.g, x, y, bar_tma);
         tma_load_2d(sb + OFF_SQ, &maps.q, x, y, bar_tma);
         tma_load_2d(sb + OFF_SK, &maps.k, x, y, bar_tma);
         tma_load_2d(sb + OFF_SV, &maps.v, x, y, bar_tma);
-        tma_load_2d(sb + OFF_SG, &maps.g, x, y, bar_tma);
+    };
+    auto issue_tma = [&](int tok_local) {
+        copy_inputs(tok_local);
         ++n_tma;
         tma_pending = true;
         if (tok_local > 0)
-            prefetch(tok_local + (int64_t)CH * kPrefetch);
+            prefetch(tok_local, CH * kPrefetch);
     };
     // one thread (`who`) waits on an mbarrier; false (for every thread) if that wait ran
     // out or another thread raised the abort flag.  CTA-wide, or within the builder (id 1)
@@ -208,12 +210,17 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             aborted = true;
         return !stop;
     };
-    auto seg_len = [&](int64_t at) -> int { return (int)(min(end, (at / CH + 1) * CH) - at); };
-    auto is_long = [&](int64_t at) -> bool { return at < end && seg_len(at) > kShort; };
-    auto ckpt_slot = [&](int64_t seg_end) -> float * {
-        if (!(C > 0 && seg_end % C == 0 && p.ckpt_slots != nullptr))
+    auto seg_len = [&](int at) -> int { return min(n - at, CH - (int)(((uint32_t)at + off) & (CH - 1))); };
+    auto is_long = [&](int at) -> bool { return at < n && seg_len(at) > kShort; };
+    // (state warps) the checkpoint due at the end of a segment, segments taken in order: the
+    // next one's token index and slot number (a position modulo the interval would be a 64-bit
+    // division on the state warps' chain)
+    int next_ck = p.first_ck[b], ck_i = p.ck_base[b];
+    auto ckpt_slot = [&](int seg_end) -> float * {
+        if (seg_end != next_ck)
             return nullptr;
-        float *slot = p.ckpt_slots[p.ck_base[b] + (seg_end / C - pos0 / C - 1)];
+        float *slot = p.ckpt_slots[ck_i++];
+        next_ck = next_ck <= n - p.ckpt_interval ? next_ck + p.ckpt_interval : 0;
         if (slot == nullptr || (reinterpret_cast<uintptr_t>(slot) & 15u) != 0) {
             if (tid == kIssuer)
                 report(p.d_err, slot == nullptr ? HS_DEVERR_NULL : HS_DEVERR_MISALIGNED);
@@ -245,14 +252,14 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     }
 
     // the output rows from local token t
-    auto outp = [&](int64_t t) { return p.o + (((int64_t)p.row0[b] + t) * p.n_heads + h) * D; };
+    auto outp = [&](int t) { return p.o + (((int64_t)p.row0[b] + t) * p.n_heads + h) * D; };
 
     // ---- a short segment (<= kShort tokens, staged inputs already waited for, no decay
     // pending): the per-token recurrence with the recurrent kernel's exact operation order
     // (fma chains over groups of 16 key rows, group partials summed left to right)
-    auto short_segment = [&](int64_t tok_s, int L, int64_t seg_end) {
-        short_state<D>(smem, tmem, L, ckpt_slot(seg_end));
-        if (tid == kLoader && seg_end < end)
+    auto short_segment = [&](int tok_s, int L) {
+        short_state<D>(smem, tmem, L, worker ? ckpt_slot(tok_s + L) : nullptr);
+        if (tid == kLoader && tok_s + L < n)
             issue_tma(tok_s + L);
         short_outputs<D>(smem, L, outp(tok_s), tstride);
         tc_fence_before();
@@ -283,23 +290,36 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
 
     // ---- one exact segment, from staged inputs, no decay pending and no MMA in flight; stages
     // the next segment once its own inputs are read; leaves the final state in TMEM, writes
-    // its outputs and checkpoint
-    auto exact_segment = [&](int64_t tok_s, int L, int64_t seg_end) -> bool {
-        exact_operands<D>(smem, tmem, L);
+    // its outputs and checkpoint.  Meanwhile the builders look ahead: the next segment's inputs
+    // waited for and its gates judged, into `ready` (see the main loop).
+    int ready = 0;
+    auto exact_segment = [&](int tok_s, int L) -> bool {
+        const int seg_end = tok_s + L;
+        exact_operands<D>(smem, tmem, L, const_cast<int *>(reinterpret_cast<volatile int *>(sMisc + 10)));
         if (tid == kIssuer) {
             tc_fence_after();
             exact_issue_update<D>(tmem, sb);
             tc_commit(bar_o);
         }
-        if (tid == kLoader && seg_end < end)
-            issue_tma(tok_s + L);
-        if (!wait_all(kIssuer, bar_o, ph_o))
-            return false;
-        state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false);   // checkpoint and |S| of the final state
-        out_epilogue<D>(tmem, outp(tok_s), tstride, L, 0, false);
+        const bool ahead = is_long(seg_end);
+        if (builder) {
+            if (tid == kLoader && seg_end < n)
+                issue_tma(seg_end);
+            if (ahead && wait_group(1, kLoader, bar_tma, ph_tma)) {
+                tma_pending = false;
+                const bool exact = gates_exact<D>(smem, seg_len(seg_end));
+                if (tid == kLoader)
+                    sMisc[9] = exact ? 1u : 2u;
+            }
+        } else if (wait_group(2, kIssuer, bar_o, ph_o)) {
+            state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false);   // checkpoint and |S| of the final state
+            out_epilogue<D>(tmem, outp(tok_s), tstride, L, 0, false);
+        }
         tc_fence_before();
-        __syncthreads();
+        if (!sync_all())
+            return false;
         tc_fence_after();
+        ready = ahead ? (int)sMisc[9] : 0;
         return true;
     };
 
@@ -317,57 +337,66 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // a run resumed from a checkpoint at that segment does.  The groups then meet CTA-wide.
     // No MMA is in flight at either end.
     int kseq = 0;   // long segments of the current run so far (slot of 2^{Lam_last}: kseq mod 4)
-    auto builder_run = [&](int64_t rpos, int64_t rtok) {
+    auto builder_run = [&](int rtok, bool waited) {
         int par = 0;
         while (true) {
-            const int L = seg_len(rpos);
-            if (!wait_group(1, kLoader, bar_tma, ph_tma))
+            const int L = seg_len(rtok);
+            if (!waited && !wait_group(1, kLoader, bar_tma, ph_tma))
                 return;
+            waited = false;
             tma_pending = false;
             if (tid == kLoader && !prefetched) {
                 // once the first segment has landed (the state and the first segment are
                 // not queued behind these): the next kPrefetch segments into L2
                 prefetched = true;
                 for (int j = 1; j <= kPrefetch; ++j)
-                    prefetch(rtok + L + (int64_t)CH * (j - 1));
+                    prefetch(rtok + L, CH * (j - 1));
             }
             const bool built = build_fast<D>(smem, tmem, L, par, kseq & 3);
             fence_proxy_async_smem();
             tc_fence_before();
             if (!sync_group(1))
                 return;
-            const bool next_long = is_long(rpos + L);
+            const bool next_long = is_long(rtok + L);
             if (tid == kLoader) {
                 sMisc[8] = built ? 1u : 0u;
                 mbar_arrive(bar_built);
             }
-            if (tid == kLoader && built) {
-                // the staged rows are consumed: stage the next segment (long or short) now;
-                // an exact decision on this one reloads it
-                if (rpos + L < end)
-                    issue_tma(rtok + L);
-                // D_A = Q~ K~^T of this segment, into its own buffer (the state warps wait on
-                // bar_a / bar_a1 by parity before they read it)
-                tc_fence_after();
-                fast_issue_scores<D>(tmem, sb, par);
-                tc_commit(par ? bar_a1 : bar_a);
+            if (built) {
+                // three threads of different warps, so that these issues overlap: D_A = Q~ K~^T of
+                // this segment into its own buffer (the state warps wait on bar_a / bar_a1 by parity
+                // before they read it); the staged rows are consumed, so the next segment (long
+                // or short) is staged now (an exact decision on this one reloads it); and the
+                // segment kPrefetch further on is requested into L2
+                const bool more = rtok + L < n;
+                if (tid == kLoader) {
+                    tc_fence_after();
+                    fast_issue_scores<D>(tmem, sb, par);
+                    tc_commit(par ? bar_a1 : bar_a);
+                    if (more) {
+                        ++n_tma;
+                        tma_pending = true;
+                    }
+                } else if (tid == kLoader + 32 && more) {
+                    copy_inputs(rtok + L);
+                } else if (tid == kLoader + 64) {
+                    prefetch(rtok + L, CH * kPrefetch);
+                }
             }
             if (!wait_group(1, kLoader, bar_go, ph_go))
                 return;
             if (sMisc[2] == 0 || !next_long)
                 return;
-            rpos += L;
             rtok += L;
             par ^= 1;
             ++kseq;
         }
     };
-    auto state_run = [&](int64_t rpos, int64_t rtok) {
+    auto state_run = [&](int rtok) {
         int par = 0;
         bool pend = false;
         uint32_t stop = 0;   // why the run ended: 0 done or short segment, 1 exact, 2 new run
-        int pend_par = 0, pend_L = 0, pend_g = 0;
-        int64_t pend_tok = 0, pend_end = 0;
+        int pend_par = 0, pend_L = 0, pend_g = 0, pend_tok = 0;
         float mk_cur = 0.f, mv_cur = 0.f;
         if (!wait_group(2, kIssuer, bar_built, ph_built))
             return;
@@ -385,8 +414,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         if (!fast && sMisc[8] != 0 && !wait_group(2, kIssuer, bar_a, ph_a0))
             return;
         while (fast) {
-            const int L = seg_len(rpos);
-            const int64_t seg_end = rpos + L;
+            const int L = seg_len(rtok);
             mk_cur = mk_new;
             mv_cur = mv_new;
             if (pend && !wait_group(2, kIssuer, bar_o, ph_o))
@@ -394,7 +422,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             // the products of the previous segment are complete: its operand set is free
             if (tid == kIssuer)
                 mbar_arrive(bar_go);
-            state_pass<D>(smem, tmem, pend ? pend_g : -1, pend ? ckpt_slot(pend_end) : nullptr, true);
+            state_pass<D>(smem, tmem, pend ? pend_g : -1, pend ? ckpt_slot(rtok) : nullptr, true);
             tc_fence_before();
             if (!sync_group(2))
                 return;
@@ -422,13 +450,11 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             pend_par = par;
             pend_tok = rtok;
             pend_L = L;
-            pend_end = seg_end;
             pend_g = kseq & 3;
-            rpos = seg_end;
             rtok += L;
             par ^= 1;
             ++kseq;
-            if (!is_long(rpos))
+            if (!is_long(rtok))
                 break;
             // the builders' next segment, and the decision on it: the state it starts from is
             // bounded by the fp16 copy's largest |S| at this segment's start plus this segment's
@@ -451,7 +477,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         if (pend) {
             if (!wait_group(2, kIssuer, bar_o, ph_o))
                 return;
-            state_pass<D>(smem, tmem, pend_g, ckpt_slot(pend_end), false);
+            state_pass<D>(smem, tmem, pend_g, ckpt_slot(rtok), false);
             out_epilogue<D>(tmem, outp(pend_tok), tstride, pend_L, pend_par, false);
             tc_fence_before();
             if (!sync_group(2))
@@ -459,8 +485,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         }
         if (tid == kIssuer) {
             sMisc[3] = stop;
-            sRun[0] = rpos;
-            sRun[1] = rtok;
+            sMisc[4] = (uint32_t)rtok;
         }
     };
 
@@ -470,27 +495,26 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // the float32 state in TMEM here (the state update is skipped and D_O reads the fp16 copy),
     // so the next segment's state is loaded while the previous segment's products run.
     int loaded = 0;   // index of the segment whose start state is in TMEM (state warps)
-    auto seg_idx = [&](int64_t at) -> int { return (int)(at / CH - pos0 / CH); };
+    auto seg_idx = [&](int at) -> int { return (int)(((uint32_t)at + off) / CH); };
     // (issuing thread) the start state of the segment at `at` into L2, one bulk request
-    auto prefetch_state = [&](int64_t at) {
+    auto prefetch_state = [&](int at) {
         const float *src = st_g + (int64_t)seg_idx(at) * p.n_heads * D * D;
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src),
                      "r"((uint32_t)(D * D * 4))
                      : "memory");
     };
-    auto state_run_restart = [&](int64_t rpos, int64_t rtok) {
+    auto state_run_restart = [&](int rtok) {
         int par = 0;
         bool pend = false;
         uint32_t stop = 0;   // 0 done or short segment, 1 exact
-        int pend_par = 0, pend_L = 0;
-        int64_t pend_tok = 0;
+        int pend_par = 0, pend_L = 0, pend_tok = 0;
         while (true) {
-            const int L = seg_len(rpos);
+            const int L = seg_len(rtok);
             if (!wait_group(2, kIssuer, bar_built, ph_built))
                 return;
-            if (loaded != seg_idx(rpos)) {
-                state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rpos) * p.n_heads * D * D);
-                loaded = seg_idx(rpos);
+            if (loaded != seg_idx(rtok)) {
+                state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rtok) * p.n_heads * D * D);
+                loaded = seg_idx(rtok);
             }
             // the loaded state (its TMEM columns and its largest |S|) visible to the group
             tc_fence_before();
@@ -512,8 +536,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                     return;
                 break;
             }
-            if (tid == kIssuer && is_long(rpos + L))
-                prefetch_state(rpos + L);   // read by the load at the end of this segment
+            if (tid == kIssuer && is_long(rtok + L))
+                prefetch_state(rtok + L);   // read by the load at the end of this segment
             if (pend && !wait_group(2, kIssuer, bar_o, ph_o))
                 return;
             // the products of the previous segment are complete: its operand set is free
@@ -545,16 +569,15 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             pend_par = par;
             pend_tok = rtok;
             pend_L = L;
-            rpos += L;
             rtok += L;
             par ^= 1;
             ++kseq;
-            if (!is_long(rpos))
+            if (!is_long(rtok))
                 break;
             // the next segment's start state, while this segment's products run and the
             // builders build it (this segment's fp16 copy is made: TMEM S is free)
-            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rpos) * p.n_heads * D * D);
-            loaded = seg_idx(rpos);
+            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rtok) * p.n_heads * D * D);
+            loaded = seg_idx(rtok);
         }
         if (pend) {
             if (!wait_group(2, kIssuer, bar_o, ph_o))
@@ -566,8 +589,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         }
         if (tid == kIssuer) {
             sMisc[3] = stop;
-            sRun[0] = rpos;
-            sRun[1] = rtok;
+            sMisc[4] = (uint32_t)rtok;
         }
     };
 
@@ -580,62 +602,65 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         wait_all(kLoader, bar_go, ph_stall);
     }
 
-    int64_t pos = pos0, tok = 0;
-    while (!aborted && pos < end) {
-        if (RESTART && worker && loaded != seg_idx(pos)) {
+    // `ready`, the long segment at tok after an exact one: its inputs are staged and waited for,
+    // and its gates alone send it to the exact path (1) or do not (2); 0: not looked at
+    int tok = 0;
+    while (!aborted && tok < n) {
+        if (RESTART && worker && loaded != seg_idx(tok)) {
             // this segment's own start state (the previous segment's state is not used)
-            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(pos) * p.n_heads * D * D);
+            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(tok) * p.n_heads * D * D);
             tc_fence_before();
             bar_staters();
             tc_fence_after();
-            loaded = seg_idx(pos);
+            loaded = seg_idx(tok);
         }
-        const int L = seg_len(pos);
+        const int L = seg_len(tok);
         if (L <= kShort) {
             // a leading or trailing short segment (its inputs are staged or in flight)
             if (!wait_tma())
                 break;
-            short_segment(tok, L, pos + L);
-            pos += L;
+            short_segment(tok, L);
             tok += L;
             continue;
         }
-        if (builder)
-            builder_run(pos, tok);
-        else if constexpr (RESTART)
-            state_run_restart(pos, tok);
-        else
-            state_run(pos, tok);
-        if (!sync_all())
-            break;
-        tc_fence_after();
-        const uint32_t stop = sMisc[3];
-        pos = sRun[0];
-        tok = sRun[1];
-        kseq = 0;
-        if (stop != 0) {
-            // the segment at pos takes the exact path (1) or starts a new run (2).  Its inputs
+        if (ready != 1) {
+            if (builder)
+                builder_run(tok, ready == 2);
+            else if constexpr (RESTART)
+                state_run_restart(tok);
+            else
+                state_run(tok);
+            ready = 0;
+            if (!sync_all())
+                break;
+            tc_fence_after();
+            const uint32_t stop = sMisc[3];
+            tok = (int)sMisc[4];
+            kseq = 0;
+            if (stop == 0)
+                continue;
+            // the segment at tok takes the exact path (1) or starts a new run (2).  Its inputs
             // are still staged if its build stopped early (sMisc[8] == 0); else restage them (the
             // copy of the next segment may be in flight)
-            const int Lx = seg_len(pos);
-            const bool staged = sMisc[8] == 0;
-            if (tid == kLoader && !staged) {
-                if (tma_pending && !mbar_wait_bounded(bar_tma, ph_tma, kTimeoutNs))
-                    sMisc[1] = 1;
-                if (tma_pending)
-                    ph_tma ^= 1;
-                issue_tma(tok);
+            if (sMisc[8] != 0) {
+                if (tid == kLoader) {
+                    if (tma_pending && !mbar_wait_bounded(bar_tma, ph_tma, kTimeoutNs))
+                        sMisc[1] = 1;
+                    if (tma_pending)
+                        ph_tma ^= 1;
+                    issue_tma(tok);
+                }
+                if (stop == 2)
+                    continue;   // the new run waits for the copy
+                if (!wait_tma())
+                    break;
             }
-            if (stop == 2)
-                continue;   // the new run waits for the copy
-            // every thread runs the exact segment
-            if (!staged && !wait_tma())
-                break;
-            if (!exact_segment(tok, Lx, pos + Lx))
-                break;
-            pos += Lx;
-            tok += Lx;
         }
+        // every thread runs the exact segment
+        const int Lx = seg_len(tok);
+        if (!exact_segment(tok, Lx))
+            break;
+        tok += Lx;
     }
 
     if (!aborted) {

@@ -48,7 +48,6 @@ __global__ void __launch_bounds__((D / 2) * (D / 16)) gla_decode_kernel(const __
     const int h = blockIdx.x - b * p.n_heads;
     if (p.n_tokens[b] <= 0)
         return;
-    const int64_t pos0 = p.pos0[b];
     const int tid = threadIdx.x;
     const int cg = tid % NCG;
     const int rg = tid / NCG;
@@ -106,8 +105,7 @@ __global__ void __launch_bounds__((D / 2) * (D / 16)) gla_decode_kernel(const __
         *reinterpret_cast<float2 *>(st + (int64_t)(16 * rg + r) * D + 2 * cg) = S[r];
     *reinterpret_cast<float2 *>(&spart[rg][2 * cg]) = acc;
 
-    const int C = p.ckpt_interval;
-    if (C > 0 && p.ckpt_slots != nullptr && (pos0 + 1) % C == 0) {
+    if (p.first_ck[b] == 1) {
         float *slot = p.ckpt_slots[p.ck_base[b]];
         if (slot == nullptr) {
             if (tid == 0)

@@ -45,12 +45,12 @@ __global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const
     const int n = p.n_tokens[b];
     if (n <= 0)
         return;
-    const int64_t pos0 = p.pos0[b];
     pdl_wait_and_release();
     const int tid = threadIdx.x;
     const int cg = tid % NCG;
     const int rg = tid / NCG;
-    const int C = p.ckpt_interval;
+    int next_ck = p.first_ck[b];      // tokens up to the next checkpoint, and its slot
+    int ck = p.ck_base[b];
 
     float *st = p.state + ((int64_t)b * p.n_heads + h) * D * D;
     float4 S[16];   // S[r] = state row 16*rg + r, columns 4*cg .. 4*cg+3
@@ -86,23 +86,20 @@ __global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const
                 acc.w = fmaf(qq, S[r].w, acc.w);
             }
             *reinterpret_cast<float4 *>(&spart[tt][rg][4 * cg]) = acc;
-            if (C > 0 && p.ckpt_slots != nullptr) {
-                const int64_t end = pos0 + t0 + tt + 1;
-                if (end % C == 0) {
-                    const int64_t slot_idx = p.ck_base[b] + (end / C - pos0 / C - 1);
-                    float *slot = p.ckpt_slots[slot_idx];
-                    if (slot == nullptr) {
-                        if (tid == 0)
-                            report(p.d_err, HS_DEVERR_NULL);
-                    } else if ((reinterpret_cast<uintptr_t>(slot) & 15u) != 0) {
-                        if (tid == 0)
-                            report(p.d_err, HS_DEVERR_MISALIGNED);
-                    } else {
-                        slot += (int64_t)h * D * D;
+            if (t0 + tt + 1 == next_ck) {
+                float *slot = p.ckpt_slots[ck++];
+                next_ck = next_ck <= n - p.ckpt_interval ? next_ck + p.ckpt_interval : 0;
+                if (slot == nullptr) {
+                    if (tid == 0)
+                        report(p.d_err, HS_DEVERR_NULL);
+                } else if ((reinterpret_cast<uintptr_t>(slot) & 15u) != 0) {
+                    if (tid == 0)
+                        report(p.d_err, HS_DEVERR_MISALIGNED);
+                } else {
+                    slot += (int64_t)h * D * D;
 #pragma unroll
-                        for (int r = 0; r < 16; ++r)
-                            *reinterpret_cast<float4 *>(slot + (int64_t)(16 * rg + r) * D + 4 * cg) = S[r];
-                    }
+                    for (int r = 0; r < 16; ++r)
+                        *reinterpret_cast<float4 *>(slot + (int64_t)(16 * rg + r) * D + 4 * cg) = S[r];
                 }
             }
         }

@@ -345,7 +345,9 @@ static hs_status prefill(const hs_linattn_shape *shp, const uint16_t *q, const u
         const int64_t r0 = cu_rows ? cu_rows[b] : (int64_t)b * s.max_tokens;
         if (r0 + n_tokens[b] > INT32_MAX)
             return HS_ERR_UNSUPPORTED;   // token rows are 32-bit
-        p.pos0[b] = pos0[b];
+        p.off[b] = (int32_t)(pos0[b] % HS_CHUNK);
+        p.first_ck[b] = p.ckpt_interval > 0
+                            ? p.ckpt_interval - (int32_t)(pos0[b] % p.ckpt_interval) : 0;
         p.n_tokens[b] = n_tokens[b];
         p.row0[b] = (int32_t)r0;
         p.ck_base[b] = (int32_t)base;
@@ -578,7 +580,8 @@ hs_status hs_linattn_prefill_scan(const hs_linattn_shape *shp, const uint16_t *q
                 e = std::min<int64_t>(end, (e / HS_CHUNK + 1) * HS_CHUNK);
                 ++n;
             }
-            p.pos0[j] = at;
+            p.off[j] = (int32_t)(at % HS_CHUNK);
+            p.first_ck[j] = 0;
             p.n_tokens[j] = (int32_t)(e - at);
             p.row0[j] = (int32_t)((int64_t)b * s.max_tokens + (at - pos0[b]));
             p.ck_base[j] = (int32_t)seg_i;
