@@ -14,6 +14,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 import threading
+from array import array
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libhs.so")
@@ -105,22 +106,68 @@ def load() -> C.CDLL:
     return _lib
 
 
+# Every call below is a decode step's host time: with the conversions written out per
+# element (ctypes arrays from int() of each entry, the torch stream object) a call of nine
+# problems spent 11 us in this module and 3.3 us in the library, launch included.
+
 def _ptr(x):
     if x is None:
         return None
+    try:
+        return x.data_ptr()
+    except AttributeError:
+        pass
     if isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
-        return x.data_ptr()
     if hasattr(x, "ctypes"):           # numpy (host arrays)
         return x.ctypes.data
     raise TypeError(f"cannot pass {type(x)} as a pointer")
 
 
+def _host_array(code, ctype, values, n: int):
+    """A host array of n integers (its address, and the object that owns it).  Lists and tuples
+    of n integers in range go through array.array, in C; anything else (other containers,
+    floats, values beyond the type, another length) through int() and ctypes as they always
+    have."""
+    if type(values) is list or type(values) is tuple:
+        try:
+            a = array(code, values)
+            if len(a) == n > 0:
+                return a.buffer_info()[0], a
+        except (TypeError, OverflowError):
+            pass
+    c = (ctype * max(n, 1))(*[int(x) for x in values])
+    return C.addressof(c), c
+
+
+def _i64(values, n: int):
+    return _host_array("q", C.c_int64, values, n)
+
+
+def _i32(values, n: int):
+    return _host_array("i", C.c_int32, values, n)
+
+
+_current_stream = None
+
+
+def _bind_current_stream():
+    """The function that returns the current torch stream's handle: torch's raw-handle query
+    (0.3 us) where this torch has it, else through the stream object (3 us)."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    device = torch.cuda.current_device
+    return lambda: raw(device())
+
+
 def _stream(s):
+    global _current_stream
     if s is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _current_stream is None:
+            _current_stream = _bind_current_stream()
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
@@ -149,7 +196,7 @@ def hs_align_prefix(N: int, hit_len: int, avail, page_size: int):
     """Strict-prefix alignment; returns (c, n_pages, tail)."""
     av = (C.c_int64 * len(avail))(*[int(a) for a in avail]) if len(avail) else None
     c, npg, tail = C.c_int64(), C.c_int64(), C.c_int64()
-    rc = load().hs_align_prefix(int(N), int(hit_len), C.cast(av, C.c_void_p) if av else None,
+    rc = (_lib or load()).hs_align_prefix(int(N), int(hit_len), C.cast(av, C.c_void_p) if av else None,
                                 len(avail), int(page_size), C.addressof(c), C.addressof(npg),
                                 C.addressof(tail))
     _check(rc, "hs_align_prefix")
@@ -158,7 +205,7 @@ def hs_align_prefix(N: int, hit_len: int, avail, page_size: int):
 
 def hs_restore_kv_pages(staging_layers, cache_layers, n_layers: int, block_table, n_pages: int,
                         page_bytes: int, num_blocks: int, d_err=None, stream=None):
-    rc = load().hs_restore_kv_pages(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
+    rc = (_lib or load()).hs_restore_kv_pages(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
                                     _ptr(block_table), int(n_pages), int(page_bytes),
                                     int(num_blocks), _ptr(d_err), _stream(stream))
     _check(rc, "hs_restore_kv_pages")
@@ -167,7 +214,7 @@ def hs_restore_kv_pages(staging_layers, cache_layers, n_layers: int, block_table
 def hs_restore_request(staging_layers, cache_layers, n_layers: int, block_table, n_pages: int,
                        page_bytes: int, num_blocks: int, src_slots, dst_slots, n_slots: int,
                        floats_each: int, d_err=None, stream=None):
-    rc = load().hs_restore_request(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
+    rc = (_lib or load()).hs_restore_request(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
                                    _ptr(block_table), int(n_pages), int(page_bytes),
                                    int(num_blocks), _ptr(src_slots), _ptr(dst_slots), int(n_slots),
                                    int(floats_each), _ptr(d_err), _stream(stream))
@@ -176,7 +223,7 @@ def hs_restore_request(staging_layers, cache_layers, n_layers: int, block_table,
 
 def hs_save_kv_pages(cache_layers, staging_layers, n_layers: int, block_table, n_pages: int,
                      page_bytes: int, num_blocks: int, d_err=None, stream=None):
-    rc = load().hs_save_kv_pages(_ptr(cache_layers), _ptr(staging_layers), int(n_layers),
+    rc = (_lib or load()).hs_save_kv_pages(_ptr(cache_layers), _ptr(staging_layers), int(n_layers),
                                  _ptr(block_table), int(n_pages), int(page_bytes),
                                  int(num_blocks), _ptr(d_err), _stream(stream))
     _check(rc, "hs_save_kv_pages")
@@ -185,7 +232,7 @@ def hs_save_kv_pages(cache_layers, staging_layers, n_layers: int, block_table, n
 def hs_restore_kv_page_slices(staging_layers, cache_layers, n_layers: int, block_table,
                               n_pages: int, page_bytes: int, rows: int, col_off: int,
                               col_bytes: int, num_blocks: int, d_err=None, stream=None):
-    rc = load().hs_restore_kv_page_slices(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
+    rc = (_lib or load()).hs_restore_kv_page_slices(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
                                           _ptr(block_table), int(n_pages), int(page_bytes),
                                           int(rows), int(col_off), int(col_bytes), int(num_blocks),
                                           _ptr(d_err), _stream(stream))
@@ -195,7 +242,7 @@ def hs_restore_kv_page_slices(staging_layers, cache_layers, n_layers: int, block
 def hs_save_kv_page_slices(cache_layers, staging_layers, n_layers: int, block_table, n_pages: int,
                            page_bytes: int, rows: int, col_off: int, col_bytes: int,
                            num_blocks: int, d_err=None, stream=None):
-    rc = load().hs_save_kv_page_slices(_ptr(cache_layers), _ptr(staging_layers), int(n_layers),
+    rc = (_lib or load()).hs_save_kv_page_slices(_ptr(cache_layers), _ptr(staging_layers), int(n_layers),
                                        _ptr(block_table), int(n_pages), int(page_bytes),
                                        int(rows), int(col_off), int(col_bytes), int(num_blocks),
                                        _ptr(d_err), _stream(stream))
@@ -203,14 +250,14 @@ def hs_save_kv_page_slices(cache_layers, staging_layers, n_layers: int, block_ta
 
 
 def hs_restore_state(src_slots, dst_slots, n: int, floats_each: int, d_err=None, stream=None):
-    rc = load().hs_restore_state(_ptr(src_slots), _ptr(dst_slots), int(n), int(floats_each),
+    rc = (_lib or load()).hs_restore_state(_ptr(src_slots), _ptr(dst_slots), int(n), int(floats_each),
                                  _ptr(d_err), _stream(stream))
     _check(rc, "hs_restore_state")
 
 
 def hs_checkpoint_states(live_states, ckpt_slots, n: int, floats_each: int, d_err=None,
                          stream=None):
-    rc = load().hs_checkpoint_states(_ptr(live_states), _ptr(ckpt_slots), int(n),
+    rc = (_lib or load()).hs_checkpoint_states(_ptr(live_states), _ptr(ckpt_slots), int(n),
                                      int(floats_each), _ptr(d_err), _stream(stream))
     _check(rc, "hs_checkpoint_states")
 
@@ -223,10 +270,10 @@ def make_shape(batch, n_heads, d_k, d_v, max_tokens, kernel=HS_LINATTN_AUTO):
 def _prefill_call(name, shape, q, k, v, log_g, o, state, pos0, n_tokens, ckpt_interval,
                   ckpt_slots, d_err, stream):
     B = int(shape.batch)
-    p0 = (C.c_int64 * max(B, 1))(*[int(x) for x in pos0])
-    nt = (C.c_int32 * max(B, 1))(*[int(x) for x in n_tokens])
-    rc = getattr(load(), name)(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o),
-                               _ptr(state), C.addressof(p0), C.addressof(nt), int(ckpt_interval),
+    p0, keep_p0 = _i64(pos0, B)
+    nt, keep_nt = _i32(n_tokens, B)
+    rc = getattr(_lib or load(), name)(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o),
+                               _ptr(state), p0, nt, int(ckpt_interval),
                                _ptr(ckpt_slots), _ptr(d_err), _stream(stream))
     _check(rc, name)
 
@@ -250,10 +297,10 @@ def hs_test_prefill_stalled(shape: hs_linattn_shape, q, k, v, log_g, o, state, p
 def hs_linattn_scan_workspace_bytes(shape: hs_linattn_shape, pos0, n_tokens) -> int:
     """Bytes of workspace hs_linattn_prefill_scan needs for these arguments."""
     B = int(shape.batch)
-    p0 = (C.c_int64 * max(B, 1))(*[int(x) for x in pos0])
-    nt = (C.c_int32 * max(B, 1))(*[int(x) for x in n_tokens])
+    p0, keep_p0 = _i64(pos0, B)
+    nt, keep_nt = _i32(n_tokens, B)
     out = C.c_int64()
-    rc = load().hs_linattn_scan_workspace_bytes(C.byref(shape), C.addressof(p0), C.addressof(nt),
+    rc = (_lib or load()).hs_linattn_scan_workspace_bytes(C.byref(shape), p0, nt,
                                                 C.addressof(out))
     _check(rc, "hs_linattn_scan_workspace_bytes")
     return out.value
@@ -265,10 +312,10 @@ def hs_linattn_prefill_scan(shape: hs_linattn_shape, q, k, v, log_g, o, state, p
     """Segment-parallel prefill (same arguments as hs_linattn_prefill_from_state plus a device
     workspace of hs_linattn_scan_workspace_bytes bytes)."""
     B = int(shape.batch)
-    p0 = (C.c_int64 * max(B, 1))(*[int(x) for x in pos0])
-    nt = (C.c_int32 * max(B, 1))(*[int(x) for x in n_tokens])
-    rc = load().hs_linattn_prefill_scan(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g),
-                                        _ptr(o), _ptr(state), C.addressof(p0), C.addressof(nt),
+    p0, keep_p0 = _i64(pos0, B)
+    nt, keep_nt = _i32(n_tokens, B)
+    rc = (_lib or load()).hs_linattn_prefill_scan(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g),
+                                        _ptr(o), _ptr(state), p0, nt,
                                         int(ckpt_interval), _ptr(ckpt_slots), _ptr(workspace),
                                         int(workspace_bytes), _ptr(d_err), _stream(stream))
     _check(rc, "hs_linattn_prefill_scan")
@@ -284,11 +331,11 @@ def hs_linattn_prefill_scan_noalloc(shape: hs_linattn_shape, q, k, v, log_g, o, 
     and race; the first call on a device does a one-time set-up and belongs before any stream
     capture."""
     B = int(shape.batch)
-    p0 = (C.c_int64 * max(B, 1))(*[int(x) for x in pos0])
-    nt = (C.c_int32 * max(B, 1))(*[int(x) for x in n_tokens])
-    rc = load().hs_linattn_prefill_scan_noalloc(C.byref(shape), _ptr(q), _ptr(k), _ptr(v),
+    p0, keep_p0 = _i64(pos0, B)
+    nt, keep_nt = _i32(n_tokens, B)
+    rc = (_lib or load()).hs_linattn_prefill_scan_noalloc(C.byref(shape), _ptr(q), _ptr(k), _ptr(v),
                                                 _ptr(log_g), _ptr(o), _ptr(state),
-                                                C.addressof(p0), C.addressof(nt),
+                                                p0, nt,
                                                 int(ckpt_interval), _ptr(ckpt_slots),
                                                 _ptr(d_err), _stream(stream))
     _check(rc, "hs_linattn_prefill_scan_noalloc")
@@ -300,22 +347,22 @@ def hs_linattn_prefill_packed(shape: hs_linattn_shape, q, k, v, log_g, o, state,
     """Packed token layout: token t of problem b is row cu_rows[b] + t.  pos0 / n_tokens /
     cu_rows: host sequences of length batch, batch, batch + 1."""
     B = int(shape.batch)
-    p0 = (C.c_int64 * max(B, 1))(*[int(x) for x in pos0])
-    nt = (C.c_int32 * max(B, 1))(*[int(x) for x in n_tokens])
-    cu = (C.c_int64 * max(B + 1, 1))(*[int(x) for x in cu_rows])
-    rc = load().hs_linattn_prefill_packed(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g),
-                                          _ptr(o), _ptr(state), C.addressof(p0), C.addressof(nt),
-                                          C.addressof(cu), int(ckpt_interval), _ptr(ckpt_slots),
+    p0, keep_p0 = _i64(pos0, B)
+    nt, keep_nt = _i32(n_tokens, B)
+    cu, keep_cu = _i64(cu_rows, B + 1)
+    rc = (_lib or load()).hs_linattn_prefill_packed(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g),
+                                          _ptr(o), _ptr(state), p0, nt,
+                                          cu, int(ckpt_interval), _ptr(ckpt_slots),
                                           _ptr(d_err), _stream(stream))
     _check(rc, "hs_linattn_prefill_packed")
 
 
 def hs_linattn_num_checkpoints(pos0, n_tokens, ckpt_interval: int) -> int:
     B = len(pos0)
-    p0 = (C.c_int64 * max(B, 1))(*[int(x) for x in pos0])
-    nt = (C.c_int32 * max(B, 1))(*[int(x) for x in n_tokens])
+    p0, keep_p0 = _i64(pos0, B)
+    nt, keep_nt = _i32(n_tokens, B)
     tot = C.c_int64()
-    rc = load().hs_linattn_num_checkpoints(B, C.addressof(p0), C.addressof(nt), int(ckpt_interval),
+    rc = (_lib or load()).hs_linattn_num_checkpoints(B, p0, nt, int(ckpt_interval),
                                            C.addressof(tot))
     _check(rc, "hs_linattn_num_checkpoints")
     return tot.value

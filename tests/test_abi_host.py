@@ -368,3 +368,20 @@ def test_c_client_compiles_links_and_runs(tmp_path):
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
     assert "FAIL" not in r.stdout and r.stdout.count("ok ") >= 12
+
+
+@pytest.mark.parametrize("values", [[], [5], list(range(9)), (1, 2, 3), [True, False], [4608.0, 7.9],
+                                    [2 ** 31 + 5, -1], [2 ** 63, 1], range(4), np.arange(4),
+                                    [np.int64(3), np.int32(4)], b"ab"])
+@pytest.mark.parametrize("n_more", [0, 2])
+@pytest.mark.parametrize("code,ctype", [("q", ctypes.c_int64), ("i", ctypes.c_int32)])
+def test_host_arrays_hold_what_element_wise_conversion_gives(values, n_more, code, ctype):
+    """The binding's host arrays: lists and tuples take a short cut; every container, float,
+    wrapped value and short list gives what int() and ctypes give for each element."""
+    n = len(values) + n_more
+    want = list((ctype * max(n, 1))(*[int(x) for x in values]))
+    addr, keep = hs._host_array(code, ctype, values, n)
+    assert list((ctype * max(n, 1)).from_address(addr)) == want
+    if n > 0:
+        with pytest.raises(IndexError):
+            hs._host_array(code, ctype, [1] * (n + 1), n)
