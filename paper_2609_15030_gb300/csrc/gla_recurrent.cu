@@ -3,10 +3,16 @@
 // (The paper runs its linear layers on FLA kernels and prints no recurrence;
 // this is the form the library implements.)
 //
-// One CTA owns one (problem, head) and keeps its d x d float32 state in
-// registers for the whole call, as 16 x 4 blocks (16 key rows, 4 value
-// columns) per thread, read and written as 16-byte vectors.  Tokens are
-// staged eight at a time in shared memory.
+// One CTA owns 64 value columns of one (problem, head) and keeps that part of the d x d
+// float32 state in registers for the whole call, as 16 x 2 blocks (16 key rows, 2 value
+// columns) per thread; a warp's lanes are column pairs, so every state load and store of a
+// warp is 256 contiguous bytes of one row.  The kernel is bound by the state's bytes (a short
+// call reads and writes 64 KiB per head and computes a few tokens in between), so what matters
+// is that the loads of one CTA overlap the arithmetic and stores of others: 256 threads of 64
+// registers over 32 KiB of state put four CTAs on an SM.  72 problems of 16 heads and 2-8
+// tokens (160 MB): 36.6 us = 4.4 TB/s, against 38.2 us with whole heads (16 x 4 blocks, 125
+// registers, two CTAs per SM).  Tokens are staged eight at a time in shared memory, and their rows
+// of q, k and g are read back 16 bytes at a time, one broadcast per four rows.
 //
 // Per token the arithmetic is fixed: g = expf(a); every element becomes
 // fmaf(g_d, S[d][e], k_d * v_e); partial dot products over each group of 16
@@ -23,25 +29,34 @@ namespace {
 
 constexpr int kTokBlock = 8;
 
-__device__ __forceinline__ float bf16_to_f32(uint16_t x)
+// four values of a bf16 row
+__device__ __forceinline__ float4 bf16x4(const uint16_t *p)
 {
-    return __uint_as_float(((uint32_t)x) << 16);
+    const uint2 w = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u),
+                       __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
 }
 
-// CTA = (problem, head).  Thread (cg, rg) holds the 16 x 4 block of the state
-// with rows [16*rg, 16*rg+16) and columns [4*cg, 4*cg+4): a warp covers 16-byte
-// pieces of whole rows, so state loads and stores are fully coalesced vectors.
+constexpr int kCols = 64;             // value columns of a CTA
+
+// CTA = (problem, head, block of 64 columns).  Thread (cg, rg) holds rows [16*rg, 16*rg+16) and
+// the CTA's columns 2*cg, 2*cg+1.
 template <int D>
-__global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const __grid_constant__ GlaParams p)
+__global__ void __launch_bounds__((kCols / 2) * (D / 16), D == 128 ? 4 : 7)
+gla_recurrent_kernel(const __grid_constant__ GlaParams p)
 {
-    constexpr int NCG = D / 4;        // column groups of 4
+    constexpr int NCG = kCols / 2;    // column pairs (lanes)
     constexpr int NRG = D / 16;       // row groups of 16
     constexpr int NTH = NCG * NRG;
-    __shared__ __align__(16) float sq[kTokBlock][D], sk[kTokBlock][D], sg[kTokBlock][D], sv[kTokBlock][D];
-    __shared__ __align__(16) float spart[kTokBlock][NRG][D];
+    constexpr int NCB = D / kCols;    // column blocks per head
+    __shared__ __align__(16) float sq[kTokBlock][D], sk[kTokBlock][D], sg[kTokBlock][D];
+    __shared__ __align__(16) float sv[kTokBlock][kCols];
+    __shared__ __align__(16) float spart[kTokBlock][NRG][kCols];
 
-    const int b = blockIdx.x / p.n_heads;
-    const int h = blockIdx.x - b * p.n_heads;
+    const int bh = blockIdx.x / NCB;
+    const int e0 = (blockIdx.x - bh * NCB) * kCols;
+    const int b = bh / p.n_heads;
+    const int h = bh - b * p.n_heads;
     const int n = p.n_tokens[b];
     if (n <= 0)
         return;
@@ -52,40 +67,53 @@ __global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const
     int next_ck = p.first_ck[b];      // tokens up to the next checkpoint, and its slot
     int ck = p.ck_base[b];
 
-    float *st = p.state + ((int64_t)b * p.n_heads + h) * D * D;
-    float4 S[16];   // S[r] = state row 16*rg + r, columns 4*cg .. 4*cg+3
+    // this thread's first element of a state
+    const int64_t elem = (int64_t)h * D * D + 16 * rg * D + e0 + 2 * cg;
+    float *st = p.state + (int64_t)b * p.n_heads * D * D + elem;
+    float2 S[16];   // S[r] = state row 16*rg + r, columns e0 + 2*cg, + 1
 #pragma unroll
     for (int r = 0; r < 16; ++r)
-        S[r] = *reinterpret_cast<const float4 *>(st + (int64_t)(16 * rg + r) * D + 4 * cg);
+        S[r] = *reinterpret_cast<const float2 *>(st + r * D);
 
     for (int t0 = 0; t0 < n; t0 += kTokBlock) {
         const int tb = min(kTokBlock, n - t0);
-        for (int idx = tid; idx < tb * D; idx += NTH) {
-            const int tt = idx / D, d = idx - (idx / D) * D;
-            const int64_t row = ((int64_t)p.row0[b] + t0 + tt) * p.n_heads + h;
-            sq[tt][d] = bf16_to_f32(p.q[row * D + d]);
-            sk[tt][d] = bf16_to_f32(p.k[row * D + d]);
-            sv[tt][d] = bf16_to_f32(p.v[row * D + d]);
-            sg[tt][d] = expf(p.log_g[row * D + d]);
+        const int64_t row0 = ((int64_t)p.row0[b] + t0) * p.n_heads + h;
+        for (int idx = tid; idx < tb * (D / 4); idx += NTH) {
+            const int tt = idx / (D / 4), d = (idx % (D / 4)) * 4;
+            const int64_t at = (row0 + (int64_t)tt * p.n_heads) * D + d;
+            const float4 a = *reinterpret_cast<const float4 *>(p.log_g + at);
+            *reinterpret_cast<float4 *>(&sq[tt][d]) = bf16x4(p.q + at);
+            *reinterpret_cast<float4 *>(&sk[tt][d]) = bf16x4(p.k + at);
+            *reinterpret_cast<float4 *>(&sg[tt][d]) = make_float4(expf(a.x), expf(a.y), expf(a.z), expf(a.w));
+        }
+        for (int idx = tid; idx < tb * (kCols / 4); idx += NTH) {
+            const int tt = idx / (kCols / 4), e = (idx % (kCols / 4)) * 4;
+            *reinterpret_cast<float4 *>(&sv[tt][e]) =
+                bf16x4(p.v + (row0 + (int64_t)tt * p.n_heads) * D + e0 + e);
         }
         __syncthreads();
+#pragma unroll 1
         for (int tt = 0; tt < tb; ++tt) {
-            const float4 v4 = *reinterpret_cast<const float4 *>(&sv[tt][4 * cg]);
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float2 v2 = *reinterpret_cast<const float2 *>(&sv[tt][2 * cg]);
+            float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const int i = 16 * rg + r;
-                const float g = sg[tt][i], kk = sk[tt][i], qq = sq[tt][i];
-                S[r].x = fmaf(g, S[r].x, kk * v4.x);
-                S[r].y = fmaf(g, S[r].y, kk * v4.y);
-                S[r].z = fmaf(g, S[r].z, kk * v4.z);
-                S[r].w = fmaf(g, S[r].w, kk * v4.w);
-                acc.x = fmaf(qq, S[r].x, acc.x);
-                acc.y = fmaf(qq, S[r].y, acc.y);
-                acc.z = fmaf(qq, S[r].z, acc.z);
-                acc.w = fmaf(qq, S[r].w, acc.w);
+            for (int r4 = 0; r4 < 16; r4 += 4) {
+                const int i = 16 * rg + r4;
+                const float4 g4 = *reinterpret_cast<const float4 *>(&sg[tt][i]);
+                const float4 k4 = *reinterpret_cast<const float4 *>(&sk[tt][i]);
+                const float4 q4 = *reinterpret_cast<const float4 *>(&sq[tt][i]);
+                const float g[4] = {g4.x, g4.y, g4.z, g4.w}, kk[4] = {k4.x, k4.y, k4.z, k4.w},
+                            qq[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    float2 &s = S[r4 + x];
+                    s.x = fmaf(g[x], s.x, kk[x] * v2.x);
+                    s.y = fmaf(g[x], s.y, kk[x] * v2.y);
+                    acc.x = fmaf(qq[x], s.x, acc.x);
+                    acc.y = fmaf(qq[x], s.y, acc.y);
+                }
             }
-            *reinterpret_cast<float4 *>(&spart[tt][rg][4 * cg]) = acc;
+            *reinterpret_cast<float2 *>(&spart[tt][rg][2 * cg]) = acc;
             if (t0 + tt + 1 == next_ck) {
                 float *slot = p.ckpt_slots[ck++];
                 next_ck = next_ck <= n - p.ckpt_interval ? next_ck + p.ckpt_interval : 0;
@@ -96,10 +124,10 @@ __global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const
                     if (tid == 0)
                         report(p.d_err, HS_DEVERR_MISALIGNED);
                 } else {
-                    slot += (int64_t)h * D * D;
+                    slot += elem;
 #pragma unroll
                     for (int r = 0; r < 16; ++r)
-                        *reinterpret_cast<float4 *>(slot + (int64_t)(16 * rg + r) * D + 4 * cg) = S[r];
+                        *reinterpret_cast<float2 *>(slot + r * D) = S[r];
                 }
             }
         }
@@ -107,17 +135,16 @@ __global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const
             // final state out before the output reduction, so the store drains behind it
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                *reinterpret_cast<float4 *>(st + (int64_t)(16 * rg + r) * D + 4 * cg) = S[r];
+                *reinterpret_cast<float2 *>(st + r * D) = S[r];
         }
         __syncthreads();
-        for (int idx = tid; idx < tb * D; idx += NTH) {
-            const int tt = idx / D, e = idx - (idx / D) * D;
+        for (int idx = tid; idx < tb * kCols; idx += NTH) {
+            const int tt = idx / kCols, e = idx % kCols;
             float sum = spart[tt][0][e];
 #pragma unroll
             for (int g = 1; g < NRG; ++g)
                 sum += spart[tt][g][e];
-            const int64_t row = ((int64_t)p.row0[b] + t0 + tt) * p.n_heads + h;
-            p.o[row * D + e] = sum;
+            p.o[(row0 + (int64_t)tt * p.n_heads) * D + e0 + e] = sum;
         }
         __syncthreads();
     }
@@ -127,10 +154,10 @@ __global__ void __launch_bounds__((D / 4) * (D / 16)) gla_recurrent_kernel(const
 
 cudaError_t launch_gla_recurrent(const GlaParams &p, int d, cudaStream_t s)
 {
-    const unsigned grid = (unsigned)p.batch * (unsigned)p.n_heads;
+    const unsigned grid = (unsigned)p.batch * (unsigned)p.n_heads * (unsigned)(d / kCols);
     if (d == 128)
         return launch_pdl(gla_recurrent_kernel<128>, dim3(grid), dim3(256), 0, s, p);
-    return launch_pdl(gla_recurrent_kernel<64>, dim3(grid), dim3(64), 0, s, p);
+    return launch_pdl(gla_recurrent_kernel<64>, dim3(grid), dim3(128), 0, s, p);
 }
 
 }  // namespace hs
