@@ -1277,6 +1277,84 @@ __device__ __forceinline__ void short_outputs(const uint8_t *smem, int L, float 
     }
 }
 
+// ---- operands of a segment's state from the zero state, dS = sum_j K^_j^T v_j with K^_j =
+// k_j 2^{Lam_last - Lam_j} (gla_dstate_kernel and the cluster prefill, same bits in both).  A
+// thread of NWARPS warps owns key dim and value dim (warp mod 4) * 32 + lane and 64 / NWARPS * 4
+// tokens, in groups of 16: Lam_last - Lam_j is the sum of the later groups' log2-decay and a
+// running sum backwards through the group, so strong decay costs no precision.  K^ (tf32)
+// goes to `op`, K-major [D][64 tokens], four tokens per store; V^T (bf16 values, exact in tf32) to
+// the 64 TMEM columns at `vt`; the segment's decay G_d = 2^{Lam_last} to g[d * gstride] (device
+// memory).  All inputs are loaded before the first store: with one thread per key dim walking
+// the 64 tokens and storing as it went, each shared-memory load waited for the store before it
+// (4,608 tokens of 16 heads through hs_linattn_prefill_scan: 112 us, now 106.5; a 512-token
+// tail 18.6 us, now 17.2).  Holds one CTA-wide barrier; the caller makes the operands visible to
+// the tensor core.
+template <int D, int NWARPS>
+__device__ __forceinline__ void dstate_operands(uint8_t *op, const uint16_t *sK, const uint16_t *sV,
+                                                const float *sG, float *sTot, uint32_t tmem, uint32_t vt,
+                                                float *g, int64_t gstride)
+{
+    constexpr int PER = 16 / NWARPS;           // token groups per thread
+    const int warp = thread_id() >> 5, lane = thread_id() & 31;
+    const int d = (warp & 3) * 32 + lane;
+    const int g0 = (warp >> 2) * PER;
+    if (d < D) {
+#pragma unroll
+        for (int y = 0; y < PER; ++y) {
+            float run = 0.f;
+#pragma unroll
+            for (int x = 15; x >= 0; --x)
+                run = fmaf(sG[(16 * (g0 + y) + x) * D + d], kLog2e, run);
+            sTot[(g0 + y) * D + d] = run;
+        }
+    }
+    __syncthreads();
+    if (d >= D)
+        return;
+#pragma unroll 1
+    for (int y = 0; y < PER; ++y) {
+        const int t0 = 16 * (g0 + y);
+        float a[16], k[16];
+        uint32_t v[16];
+#pragma unroll
+        for (int x = 0; x < 16; ++x) {
+            a[x] = sG[(t0 + x) * D + d];
+            k[x] = bf16f(sK[(t0 + x) * D + d]);
+            v[x] = (uint32_t)sV[(t0 + x) * D + d] << 16;
+        }
+        float later = 0.f;                     // log2-decay of the later groups
+#pragma unroll
+        for (int u = 3; u > 0; --u)
+            if (u > g0 + y)
+                later += sTot[u * D + d];
+        float run = 0.f;
+#pragma unroll
+        for (int x = 15; x >= 0; --x) {
+            k[x] = rna_tf32(k[x] * ex2(later + run));
+            run = fmaf(a[x], kLog2e, run);
+        }
+        if (t0 == 0)
+            g[d * gstride] = ex2(later + run);
+#pragma unroll
+        for (int x = 0; x < 16; x += 4)
+            *reinterpret_cast<float4 *>(op + t_off(D, d, t0 + x)) =
+                make_float4(k[x], k[x + 1], k[x + 2], k[x + 3]);
+        tmem_st16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + vt + t0, v);
+    }
+    tmem_wait_st();
+}
+
+// (one thread) dS^T = V^T K^ of those operands into the D TMEM columns at `dst`
+template <int D>
+__device__ __forceinline__ void dstate_issue(uint32_t tmem, uint32_t op, uint32_t vt, uint32_t dst)
+{
+#pragma unroll
+    for (int kk = 0; kk < CH / 8; ++kk)
+        mma_tf32_ts(tmem + dst, tmem + vt + kk * 8,
+                    sdesc_sw128(op + (kk >> 2) * (D * 128) + (kk & 3) * 32, 16, 1024),
+                    idesc_tf32(128, D, 0, 0), kk > 0);
+}
+
 // ---- tensor maps of the q / k / v / log-gate rows ([rows][n_heads * 128], one 64-row x
 // 128-element box per head and segment) ----
 

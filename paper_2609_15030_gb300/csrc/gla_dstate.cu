@@ -8,18 +8,15 @@
 // One unit = one (segment, head).  All 256 threads stage the segment's k, v and log-gates
 // in shared memory with cp.async (zeros past the segment's end, which leave the results
 // unchanged); a CTA stages its next unit as soon as the current one's operands are built, so
-// the copies overlap that unit's products and stores.  Then the 128 key-dim threads walk the 64 tokens backwards, keeping
-// Lam_last - Lam_j as a running sum of the later tokens' log2-gates, and write K^ rounded to
-// tf32 into a K-major operand (token = K), while the 128 value-dim threads put V^T into TMEM
-// (bf16 values, exact in tf32); one thread issues dS^T = V^T K^ as eight M = 128, N = d,
-// K = 8 tf32 products; the eight warps read dS^T back from TMEM and store it row by row
-// (row = key dim), as the state layout wants.  Each key-dim thread also leaves the segment's
-// decay of its row, G_d = 2^{Lam_last} (its final running sum), at element (d, 0) of the
-// segment's start-state block, where the scan reads it before it writes the start state
-// there.  A unit depends only on its segment's inputs, so resumed and full computations
-// produce the same dS and G for a segment.
+// the copies overlap that unit's products and stores.  Then all 256 threads form the operands
+// (dstate_operands: K^ rounded to tf32, token = K, and V^T in TMEM); one thread issues dS^T =
+// V^T K^ as eight M = 128, N = d, K = 8 tf32 products; the eight warps read dS^T back from TMEM
+// and store it row by row (row = key dim), as the state layout wants.  The segment's decay of row
+// d, G_d = 2^{Lam_last}, is left at element (d, 0) of the segment's start-state block, where
+// the scan reads it before it writes the start state there.  A unit depends only on its
+// segment's inputs, so resumed and full computations produce the same dS and G for a segment.
 //
-// Each CTA holds 256 TMEM columns (S^T in 0..d-1, V^T in 128..191) and 97 KiB of shared
+// Each CTA holds 256 TMEM columns (S^T in 0..d-1, V^T in 128..191) and 99 KiB of shared
 // memory, so at most two CTAs share an SM and their TMEM allocations always fit.  The
 // grid is persistent, each CTA walking units blockIdx.x, + gridDim.x, ...  The wait for the
 // products is bounded (1 s): on timeout the CTA reports HS_DEVERR_TIMEOUT, waits once more
@@ -31,10 +28,6 @@ namespace hs {
 namespace {
 
 using namespace ptx;
-using gck::bf16f;
-using gck::ex2;
-using gck::rna_tf32;
-using gck::t_off;
 
 constexpr int kThreads = 256;
 constexpr int kChunk = 64;
@@ -48,7 +41,6 @@ constexpr uint32_t OFF_V = 49152;             // v  bf16 [64][d]                
 constexpr uint32_t OFF_A = 65536;             // log-gates f32 [64][d]                  32 KiB
 constexpr uint32_t kSmemBytes = 98304 + 1024;
 constexpr uint64_t kTimeoutNs = 1000000000ull;
-constexpr float kLog2e = 1.4426950408889634f;
 
 // 16 bytes global -> shared, asynchronous; the first `n` bytes copied, the rest zero-filled
 __device__ __forceinline__ void cp_async16_zfill(void *smem_dst, const void *gmem_src, uint32_t n)
@@ -66,6 +58,7 @@ gla_dstate_kernel(const __grid_constant__ DStateParams p)
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t s_bar;
     __shared__ uint32_t s_tmem;
+    __shared__ float s_tot[4 * D];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const uint32_t sb = smem_u32(smem);
@@ -85,7 +78,6 @@ gla_dstate_kernel(const __grid_constant__ DStateParams p)
     const uint32_t tmem = s_tmem;
     const int64_t tstride = (int64_t)p.n_heads * D;     // elements between consecutive tokens
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
-    constexpr uint32_t idesc = idesc_tf32(128, D, 0, 0);
     uint32_t ph = 0;
     bool aborted = false;
 
@@ -143,44 +135,16 @@ gla_dstate_kernel(const __grid_constant__ DStateParams p)
         const int g = w.g, h = w.h;
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        if (warp < 4) {
-            const int d = tid;
-            if (d < D) {
-                const uint16_t *sk = reinterpret_cast<const uint16_t *>(smem + OFF_K) + d;
-                const float *sa = reinterpret_cast<const float *>(smem + OFF_A) + d;
-                float suf = 0.f;   // log2-decay from token j to the segment's end
-#pragma unroll 16
-                for (int j = kChunk - 1; j >= 0; --j) {
-                    *reinterpret_cast<float *>(smem + OFF_OP + t_off(D, d, j)) =
-                        rna_tf32(bf16f(sk[j * D]) * ex2(suf));
-                    suf = fmaf(sa[j * D], kLog2e, suf);
-                }
-                p.Sn[((int64_t)g * p.n_heads + h) * D * D + (int64_t)d * D] = ex2(suf);
-                fence_proxy_async_smem();
-            }
-        } else if ((warp & 3) * 32 < D) {
-            const int e = (warp & 3) * 32 + lane;
-            const uint16_t *sv = reinterpret_cast<const uint16_t *>(smem + OFF_V) + e;
-#pragma unroll
-            for (int c = 0; c < kChunk; c += 16) {
-                uint32_t w[16];
-#pragma unroll
-                for (int x = 0; x < 16; ++x)
-                    w[x] = (uint32_t)sv[(c + x) * D] << 16;
-                tmem_st16(tmem + lrow + kTmV + c, w);
-            }
-            tmem_wait_st();
-        }
+        gck::dstate_operands<D, kThreads / 32>(
+            smem + OFF_OP, reinterpret_cast<const uint16_t *>(smem + OFF_K),
+            reinterpret_cast<const uint16_t *>(smem + OFF_V), reinterpret_cast<const float *>(smem + OFF_A),
+            s_tot, tmem, kTmV, p.Sn + ((int64_t)g * p.n_heads + h) * D * D, D);
+        fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();   // the operands are built: the staging areas are free
         if (tid == 0) {
             tc_fence_after();
-#pragma unroll
-            for (int kk = 0; kk < kChunk / 8; ++kk)
-                mma_tf32_ts(tmem, tmem + kTmV + kk * 8,
-                            sdesc_sw128(sb + OFF_OP + (kk >> 2) * (D * 128) + (kk & 3) * 32, 16, 1024),
-                            idesc,
-                            kk > 0);
+            gck::dstate_issue<D>(tmem, sb + OFF_OP, kTmV, 0);
             tc_commit(bar);
         }
         // the next unit's inputs arrive while this one's products and stores run
