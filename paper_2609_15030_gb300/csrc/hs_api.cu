@@ -558,7 +558,6 @@ hs_status hs_linattn_prefill_scan(const hs_linattn_shape *shp, const uint16_t *q
         p.state = ws_Sn;
         p.d_err = d_err;
         p.n_heads = s.n_heads;
-        p.no_state_out = 1;
     };
     auto flush = [&]() -> hs_status {
         if (j == 0)

@@ -104,7 +104,6 @@ struct GlaParams {
     int32_t n_heads;
     int32_t ckpt_interval;     // 0: none
     int32_t stall_for_test;    // tensor-core kernel only: one wait that nothing completes (failure-detection tests)
-    int32_t no_state_out;      // tensor-core kernel only: the final state is not written
     int32_t off[HS_MAX_BATCH];      // absolute position of the first token within its chunk
     int32_t first_ck[HS_MAX_BATCH]; // tokens up to the problem's first checkpoint position (which
                                     // may lie past n_tokens); 0: no checkpoints
