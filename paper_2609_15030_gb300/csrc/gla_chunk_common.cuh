@@ -27,7 +27,8 @@ constexpr int NB = 256;   // operand builders (warps 0..7): cumulative gates, Q~
 constexpr int NW = 256;   // state warps (warps 8..15): state passes, masks, epilogues
 constexpr int NT = NB + NW;
 constexpr int kLoader = 0;   // the first builder thread issues every TMA copy
-constexpr int kIssuer = NB;  // the first state thread issues every MMA
+constexpr int kIssuer = NB + 64;  // the state thread that issues every MMA but D_A: in a warp of
+                                  // TMEM lane quarter 2, which has no part in the masking of A
 constexpr int kShort = 8; // segments of at most this many tokens run token by token
 constexpr float kLog2e = 1.4426950408889634f;
 // exact path: log-gates below this are taken at this value.  2^(kGateFloor * log2 e) = 2^-144
@@ -49,27 +50,27 @@ constexpr int kPrefetch = 2;                // segments requested into L2 ahead 
 // shared memory map (offsets from a 1024-byte aligned base), sized for the head width
 // D = d_k = d_v = 128 (a D = 64 head uses the first part of each region).  Operands are
 // K-major with the 128-byte swizzle.
-constexpr uint32_t SET_BYTES = 57344;   // one fast operand set:
+constexpr uint32_t SET_BYTES = 40960;   // one of three fast operand sets:
 constexpr uint32_t S_QH = 0;            //   Q~  fp16 [64 tok i][D]                     16 KiB
 constexpr uint32_t S_KH = 16384;        //   K~  fp16 [64 tok j][D]                     16 KiB
 constexpr uint32_t S_AH = 32768;        //   A   fp16 [64 tok i][64 tok j]                8 KiB
-                                        //   (16 KiB after it unused)
-constexpr uint32_t X_QT = 0;            // exact path (over both sets): Q~ tf32 [64][D]         32 KiB
+constexpr uint32_t X_QT = 0;            // exact path (over the sets): Q~ tf32 [64][D]         32 KiB
 constexpr uint32_t X_LAM = 32768;       //   Lam f32 [64 tok][D], row-major                     32 KiB
 constexpr uint32_t X_B2 = 65536;        //   [A ; K^^T] tf32 [64 i + D][64 tok j]               48 KiB
-constexpr uint32_t OFF_SQ = 114688;     // staged q  bf16 [64][D]                  16 KiB
-constexpr uint32_t OFF_SK = 131072;     // staged k                                 16 KiB
-constexpr uint32_t OFF_SV = 147456;     // staged v                                 16 KiB
-constexpr uint32_t OFF_SG = 163840;     // staged log-gates f32 [64][D]             32 KiB
-constexpr uint32_t OFF_GAM = 196608;    // 2^{Lam_last} per key dim, four slots by chunk number   2 KiB
-constexpr uint32_t OFF_TOT = 198656;    // partial log2-decay totals [token groups][D]        2 KiB
-constexpr uint32_t OFF_RED = 200704;    // per warp [8][8]: builders max |q|, fast-path flag, max |k|,
-                                        //   max |v| (0..3); state warps max |S| (4)
-constexpr uint32_t OFF_BAR = 200960;    // 8 mbarriers
-constexpr uint32_t OFF_MISC = 201024;   // TMEM base address, abort flag, decision, run result
-constexpr uint32_t OFF_DG = 201088;     // diagonal of A in float32, two sets by segment parity:
-                                        //   [set][key-dim half][64 tokens] partial sums  1 KiB
-constexpr uint32_t SMEM_BYTES = 202112 + 1024;
+constexpr uint32_t OFF_SQ = 122880;     // staged q  bf16 [64][D]                  16 KiB
+constexpr uint32_t OFF_SK = 139264;     // staged k                                 16 KiB
+constexpr uint32_t OFF_SV = 155648;     // staged v                                 16 KiB
+constexpr uint32_t OFF_SG = 172032;     // staged log-gates f32 [64][D]             32 KiB
+constexpr uint32_t OFF_GAM = 204800;    // 2^{Lam_last} per key dim, four slots by chunk number   2 KiB
+constexpr uint32_t OFF_TOT = 206848;    // partial log2-decay totals [token groups][D]        2 KiB
+constexpr uint32_t OFF_RED = 208896;    // two sets of [8 warps][8]: builders' max |q|, fast-path flag,
+                                        //   max |k|, max |v| (0..3; set by segment parity); state
+                                        //   warps' max |S| (4; a set per pass, in turn)
+constexpr uint32_t OFF_BAR = 209408;    // 9 mbarriers
+constexpr uint32_t OFF_MISC = 209536;   // TMEM base address, abort flag, decision, run result
+constexpr uint32_t OFF_DG = 209600;     // diagonal of A in float32, with the operand sets:
+                                        //   [set][key-dim half][64 tokens] partial sums  1.5 KiB
+constexpr uint32_t SMEM_BYTES = 211136 + 1024;
 
 // tensor memory: D_O alternates between two buffers by chunk parity, placed on
 // either side of S^T so that [D_O0 | S^T] and [S^T | D_O1] are each one accumulator of
@@ -106,7 +107,8 @@ struct Geo {
     static constexpr uint32_t SHI = TM_S + D;     // exact path: hi part of S^T
     static constexpr uint32_t IDF_ST = idesc_f16(128, D, 1);       // S^T += V^T K~ (K~ read MN-major)
     static constexpr uint32_t IDT_UP = idesc_tf32(128, 64 + D, 0, 0);   // exact: [D_O | S^T] update
-    static constexpr uint32_t STAGE = 3 * CH * D * 2 + CH * D * 4;  // staged q, k, v, log-gates
+    static constexpr uint32_t STAGE = 2 * CH * D * 2 + CH * D * 4;  // staged q, k, log-gates
+    static constexpr uint32_t STAGE_V = CH * D * 2;                 // staged v
 };
 
 struct TmaMaps {
@@ -245,29 +247,31 @@ __device__ __forceinline__ int thread_id()
     return t;
 }
 
-// zero the staged rows past a segment of L < 64 tokens (all threads, or the builder
-// warps only)
-template <int D>
+// zero the staged rows past a segment of L < 64 tokens: q, k and the gates (QKG), v (V), by
+// all threads or the builder warps only; the copies concerned have landed
+template <int D, bool QKG, bool V>
 __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, bool builders_only)
 {
     const int tid = threadIdx.x;
-    constexpr int QV = D / 8, RV = 5 * D / 8;   // 16-byte vectors per q/k/v row, per token
+    constexpr int QV = D / 8, GV = D / 4;   // 16-byte vectors per q/k/v row, per gate row
+    constexpr int RV = (QKG ? 2 * QV + GV : 0) + (V ? QV : 0);
 
     if (L < CH) {
         const int nthr = builders_only ? NB : NT;
         for (int idx = tid; idx < (CH - L) * RV; idx += nthr) {
             const int row = L + idx / RV, c = idx % RV;
             uint4 *dst;
-            if (c < QV)
+            if (QKG && c < QV)
                 dst = reinterpret_cast<uint4 *>(smem + OFF_SQ + row * 2 * D) + c;
-            else if (c < 2 * QV)
+            else if (QKG && c < 2 * QV)
                 dst = reinterpret_cast<uint4 *>(smem + OFF_SK + row * 2 * D) + (c - QV);
-            else if (c < 3 * QV)
-                dst = reinterpret_cast<uint4 *>(smem + OFF_SV + row * 2 * D) + (c - 2 * QV);
+            else if (QKG && c < 2 * QV + GV)
+                dst = reinterpret_cast<uint4 *>(smem + OFF_SG + row * 4 * D) + (c - 2 * QV);
             else
-                dst = reinterpret_cast<uint4 *>(smem + OFF_SG + row * 4 * D) + (c - 3 * QV);
+                dst = reinterpret_cast<uint4 *>(smem + OFF_SV + row * 2 * D) + (c - (RV - QV));
             *dst = make_uint4(0u, 0u, 0u, 0u);
         }
+        fence_proxy_async_smem();   // the next copies overwrite these rows
         if (builders_only)
             bar_builders();
         else
@@ -276,14 +280,13 @@ __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, bool builders_on
 }
 
 
-// ---- fast operands of a staged long segment into set `par` (builder warps).  Thread
+// ---- fast operands of a staged long segment into set iset (builder warps).  Thread
 // (dp, qt) owns key dims 2dp, 2dp+1 for the TPG tokens of group qt (16 tokens x 4 groups at
 // D = 128, 8 x 8 at D = 64): it sums their log2-gates, then runs the cumulative sum again
 // from the earlier groups' totals (shared memory; 2^{Lam_last} into gam slot `gslot`) while
 // it writes Q~ and K~ (token-major, the d-contractions' operands) and K~^T (rows of
-// [A ; K~^T]), fp16, with 4- and 16-byte stores.  Then thread (e, half) packs V^T into TMEM
-// (zeros in the lanes e >= D).  Per warp: max |q|, |k|, |v| and whether every operand fits
-// fp16 (for the guard).  The diagonal A_ii = q_i . k_i (no decay between a token and itself)
+// [A ; K~^T]), fp16, with 4- and 16-byte stores.  Per warp: max |q|, |k| and per thread
+// whether its operands fit fp16 (for the guard).  The diagonal A_ii = q_i . k_i (no decay between a token and itself)
 // is summed in float32 from the bf16 inputs, each warp's 64 key dims by a butterfly, into
 // the set's diagonal partials: fp16 Q~ and K~ would round the terms of that dot product to
 // 11 bits, which a token whose own q . k cancels cannot afford.
@@ -292,26 +295,18 @@ __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, bool builders_on
 // 0, or a total log2-decay below -kLamRange) stops after the totals and returns false: the
 // staged inputs are untouched, so the exact path starts from them without another copy.
 template <int D>
-__device__ __forceinline__ bool build_fast(uint8_t *smem, uint32_t tmem, int L, int par, int gslot)
+__device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int iset, int gslot, float &mq,
+                                           float &mk, bool &ok)
 {
     using G = Geo<D>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool worker = warp < 8;
-    const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;   // this warp's TMEM lane quarter
-    const int colhalf = warp >> 2;
-    const int e_own = (warp & 3) * 32 + lane;                  // TMEM lane = value dim e
-    const int th = colhalf;
     const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
     const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
-    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
     const float *sG = reinterpret_cast<const float *>(smem + OFF_SG);
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
     float *sGam = reinterpret_cast<float *>(smem + OFF_GAM);
-    float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
 
-    if (!worker)
-        return true;
-    zero_tail<D>(smem, L, true);
+    zero_tail<D, true, false>(smem, L, true);
     const int dp = tid % G::DP, qt = tid / G::DP;
     float amax = -INFINITY;
     {
@@ -346,48 +341,71 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, uint32_t tmem, int L, 
             *reinterpret_cast<float2 *>(sGam + gslot * D + 2 * dp) = make_float2(ex2(t0), ex2(t1));
         lam_ok = t0 >= -kLamRange && t1 >= -kLamRange;
     }
-    if (bar_or(1, !(amax <= 0.f && lam_ok))) {
-        if (lane == 0)
-            sRed[warp * 8 + 1] = 0.f;
+    if (bar_or(1, !(amax <= 0.f && lam_ok)))
         return false;
-    }
-    uint8_t *set = smem + par * SET_BYTES;
+    uint8_t *set = smem + iset * SET_BYTES;
     __nv_bfloat162 bq = __float2bfloat162_rn(0.f), bk = bq;   // max |q|, |k|
     __half2 hq = __float2half2_rn(0.f), hk = hq;                 // max |Q~|, |K~| (fp16)
     // runs of 8 tokens; within a run, token pairs: Q~ and K~ as fp16 pairs of key dims
-    float *sDg = reinterpret_cast<float *>(smem + OFF_DG) + par * 128 + (dp >> 5) * 64;
+    float *sDg = reinterpret_cast<float *>(smem + OFF_DG) + iset * 128 + (dp >> 5) * 64;
 #pragma unroll 1
     for (int grp = 0; grp < G::TPG / 8; ++grp) {
+        const int j0 = G::TPG * qt + 8 * grp;
+        // the eight tokens' inputs first: the compiler cannot move a load over the operand stores
+        float2 a[8];
+        uint32_t q2[8], k2[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            a[t] = *reinterpret_cast<const float2 *>(sG + (j0 + t) * D + 2 * dp);
+            q2[t] = *reinterpret_cast<const uint32_t *>(sQ + (j0 + t) * D + 2 * dp);
+            k2[t] = *reinterpret_cast<const uint32_t *>(sK + (j0 + t) * D + 2 * dp);
+        }
         float pd[8];   // q . k over this thread's two key dims, tokens 8 grp + 0..7 of its group
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const int i = G::TPG * qt + 8 * grp + 2 * u + t;
-                const float2 a = *reinterpret_cast<const float2 *>(sG + i * D + 2 * dp);
-                run0 = fmaf(a.x, kLog2e, run0);
-                run1 = fmaf(a.y, kLog2e, run1);
-                const uint32_t q2 = *reinterpret_cast<const uint32_t *>(sQ + i * D + 2 * dp);
-                const uint32_t k2 = *reinterpret_cast<const uint32_t *>(sK + i * D + 2 * dp);
-                const float q0 = __uint_as_float(q2 << 16), q1 = __uint_as_float(q2 & 0xFFFF0000u);
-                const float k0 = __uint_as_float(k2 << 16), k1 = __uint_as_float(k2 & 0xFFFF0000u);
-                const uint32_t qp = pack_h2(q0 * ex2(run0), q1 * ex2(run1));
-                const uint32_t kp = pack_h2(k0 * ex2(-run0), k1 * ex2(-run1));
-                pd[2 * u + t] = fmaf(q1, k1, q0 * k0);
-                *reinterpret_cast<uint32_t *>(set + S_QH + h_off(64, i, 2 * dp)) = qp;
-                *reinterpret_cast<uint32_t *>(set + S_KH + h_off(64, i, 2 * dp)) = kp;
-                bq = bmax_abs(bq, q2);
-                bk = bmax_abs(bk, k2);
-                hq = hmax_abs(hq, qp);
-                hk = hmax_abs(hk, kp);
-            }
+        for (int t = 0; t < 8; ++t) {
+            run0 = fmaf(a[t].x, kLog2e, run0);
+            run1 = fmaf(a[t].y, kLog2e, run1);
+            const float q0 = __uint_as_float(q2[t] << 16), q1 = __uint_as_float(q2[t] & 0xFFFF0000u);
+            const float k0 = __uint_as_float(k2[t] << 16), k1 = __uint_as_float(k2[t] & 0xFFFF0000u);
+            const uint32_t qp = pack_h2(q0 * ex2(run0), q1 * ex2(run1));
+            const uint32_t kp = pack_h2(k0 * ex2(-run0), k1 * ex2(-run1));
+            pd[t] = fmaf(q1, k1, q0 * k0);
+            *reinterpret_cast<uint32_t *>(set + S_QH + h_off(64, j0 + t, 2 * dp)) = qp;
+            *reinterpret_cast<uint32_t *>(set + S_KH + h_off(64, j0 + t, 2 * dp)) = kp;
+            bq = bmax_abs(bq, q2[t]);
+            bk = bmax_abs(bk, k2[t]);
+            hq = hmax_abs(hq, qp);
+            hk = hmax_abs(hk, kp);
         }
-        const int j0 = G::TPG * qt + 8 * grp;
         const float dsum = warp_sum8(pd, lane);
         if ((lane & 3) == 0)
             sDg[j0 + ((lane >> 2) & 7)] = dsum;
     }
-    // V^T: thread (e, half) packs tokens [32 half, 32 half + 32) of value dim e
+    mq = warp_max(bmax_of(bq));
+    mk = warp_max(bmax_of(bk));
+    ok = hmax_of(hq) < kF16Lim && hmax_of(hk) < kF16Lim;
+    return true;
+}
+
+// ... then, once the V^T buffer `par` and the guard words of the segment before are free: V^T,
+// thread (e, half) packing tokens [32 half, 32 half + 32) of value dim e, and the guard words
+// (`built`: whether build_fast went through; if not, a failing flag only)
+template <int D>
+__device__ __forceinline__ void build_values(uint8_t *smem, uint32_t tmem, int L, int par, bool built,
+                                             float mq, float mk, bool ok)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;   // this warp's TMEM lane quarter
+    const int e_own = (warp & 3) * 32 + lane;                  // TMEM lane = value dim e
+    const int th = warp >> 2;
+    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
+    float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + par * 64;
+    if (!built) {
+        if (lane == 0)
+            sRed[warp * 8 + 1] = 0.f;
+        return;
+    }
+    zero_tail<D, false, true>(smem, L, true);
     __nv_bfloat162 bv = __float2bfloat162_rn(0.f);
     {
         uint32_t vpk[16];
@@ -402,15 +420,11 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, uint32_t tmem, int L, 
         }
         tmem_st16(tmem + lrow + TM_V + 32 * par + 16 * th, vpk);
     }
-    float mq = warp_max(bmax_of(bq));
-    float mk = warp_max(bmax_of(bk));
-    float mv = warp_max(bmax_of(bv));
+    const float mv = warp_max(bmax_of(bv));
     // non-increasing Lam (|Q~| <= |q|, |A| <= D max|q| max|k|), a total decay of at most
     // 2^-10 (Q~ of the segment's last tokens keeps its precision) and every fp16 operand below
     // 2^15; NaN fails
-    bool ok = hmax_of(hq) < kF16Lim && hmax_of(hk) < kF16Lim &&
-              mv < kF16Lim;
-    ok = __all_sync(0xffffffffu, ok);
+    ok = __all_sync(0xffffffffu, ok && mv < kF16Lim);
     if (lane == 0) {
         sRed[warp * 8 + 0] = mq;
         sRed[warp * 8 + 1] = ok ? 1.f : 0.f;
@@ -418,14 +432,14 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, uint32_t tmem, int L, 
         sRed[warp * 8 + 3] = mv;
     }
     tmem_wait_st();
-    return true;
 }
 
 
 // ---- state pass (state warps): decay by gam slot gpar (gpar < 0: none), checkpoint slot,
-// fp16 copy of S^T for the next S^T Q~^T, and the largest |S|
+// fp16 copy of S^T for the next S^T Q~^T, and the largest |S| (into maxima set mset)
 template <int D>
-__device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpar, float *slot, bool copy)
+__device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpar, float *slot, bool copy,
+                                           int mset)
 {
     constexpr int CW = Geo<D>::CW;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -434,56 +448,53 @@ __device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpa
     const int colhalf = (warp >> 2) & 1;
     const int e_own = (warp & 3) * 32 + lane;                  // TMEM lane = value dim e
     const float *sGam = reinterpret_cast<const float *>(smem + OFF_GAM);
-    float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
+    float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + mset * 64;
 
     if (!worker)
         return;
     float m = 0.f;
     if (e_own < D) {
-        const int db = colhalf * CW;
-        float r[CW];
+        // 32 columns at a time
+        __half2 hm = __float2half2_rn(0.f);
+#pragma unroll 1
+        for (int db = colhalf * CW; db < colhalf * CW + CW; db += 32) {
+            float r[32];
+            tmem_ld32(tmem + lrow + TM_S + db, r);
+            tmem_wait_ld();
+            if (gpar >= 0) {
+                const float *gam = sGam + gpar * D + db;
 #pragma unroll
-        for (int c0 = 0; c0 < CW; c0 += 32)
-            tmem_ld32(tmem + lrow + TM_S + db + c0, *reinterpret_cast<float(*)[32]>(&r[c0]));
-        tmem_wait_ld();
-        if (gpar >= 0) {
-            const float *gam = sGam + gpar * D + db;
-#pragma unroll
-            for (int c = 0; c < CW / 4; ++c) {
-                const float4 g4 = *reinterpret_cast<const float4 *>(gam + 4 * c);
-                r[4 * c] *= g4.x;
-                r[4 * c + 1] *= g4.y;
-                r[4 * c + 2] *= g4.z;
-                r[4 * c + 3] *= g4.w;
+                for (int c = 0; c < 8; ++c) {
+                    const float4 g4 = *reinterpret_cast<const float4 *>(gam + 4 * c);
+                    r[4 * c] *= g4.x;
+                    r[4 * c + 1] *= g4.y;
+                    r[4 * c + 2] *= g4.z;
+                    r[4 * c + 3] *= g4.w;
+                }
+                tmem_st32(tmem + lrow + TM_S + db, r);
             }
+            if (slot != nullptr) {
 #pragma unroll
-            for (int c0 = 0; c0 < CW; c0 += 32)
-                tmem_st32(tmem + lrow + TM_S + db + c0, *reinterpret_cast<float(*)[32]>(&r[c0]));
-        }
-        if (slot != nullptr) {
-#pragma unroll
-            for (int x = 0; x < CW; ++x)
-                slot[(int64_t)(db + x) * D + e_own] = r[x];
-        }
-        if (copy) {
-            // the fp16 copy, two key dims per column; its largest magnitude (inf past fp16)
-            __half2 hm = __float2half2_rn(0.f);
-#pragma unroll
-            for (int hh = 0; hh < CW / 32; ++hh) {
+                for (int x = 0; x < 32; ++x)
+                    slot[(int64_t)(db + x) * D + e_own] = r[x];
+            }
+            if (copy) {
+                // the fp16 copy, two key dims per column; its largest magnitude (inf past fp16)
                 uint32_t u[16];
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
-                    u[c] = pack_h2(r[32 * hh + 2 * c], r[32 * hh + 2 * c + 1]);
+                    u[c] = pack_h2(r[2 * c], r[2 * c + 1]);
                     hm = hmax_abs(hm, u[c]);
                 }
-                tmem_st16(tmem + lrow + TM_SH + db / 2 + 16 * hh, u);
-            }
-            m = hmax_of(hm);
-        } else {
+                tmem_st16(tmem + lrow + TM_SH + db / 2, u);
+            } else {
 #pragma unroll
-            for (int x = 0; x < CW; ++x)
-                m = fmaxf(m, fabsf(r[x]));
+                for (int x = 0; x < 32; ++x)
+                    m = fmaxf(m, fabsf(r[x]));
+            }
         }
+        if (copy)
+            m = hmax_of(hm);
         tmem_wait_st();
     }
     m = warp_max(m);
@@ -492,10 +503,10 @@ __device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpa
 }
 
 
-// ---- the causally masked intra-chunk matrix A (D_A) -> set par's A operand (state warps of
-// TMEM lane quarters 0 and 1)
+// ---- the causally masked intra-chunk matrix A (D_A buffer `par`) -> operand set iset's A
+// (state warps of TMEM lane quarters 0 and 1)
 template <int D>
-__device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int par)
+__device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int par, int iset)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool worker = warp >= 8;
@@ -508,10 +519,10 @@ __device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int par)
     float r[32];
     tmem_ld32(tmem + lrow + (par ? TM_A1 : TM_A0) + jb, r);
     // the diagonal from the builders' float32 partials (one per 64 key dims)
-    const float *sDg = reinterpret_cast<const float *>(smem + OFF_DG) + par * 128;
+    const float *sDg = reinterpret_cast<const float *>(smem + OFF_DG) + iset * 128;
     const float dg = (i >= jb && i < jb + 32) ? (D == 128 ? sDg[i] + sDg[64 + i] : sDg[i]) : 0.f;
     tmem_wait_ld();
-    uint8_t *set = smem + par * SET_BYTES;
+    uint8_t *set = smem + iset * SET_BYTES;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         uint32_t w[4];
@@ -529,11 +540,9 @@ __device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int par)
 
 
 // ---- output epilogue of a processed segment (state warps): D_O buffer `par` -> o (lane e,
-// 32 rows per warp).  With `spare_issuer`, the warp of the MMA-issuing thread (warp 8) is
-// left out while it issues, and warp 12 (the same TMEM lane quarter) writes both halves.
+// 32 rows per warp)
 template <int D>
-__device__ __forceinline__ void out_epilogue(uint32_t tmem, float *ob, int64_t tstride, int L, int par,
-                                             bool spare_issuer)
+__device__ __forceinline__ void out_epilogue(uint32_t tmem, float *ob, int64_t tstride, int L, int par)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool worker = warp >= 8;
@@ -541,26 +550,23 @@ __device__ __forceinline__ void out_epilogue(uint32_t tmem, float *ob, int64_t t
     const int colhalf = (warp >> 2) & 1;
     const int e_own = (warp & 3) * 32 + lane;                  // TMEM lane = value dim e
 
-    if (!worker || (spare_issuer && warp == 8) || e_own >= D)
+    if (!worker || e_own >= D)
         return;
-    const int h0 = (spare_issuer && warp == 12) ? 0 : colhalf;
-    const int h1 = (spare_issuer && warp == 12) ? 2 : colhalf + 1;
 #pragma unroll 1
-    for (int hh = h0; hh < h1; ++hh) {
-        float r[32];
-        const int ib = hh * 32;
-        tmem_ld32(tmem + lrow + (par ? Geo<D>::O1 : TM_O0) + ib, r);
+    for (int ib = colhalf * 32; ib < colhalf * 32 + 32; ib += 16) {
+        uint32_t r[16];
+        tmem_ld16(tmem + lrow + (par ? Geo<D>::O1 : TM_O0) + ib, r);
         tmem_wait_ld();
         float *op = ob + (int64_t)ib * tstride + e_own;
         if (L == CH) {
 #pragma unroll
-            for (int x = 0; x < 32; ++x)
-                __stcs(op + (int64_t)x * tstride, r[x]);
+            for (int x = 0; x < 16; ++x)
+                __stcs(op + (int64_t)x * tstride, __uint_as_float(r[x]));
         } else {
 #pragma unroll
-            for (int x = 0; x < 32; ++x)
+            for (int x = 0; x < 16; ++x)
                 if (ib + x < L)
-                    __stcs(op + (int64_t)x * tstride, r[x]);
+                    __stcs(op + (int64_t)x * tstride, __uint_as_float(r[x]));
         }
     }
 }
@@ -570,7 +576,7 @@ __device__ __forceinline__ void out_epilogue(uint32_t tmem, float *ob, int64_t t
 
 // (state warps) load a state into TMEM and record its largest |S| (float32) for the guard
 template <int D>
-__device__ __forceinline__ void state_load(uint8_t *smem, uint32_t tmem, const float *src)
+__device__ __forceinline__ void state_load(uint8_t *smem, uint32_t tmem, const float *src, int mset)
 {
     constexpr int CW = Geo<D>::CW;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -579,7 +585,7 @@ __device__ __forceinline__ void state_load(uint8_t *smem, uint32_t tmem, const f
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
     const int colhalf = (warp >> 2) & 1;
     const int e_own = (warp & 3) * 32 + lane;
-    float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
+    float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + mset * 64;
     float r[32];
     float m = 0.f;
     if (e_own < D) {
@@ -649,7 +655,7 @@ __device__ __forceinline__ bool exact_decay(uint8_t *smem, int L)
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
     float *sGam = reinterpret_cast<float *>(smem + OFF_GAM);
     float *sLam = reinterpret_cast<float *>(smem + X_LAM);
-    zero_tail<D>(smem, L, false);
+    zero_tail<D, true, true>(smem, L, false);
     float lam[16];
     bool up = false;
     if (worker) {
@@ -977,7 +983,7 @@ __device__ __forceinline__ bool gates_exact(uint8_t *smem, int L)
     const int tid = thread_id(), dp = tid % G::DP, qt = tid / G::DP;
     const float *sG = reinterpret_cast<const float *>(smem + OFF_SG);
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
-    zero_tail<D>(smem, L, true);
+    zero_tail<D, true, true>(smem, L, true);
     float amax = -INFINITY, r0 = 0.f, r1 = 0.f;
 #pragma unroll
     for (int x = 0; x < G::TPG; ++x) {
@@ -1150,11 +1156,11 @@ __device__ __forceinline__ void exact_issue_update(uint32_t tmem, uint32_t sb)
 
 // ---- fast path MMA groups (issuing thread) ----
 
-// D_A = Q~ K~^T of operand set `par` into its own buffer
+// D_A = Q~ K~^T of an operand set into D_A buffer `par`
 template <int D>
-__device__ __forceinline__ void fast_issue_scores(uint32_t tmem, uint32_t sb, int par)
+__device__ __forceinline__ void fast_issue_scores(uint32_t tmem, uint32_t sb, int par, int iset)
 {
-    const uint32_t setb = sb + (uint32_t)par * SET_BYTES;
+    const uint32_t setb = sb + (uint32_t)iset * SET_BYTES;
 #pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         const uint32_t koff = (kk >> 2) * 8192 + (kk & 3) * 32;
@@ -1165,9 +1171,9 @@ __device__ __forceinline__ void fast_issue_scores(uint32_t tmem, uint32_t sb, in
 
 // D_O = S^T Q~^T (A operand: the fp16 copy of S^T; the update product accumulates onto it)
 template <int D>
-__device__ __forceinline__ void fast_issue_sq(uint32_t tmem, uint32_t sb, int par)
+__device__ __forceinline__ void fast_issue_sq(uint32_t tmem, uint32_t sb, int par, int iset)
 {
-    const uint32_t setb = sb + (uint32_t)par * SET_BYTES;
+    const uint32_t setb = sb + (uint32_t)iset * SET_BYTES;
 #pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         const uint32_t koff = (kk >> 2) * 8192 + (kk & 3) * 32;
@@ -1182,9 +1188,9 @@ __device__ __forceinline__ void fast_issue_sq(uint32_t tmem, uint32_t sb, int pa
 // 1 KiB apart (stride byte offset), 16 tokens = 2 KiB per step.
 // (WITH_STATE false: D_O only, for launches that discard the state)
 template <int D, bool WITH_STATE = true>
-__device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, int par)
+__device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, int par, int iset)
 {
-    const uint32_t setb = sb + (uint32_t)par * SET_BYTES;
+    const uint32_t setb = sb + (uint32_t)iset * SET_BYTES;
     const uint32_t vt = tmem + TM_V + 32 * par;
 #pragma unroll
     for (int kk = 0; kk < CH / 16; ++kk) {
@@ -1202,7 +1208,7 @@ __device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, in
 // update S in TMEM, write the slot and the largest |S|, and leave each token's group partials
 // in the operand sets) ...
 template <int D>
-__device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L, float *slot)
+__device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L, float *slot, int mset)
 {
     constexpr int CW = Geo<D>::CW, NG = Geo<D>::NG;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1214,7 +1220,7 @@ __device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L,
     const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
     const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
     float *sG = reinterpret_cast<float *>(smem + OFF_SG);
-    float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
+    float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + mset * 64;
     for (int idx = tid; idx < L * D; idx += NT)
         sG[idx] = expf(sG[idx]);
     __syncthreads();

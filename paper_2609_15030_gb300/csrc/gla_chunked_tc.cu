@@ -23,14 +23,14 @@
 // D_A = Q~ K~^T, then per 16 tokens D_O += V^T A^T (N = 64) and S^T += V^T K~
 // (N = D, the K~ tile read MN-major), V^T in TMEM.  fp16 keeps the 10-bit
 // mantissa of tf32 but halves the instructions (K = 16 per MMA).  The CTA's
-// 16 warps form two groups in a pipeline over two alternating operand sets:
+// 16 warps form two groups in a pipeline over three operand sets in turn:
 // while the eight state warps finish chunk c (the state pass, which applies
 // the pending decay 2^{Lam_last}, writes a due checkpoint and refreshes the
 // fp16 copy of S^T; the causal mask with each token's own score summed in
 // float32 on the diagonal; the output epilogue) the eight builder warps stage
-// chunk c+1 and build its operands (cumulative decay scan, Q~, K~, V^T).  The
-// first builder thread issues the TMA copies and D_A, the first state thread
-// the other MMAs.
+// chunk c+1 and build its operands (cumulative decay scan, Q~, K~, V^T).  Threads
+// of two builder warps and a state warp issue the TMA copies, one state thread
+// the MMAs (the first builder thread D_A in the RESTART instantiation).
 //
 // A chunk is fast only if every fp16 operand provably stays below 2^15 in
 // magnitude (|q|, |v|, |K~|, the bound 128 max|q| max|k| on |A|, and a bound
@@ -81,8 +81,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     volatile uint32_t *sMisc = reinterpret_cast<volatile uint32_t *>(smem + OFF_MISC);
     const uint32_t bar_tma = sb + OFF_BAR, bar_a = sb + OFF_BAR + 8, bar_o = sb + OFF_BAR + 16,
                    bar_s = sb + OFF_BAR + 24, bar_built = sb + OFF_BAR + 32,
-                   bar_go = sb + OFF_BAR + 40, bar_ld = sb + OFF_BAR + 48,
-                   bar_a1 = sb + OFF_BAR + 56;
+                   bar_go = sb + OFF_BAR + 40, bar_v = sb + OFF_BAR + 48,
+                   bar_a1 = sb + OFF_BAR + 56, bar_ld = sb + OFF_BAR + 64;
 
     const int tid = threadIdx.x, warp = tid >> 5;
     // (signed: the unsigned division left the d = 128 kernel with 56 bytes of spills, which cost
@@ -104,8 +104,9 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         mbar_init(bar_s, 1);
         mbar_init(bar_built, 1);
         mbar_init(bar_go, 1);
-        mbar_init(bar_ld, 1);
+        mbar_init(bar_v, 1);
         mbar_init(bar_a1, 1);
+        mbar_init(bar_ld, 1);
         fence_mbar_init();
         sMisc[1] = 0;   // abort flag
     }
@@ -131,10 +132,10 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
 
     // bookkeeping of the loader (copies issued, one still in flight) and of the issuer,
     // for the waits and the abort path; every mbarrier is waited on by one thread only
-    uint32_t n_tma = 0;
-    bool tma_pending = false;
-    uint32_t ph_tma = 0, ph_o = 0, ph_s = 0, ph_built = 0, ph_go = 0;
-    uint32_t ph_a0 = 0, ph_a1 = 0;   // D_A products of even / odd segments (bar_a, bar_a1)
+    uint32_t n_tma = 0, n_v = 0;      // copies of (q, k, gates) and of v
+    bool tma_pending = false, v_pending = false;
+    uint32_t ph_tma = 0, ph_v = 0, ph_o = 0, ph_s = 0, ph_built = 0, ph_go = 0;
+    uint32_t ph_a = 0, ph_a1 = 0;    // D_A products (RESTART: of even / odd segments)
     bool aborted = false;
 
     // L2 prefetch of the 64 tokens `ahead` tokens past token t (if any are this problem's)
@@ -151,19 +152,25 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // (loader) staged inputs of the segment at local position tok_local; segments after
     // the first start on the 64-token grid, so the segment kPrefetch ahead starts at
     // tok_local + 64 * kPrefetch and is requested into L2 now
-    auto copy_inputs = [&](int tok_local) {
+    // (q, k and the gates, then v, which the builders are done with later)
+    auto copy_qkg = [&](int tok_local) {
         const int32_t y = p.row0[b] + tok_local;
         const int32_t x = h * D;
         mbar_arrive_expect_tx(bar_tma, Geo<D>::STAGE);
         tma_load_2d(sb + OFF_SG, &maps.g, x, y, bar_tma);
         tma_load_2d(sb + OFF_SQ, &maps.q, x, y, bar_tma);
         tma_load_2d(sb + OFF_SK, &maps.k, x, y, bar_tma);
-        tma_load_2d(sb + OFF_SV, &maps.v, x, y, bar_tma);
+    };
+    auto copy_v = [&](int tok_local) {
+        mbar_arrive_expect_tx(bar_v, Geo<D>::STAGE_V);
+        tma_load_2d(sb + OFF_SV, &maps.v, h * D, p.row0[b] + tok_local, bar_v);
     };
     auto issue_tma = [&](int tok_local) {
-        copy_inputs(tok_local);
+        copy_qkg(tok_local);
+        copy_v(tok_local);
         ++n_tma;
-        tma_pending = true;
+        ++n_v;
+        tma_pending = v_pending = true;
         if (tok_local > 0)
             prefetch(tok_local, CH * kPrefetch);
     };
@@ -183,10 +190,6 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             aborted = true;
         return !stop;
     };
-    auto wait_tma = [&]() -> bool {
-        tma_pending = false;
-        return wait_all(kLoader, bar_tma, ph_tma);
-    };
     auto wait_group = [&](int id, int who, uint32_t bar, uint32_t &ph) -> bool {
         bool bad = false;
         if (tid == who)
@@ -195,6 +198,40 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             sMisc[1] = 1;
         ph ^= 1;
         const bool stop = bar_or(id, bad || sMisc[1] != 0);
+        tc_fence_after();
+        if (stop)
+            aborted = true;
+        return !stop;
+    };
+    // (builders) `bar` and the copy of v, waited for by the loader with one barrier
+    auto wait_group_v = [&](uint32_t bar, uint32_t &ph) -> bool {
+        bool bad = false;
+        if (tid == kLoader)
+            bad = !mbar_wait_bounded(bar, ph, kTimeoutNs) || !mbar_wait_bounded(bar_v, ph_v, kTimeoutNs);
+        if (bad)
+            sMisc[1] = 1;
+        ph ^= 1;
+        ph_v ^= 1;
+        v_pending = false;
+        const bool stop = bar_or(1, bad || sMisc[1] != 0);
+        tc_fence_after();
+        if (stop)
+            aborted = true;
+        return !stop;
+    };
+    // (state warps) the next segment built and, if `o` as well, the issued products complete,
+    // waited for by the issuer with one barrier
+    auto wait_group_o = [&](bool o) -> bool {
+        bool bad = false;
+        if (tid == kIssuer)
+            bad = (o && !mbar_wait_bounded(bar_o, ph_o, kTimeoutNs)) ||
+                  !mbar_wait_bounded(bar_built, ph_built, kTimeoutNs);
+        if (bad)
+            sMisc[1] = 1;
+        if (o)
+            ph_o ^= 1;
+        ph_built ^= 1;
+        const bool stop = bar_or(2, bad || sMisc[1] != 0);
         tc_fence_after();
         if (stop)
             aborted = true;
@@ -212,6 +249,13 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         if (stop)
             aborted = true;
         return !stop;
+    };
+    // both copies of the staged inputs, CTA-wide
+    auto wait_tma = [&]() -> bool {
+        tma_pending = false;
+        if (builder && !wait_group_v(bar_tma, ph_tma))
+            sMisc[1] = 1;
+        return sync_all();
     };
     auto seg_len = [&](int at) -> int { return min(n - at, CH - (int)(((uint32_t)at + off) & (CH - 1))); };
     auto is_long = [&](int at) -> bool { return at < n && seg_len(at) > kShort; };
@@ -231,14 +275,18 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         }
         return slot + (int64_t)h * D * D;
     };
+    int smax = 0;   // maxima set of the last state pass (state warps)
     // largest |S| recorded by the last state pass (valid after the barrier that follows it)
     auto state_max = [&]() -> float {
         float m = 0.f;
 #pragma unroll
         for (int w = 0; w < 8; ++w)
-            m = fmaxf(m, sRed[w * 8 + 4]);
+            m = fmaxf(m, sRed[smax * 64 + w * 8 + 4]);
         return m;
     };
+    // the set the next pass records its maximum in: the other one, since a warp may still be
+    // reading the last
+    auto next_max = [&]() -> int { return smax ^= 1; };
 
     if (tid == kLoader)
         issue_tma(0);
@@ -248,7 +296,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // largest magnitude.  The builders meanwhile stage and build the first segment.
     float *st_g = p.state + ((int64_t)(RESTART ? p.ck_base[b] : b) * p.n_heads + h) * D * D;
     if (worker) {
-        state_load<D>(smem, tmem, st_g);
+        state_load<D>(smem, tmem, st_g, next_max());
         tc_fence_before();
         bar_staters();
         tc_fence_after();
@@ -261,7 +309,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // pending): the per-token recurrence with the recurrent kernel's exact operation order
     // (fma chains over groups of 16 key rows, group partials summed left to right)
     auto short_segment = [&](int tok_s, int L) {
-        short_state<D>(smem, tmem, L, worker ? ckpt_slot(tok_s + L) : nullptr);
+        short_state<D>(smem, tmem, L, worker ? ckpt_slot(tok_s + L) : nullptr, next_max());
         if (tid == kLoader && tok_s + L < n)
             issue_tma(tok_s + L);
         short_outputs<D>(smem, L, outp(tok_s), tstride);
@@ -270,20 +318,22 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         tc_fence_after();
     };
 
+    int kseq = 0;   // long segments of the current run so far (slot of 2^{Lam_last}: kseq mod 4)
     // the guard of a built fast segment (state warps, after the wait for the builders): log-gates
     // <= 0, and every fp16 operand (Q~, K~, V, A, the fp16 copy of the state it starts from)
     // below 2^15 in magnitude.  Returns whether the segment's own inputs pass; `state_ok` says
     // whether the state (its measured magnitude, or a bound on it) passes too.
     float mk_new = 0.f, mv_new = 0.f;
     auto guard = [&](float s_mag, bool &state_ok) -> bool {
+        const float *red = sRed + (kseq & 1) * 64;
         float mq = 0.f, mk = 0.f, mv = 0.f;
         bool ok = true;
 #pragma unroll
         for (int w = 0; w < 8; ++w) {
-            mq = fmaxf(mq, sRed[w * 8 + 0]);
-            ok = ok && sRed[w * 8 + 1] != 0.f;
-            mk = fmaxf(mk, sRed[w * 8 + 2]);
-            mv = fmaxf(mv, sRed[w * 8 + 3]);
+            mq = fmaxf(mq, red[w * 8 + 0]);
+            ok = ok && red[w * 8 + 1] != 0.f;
+            mk = fmaxf(mk, red[w * 8 + 2]);
+            mv = fmaxf(mv, red[w * 8 + 3]);
         }
         mk_new = mk;
         mv_new = mv;
@@ -308,15 +358,15 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         if (builder) {
             if (tid == kLoader && seg_end < n)
                 issue_tma(seg_end);
-            if (ahead && wait_group(1, kLoader, bar_tma, ph_tma)) {
+            if (ahead && wait_group_v(bar_tma, ph_tma)) {
                 tma_pending = false;
                 const bool exact = gates_exact<D>(smem, seg_len(seg_end));
                 if (tid == kLoader)
                     sMisc[9] = exact ? 1u : 2u;
             }
         } else if (wait_group(2, kIssuer, bar_o, ph_o)) {
-            state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false);   // checkpoint and |S| of the final state
-            out_epilogue<D>(tmem, outp(tok_s), tstride, L, 0, false);
+            state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false, next_max());   // checkpoint and |S| of the final state
+            out_epilogue<D>(tmem, outp(tok_s), tstride, L, 0);
         }
         tc_fence_before();
         if (!sync_all())
@@ -331,7 +381,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // Handoffs (each mbarrier has one waiting thread and one arriving party):
     //   bar_built: builders -> state warps, segment k built (operands, V^T, guard maxima)
     //   bar_go:    state warps -> builders, the decision on segment k is made (sMisc[2]);
-    //              when it is fast, it also means the operand set of segment k+1 is free
+    //              when it is fast, it also means the V^T and D_A buffers of segment k+1 are free
     //              (the products of segment k-1 are complete)
     // A run ends after the last long segment, before a segment whose own inputs the guard
     // sends to the exact path, or before a segment whose state bound fails: a decision inside a
@@ -339,14 +389,23 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // such a segment starts a new run, whose first decision reads the measured state exactly as
     // a run resumed from a checkpoint at that segment does.  The groups then meet CTA-wide.
     // No MMA is in flight at either end.
-    int kseq = 0;   // long segments of the current run so far (slot of 2^{Lam_last}: kseq mod 4)
+    // The builders run up to one segment ahead of the decisions: Q~ and K~ of segment k+1 go into
+    // a third operand set while segment k is judged and segment k-1 finishes; only V^T and the
+    // guard words wait for "go" on segment k, and only then are the next segment's q, k and gates
+    // copied over the consumed ones (v, consumed last, follows from the state warps).  With two
+    // sets and one copy of all four, the builders' chain (build, hand over, issue, wait for the
+    // decision, wait for the copy) set the pace at ~9 k cycles a segment; the D_A and copy issues
+    // (~1 k cycles of single-thread work) and two barriers a segment are off it, and the state
+    // warps' passes run in rolled halves (less code, fewer registers): 4 x 32 heads of 16,384
+    // tokens 1,088 -> 1,001 us, 256-token tails of 9 x 16 heads 28.5 -> 27.8 us.
     auto builder_run = [&](int rtok, bool waited) {
-        int par = 0;
+        int iset = 0;
         while (true) {
             const int L = seg_len(rtok);
-            if (!waited && !wait_group(1, kLoader, bar_tma, ph_tma))
+            // a run's first segment: both copies (unless the look ahead has waited for them)
+            if (kseq > 0 ? !wait_group(1, kLoader, bar_tma, ph_tma)
+                         : !waited && !wait_group_v(bar_tma, ph_tma))
                 return;
-            waited = false;
             tma_pending = false;
             if (tid == kLoader && !prefetched) {
                 // once the first segment has landed (the state and the first segment are
@@ -355,134 +414,143 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                 for (int j = 1; j <= kPrefetch; ++j)
                     prefetch(rtok + L, CH * (j - 1));
             }
-            const bool built = build_fast<D>(smem, tmem, L, par, kseq & 3);
+            float mq, mk;
+            bool ok;
+            const bool built = build_fast<D>(smem, L, iset, kseq & 3, mq, mk, ok);
             fence_proxy_async_smem();
+            // the decision on the segment before, and v; for the first segment only a barrier
+            // before the staged rows are overwritten
+            const bool more = rtok + L < n;
+            if (kseq > 0) {
+                if (!wait_group_v(bar_go, ph_go) || sMisc[2] == 0)
+                    return;
+            } else if (built && more && !sync_group(1)) {
+                return;
+            }
+            // q, k and the gates are consumed: stage those of the next segment (long or short); an
+            // exact decision on this one reloads it
+            if (tid == kLoader && built && more) {
+                ++n_tma;
+                ++n_v;
+                tma_pending = v_pending = true;
+            }
+            if (tid == kLoader + 32 && built && more)
+                copy_qkg(rtok + L);
+            build_values<D>(smem, tmem, L, kseq & 1, built, mq, mk, ok);
             tc_fence_before();
             if (!sync_group(1))
                 return;
-            const int next = rtok + L;
-            const bool next_long = is_long(next);
             if (tid == kLoader) {
                 sMisc[8] = built ? 1u : 0u;
                 mbar_arrive(bar_built);
-            }
-            if (built) {
-                // three threads of different warps, so that these issues overlap: D_A = Q~ K~^T of
-                // this segment into its own buffer (the state warps wait on bar_a / bar_a1 by parity
-                // before they read it); the staged rows are consumed, so the next segment (long
-                // or short) is staged now (an exact decision on this one reloads it); and the
-                // segment kPrefetch further on is requested into L2
-                const bool more = next < n;
-                if (tid == kLoader) {
+                if (RESTART && built) {
+                    // D_A at once: the state warps have their start state to load as well, and
+                    // many restart CTAs have a single segment, whose latency this shortens
                     tc_fence_after();
-                    fast_issue_scores<D>(tmem, sb, par);
-                    tc_commit(par ? bar_a1 : bar_a);
-                    if (more) {
-                        ++n_tma;
-                        tma_pending = true;
-                    }
-                } else if (tid == kLoader + 32 && more) {
-                    copy_inputs(next);
-                } else if (tid == kLoader + 64) {
-                    prefetch(next, CH * kPrefetch);
+                    fast_issue_scores<D>(tmem, sb, kseq & 1, iset);
+                    tc_commit((kseq & 1) ? bar_a1 : bar_a);
                 }
             }
-            if (!wait_group(1, kLoader, bar_go, ph_go))
+            if (!built || !is_long(rtok + L)) {
+                wait_group(1, kLoader, bar_go, ph_go);   // the run ends with this segment
                 return;
-            if (sMisc[2] == 0 || !next_long)
-                return;
+            }
             rtok += L;
-            par ^= 1;
+            iset = iset == 2 ? 0 : iset + 1;
             ++kseq;
         }
     };
-    auto state_run = [&](int rtok) {
-        int par = 0;
-        bool pend = false;
-        uint32_t stop = 0;   // why the run ended: 0 done or short segment, 1 exact, 2 new run
-        int pend_par = 0, pend_L = 0, pend_g = 0, pend_tok = 0;
-        float mk_cur = 0.f, mv_cur = 0.f;
-        if (!wait_group(2, kIssuer, bar_built, ph_built))
-            return;
-        // first segment of a run: the measured state (float32 maximum of the last state pass
-        // or of the loaded state)
-        bool state_ok;
-        bool fast = guard(state_max(), state_ok) && state_ok;
+    // What the builders leave to the state warps, which wait for them each segment: (issuer) D_A =
+    // Q~ K~^T of a built segment, into its own buffer; (one thread each of two other warps) the copy
+    // of the next segment's v, now that a built segment's own is packed (an early stopped build
+    // has not consumed it), and the L2 requests of the segment kPrefetch further on
+    auto issue_scores = [&](int par, int iset) {
         if (tid == kIssuer) {
-            sMisc[2] = fast ? 1u : 0u;
-            if (!fast)
-                mbar_arrive(bar_go);
+            fast_issue_scores<D>(tmem, sb, par, iset);
+            tc_commit(bar_a);
         }
-        stop = fast ? 0u : 1u;
-        // a segment sent to the exact path: its (unused) D_A product is drained first
-        if (!fast && sMisc[8] != 0 && !wait_group(2, kIssuer, bar_a, ph_a0))
-            return;
-        while (fast) {
+        __syncwarp();
+    };
+    auto copy_next_v = [&](int next) {
+        if (tid == NB + 96 && sMisc[8] != 0 && next < n)
+            copy_v(next);
+        if (tid == NB + 7 * 32)
+            prefetch(next, CH * kPrefetch);
+        __syncwarp();
+    };
+    // Per segment the state warps' chain is: built (with the products of the segment before),
+    // decision, state pass, D_A, the mask of A beside the issue of D_O, the issue of the update;
+    // the outputs of the segment before are written behind that, while the update runs.
+    auto state_run = [&](int rtok) {
+        int iset = 0;
+        bool drained = true;   // no products outstanding
+        uint32_t stop = 0;   // why the run ended: 0 done or short segment, 1 exact, 2 new run
+        int pend_L = 0;        // the previous segment's tokens
+        float mk_cur = 0.f, mv_cur = 0.f;
+        while (true) {
+            // the segment at rtok built, and the products of the previous one complete: the V^T and
+            // D_A buffers of the next one are free
+            tc_fence_before();
+            if (!wait_group_o(kseq > 0))
+                return;
+            drained = true;
+            // first segment of a run: the measured state (float32 maximum of the last state pass
+            // or of the loaded state).  Else the state it starts from is bounded by the fp16
+            // copy's largest |S| at the previous segment's start plus that segment's largest
+            // update, 64 max|k| max|v| (the decay factors are <= 1)
+            bool state_ok;
+            const bool inputs_ok =
+                guard(kseq > 0 ? (state_max() + 64.0f * mk_cur * mv_cur) * kBoundMargin : state_max(), state_ok);
+            const bool fast = inputs_ok && state_ok;
+            if (tid == kIssuer) {
+                sMisc[2] = fast ? 1u : 0u;
+                mbar_arrive(bar_go);
+            }
             const int L = seg_len(rtok);
+            copy_next_v(rtok + L);
+            if (!fast) {
+                stop = kseq > 0 && inputs_ok ? 2u : 1u;   // the exact path or a new run takes this segment
+                break;
+            }
+            issue_scores(kseq & 1, iset);
             mk_cur = mk_new;
             mv_cur = mv_new;
-            if (pend && !wait_group(2, kIssuer, bar_o, ph_o))
-                return;
-            // the products of the previous segment are complete: its operand set is free
-            if (tid == kIssuer)
-                mbar_arrive(bar_go);
-            state_pass<D>(smem, tmem, pend ? pend_g : -1, pend ? ckpt_slot(rtok) : nullptr, true);
+            state_pass<D>(smem, tmem, kseq > 0 ? (kseq - 1) & 3 : -1,
+                          kseq > 0 ? ckpt_slot(rtok) : nullptr, true,
+                          next_max());
             tc_fence_before();
-            if (!sync_group(2))
+            // the state in place, and D_A of this segment
+            if (!wait_group(2, kIssuer, bar_a, ph_a))
                 return;
-            if (tid == kIssuer) {
-                // D_O = S^T Q~^T (the N = 192 product below accumulates onto it in order)
-                tc_fence_after();
-                fast_issue_sq<D>(tmem, sb, par);
-            }
-            if (pend)
-                out_epilogue<D>(tmem, outp(pend_tok), tstride, pend_L, pend_par, true);
-            // D_A of this segment (issued by the builders' loader)
-            if (!(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
-                return;
-            a_build<D>(smem, tmem, par);
+            if (tid == kIssuer)
+                fast_issue_sq<D>(tmem, sb, kseq & 1, iset);   // D_O = S^T Q~^T
+            __syncwarp();
+            a_build<D>(smem, tmem, kseq & 1, iset);
             fence_proxy_async_smem();
             tc_fence_before();
             if (!sync_group(2))
                 return;
             if (tid == kIssuer) {
                 tc_fence_after();
-                fast_issue_update<D>(tmem, sb, par);
+                fast_issue_update<D>(tmem, sb, kseq & 1, iset);
                 tc_commit(bar_o);
             }
-            pend = true;
-            pend_par = par;
-            pend_tok = rtok;
+            __syncwarp();
+            if (kseq > 0)
+                out_epilogue<D>(tmem, outp(rtok - pend_L), tstride, pend_L, (kseq - 1) & 1);
+            drained = false;
             pend_L = L;
-            pend_g = kseq & 3;
             rtok += L;
-            par ^= 1;
+            iset = iset == 2 ? 0 : iset + 1;
             ++kseq;
             if (!is_long(rtok))
                 break;
-            // the builders' next segment, and the decision on it: the state it starts from is
-            // bounded by the fp16 copy's largest |S| at this segment's start plus this segment's
-            // largest update, 64 max|k| max|v| (the decay factors are <= 1)
-            if (!wait_group(2, kIssuer, bar_built, ph_built))
-                return;
-            const bool inputs_ok =
-                guard((state_max() + 64.0f * mk_cur * mv_cur) * kBoundMargin, state_ok);
-            fast = inputs_ok && state_ok;
-            if (tid == kIssuer) {
-                sMisc[2] = fast ? 1u : 0u;
-                if (!fast)
-                    mbar_arrive(bar_go);
-            }
-            stop = fast ? 0u : (inputs_ok ? 2u : 1u);
-            if (!fast && sMisc[8] != 0 &&
-                !(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
-                return;
         }
-        if (pend) {
-            if (!wait_group(2, kIssuer, bar_o, ph_o))
+        if (kseq > 0) {
+            if (!drained && !wait_group(2, kIssuer, bar_o, ph_o))
                 return;
-            state_pass<D>(smem, tmem, pend_g, ckpt_slot(rtok), false);
-            out_epilogue<D>(tmem, outp(pend_tok), tstride, pend_L, pend_par, false);
+            state_pass<D>(smem, tmem, (kseq - 1) & 3, ckpt_slot(rtok), false, next_max());
+            out_epilogue<D>(tmem, outp(rtok - pend_L), tstride, pend_L, (kseq - 1) & 1);
             tc_fence_before();
             if (!sync_group(2))
                 return;
@@ -508,85 +576,78 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                      : "memory");
     };
     auto state_run_restart = [&](int rtok) {
-        int par = 0;
-        bool pend = false;
+        int iset = 0;
+        bool drained = true;
+        auto wait_scores = [&]() -> bool {
+            return (kseq & 1) ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a);
+        };
         uint32_t stop = 0;   // 0 done or short segment, 1 exact
-        int pend_par = 0, pend_L = 0, pend_tok = 0;
+        int pend_L = 0;
         while (true) {
             const int L = seg_len(rtok);
-            if (!wait_group(2, kIssuer, bar_built, ph_built))
-                return;
             if (loaded != seg_idx(rtok)) {
-                state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rtok) * p.n_heads * D * D);
+                state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rtok) * p.n_heads * D * D, next_max());
                 loaded = seg_idx(rtok);
             }
-            // the loaded state (its TMEM columns and its largest |S|) visible to the group
+            // the loaded state (its TMEM columns and its largest |S|) visible to the group, the
+            // segment built, the products of the previous one complete
             tc_fence_before();
-            if (!sync_group(2))
+            if (!wait_group_o(kseq > 0))
                 return;
-            tc_fence_after();
+            drained = true;
             bool state_ok;
             const bool fast = guard(state_max(), state_ok) && state_ok;
             if (tid == kIssuer) {
                 sMisc[2] = fast ? 1u : 0u;
-                if (!fast)
-                    mbar_arrive(bar_go);
+                mbar_arrive(bar_go);
             }
+            copy_next_v(rtok + L);
             if (!fast) {
                 // the exact path takes this segment: its (unused) D_A product drained first
                 stop = 1;
-                if (sMisc[8] != 0 &&
-                    !(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
+                if (sMisc[8] != 0 && !wait_scores())
                     return;
                 break;
             }
             if (tid == kIssuer && is_long(rtok + L))
                 prefetch_state(rtok + L);   // read by the load at the end of this segment
-            if (pend && !wait_group(2, kIssuer, bar_o, ph_o))
-                return;
-            // the products of the previous segment are complete: its operand set is free
-            if (tid == kIssuer)
-                mbar_arrive(bar_go);
-            state_pass<D>(smem, tmem, -1, nullptr, true);   // the fp16 copy of S for D_O
+            __syncwarp();
+            state_pass<D>(smem, tmem, -1, nullptr, true, next_max());   // the fp16 copy of S for D_O
             tc_fence_before();
-            if (!sync_group(2))
+            if (!wait_scores())
                 return;
-            if (tid == kIssuer) {
-                tc_fence_after();
-                fast_issue_sq<D>(tmem, sb, par);
-            }
-            if (pend)
-                out_epilogue<D>(tmem, outp(pend_tok), tstride, pend_L, pend_par, true);
-            if (!(par ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a0)))
-                return;
-            a_build<D>(smem, tmem, par);
+            if (tid == kIssuer)
+                fast_issue_sq<D>(tmem, sb, kseq & 1, iset);
+            __syncwarp();
+            a_build<D>(smem, tmem, kseq & 1, iset);
             fence_proxy_async_smem();
             tc_fence_before();
             if (!sync_group(2))
                 return;
             if (tid == kIssuer) {
                 tc_fence_after();
-                fast_issue_update<D, false>(tmem, sb, par);   // D_O only: the state is discarded
+                fast_issue_update<D, false>(tmem, sb, kseq & 1, iset);   // D_O only: the state is discarded
                 tc_commit(bar_o);
             }
-            pend = true;
-            pend_par = par;
-            pend_tok = rtok;
+            __syncwarp();
+            if (kseq > 0)
+                out_epilogue<D>(tmem, outp(rtok - pend_L), tstride, pend_L, (kseq - 1) & 1);
+            drained = false;
             pend_L = L;
             rtok += L;
-            par ^= 1;
+            iset = iset == 2 ? 0 : iset + 1;
             ++kseq;
             if (!is_long(rtok))
                 break;
             // the next segment's start state, while this segment's products run and the
             // builders build it (this segment's fp16 copy is made: TMEM S is free)
-            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rtok) * p.n_heads * D * D);
+            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(rtok) * p.n_heads * D * D, next_max());
             loaded = seg_idx(rtok);
         }
-        if (pend) {
-            if (!wait_group(2, kIssuer, bar_o, ph_o))
+        if (kseq > 0) {
+            if (!drained && !wait_group(2, kIssuer, bar_o, ph_o))
                 return;
-            out_epilogue<D>(tmem, outp(pend_tok), tstride, pend_L, pend_par, false);
+            out_epilogue<D>(tmem, outp(rtok - pend_L), tstride, pend_L, (kseq - 1) & 1);
             tc_fence_before();
             if (!sync_group(2))
                 return;
@@ -612,7 +673,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     while (!aborted && tok < n) {
         if (RESTART && worker && loaded != seg_idx(tok)) {
             // this segment's own start state (the previous segment's state is not used)
-            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(tok) * p.n_heads * D * D);
+            state_load<D>(smem, tmem, st_g + (int64_t)seg_idx(tok) * p.n_heads * D * D, next_max());
             tc_fence_before();
             bar_staters();
             tc_fence_after();
@@ -652,6 +713,10 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                         sMisc[1] = 1;
                     if (tma_pending)
                         ph_tma ^= 1;
+                    if (v_pending && !mbar_wait_bounded(bar_v, ph_v, kTimeoutNs))
+                        sMisc[1] = 1;
+                    if (v_pending)
+                        ph_v ^= 1;
                     issue_tma(tok);
                 }
                 if (stop == 2)
@@ -676,7 +741,9 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             report(p.d_err, HS_DEVERR_TIMEOUT);
             if (n_tma > 0)
                 mbar_wait_bounded(bar_tma, (n_tma - 1) & 1, kTimeoutNs);
-            tc_commit(bar_ld);   // the D_A products this thread issued
+            if (n_v > 0)
+                mbar_wait_bounded(bar_v, (n_v - 1) & 1, kTimeoutNs);
+            tc_commit(bar_ld);   // the D_A products this thread issued (RESTART)
             mbar_wait_bounded(bar_ld, 0, kTimeoutNs);
         }
         if (tid == kIssuer) {
