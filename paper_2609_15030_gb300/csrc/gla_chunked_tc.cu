@@ -122,7 +122,12 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         tma_prefetch_2d(&maps.v, h * D, y);
         tma_prefetch_2d(&maps.g, h * D, y);
     }
-    pdl_wait();
+    // RESTART: only the start states come from the kernel before (the scan).  The inputs are
+    // final already: the scan's CTAs released this launch after their own wait, hence after the
+    // segment-state pass, which itself waited for whatever wrote them.  So the builders stage and
+    // build at once, and the state warps wait below, before they load a state
+    if (!RESTART)
+        pdl_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -296,6 +301,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // largest magnitude.  The builders meanwhile stage and build the first segment.
     float *st_g = p.state + ((int64_t)(RESTART ? p.ck_base[b] : b) * p.n_heads + h) * D * D;
     if (worker) {
+        if (RESTART)
+            pdl_wait();
         state_load<D>(smem, tmem, st_g, next_max());
         tc_fence_before();
         bar_staters();

@@ -77,9 +77,8 @@ gla_scan_kernel(const __grid_constant__ ScanParams p)
     const int64_t hs_ = (int64_t)h * D * D + f;        // offset inside one [n_heads][D][D] state
     const int64_t sstride = (int64_t)p.n_heads * D * D;
     const int C = p.ckpt_interval;
-    pdl_wait_and_release();
-
     float4 *st = reinterpret_cast<float4 *>(p.state + (int64_t)b * sstride + hs_);
+    pdl_wait_and_release();
     float4 S = *st;
     auto seg_end_of = [&](int64_t at) -> int64_t { return min(end, (at / kChunk + 1) * kChunk); };
     // the rings: one commit group per segment (empty past the last), kStages in flight
