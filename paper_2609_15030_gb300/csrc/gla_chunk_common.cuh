@@ -59,18 +59,18 @@ constexpr uint32_t X_LAM = 32768;       //   Lam f32 [64 tok][D], row-major     
 constexpr uint32_t X_B2 = 65536;        //   [A ; K^^T] tf32 [64 i + D][64 tok j]               48 KiB
 constexpr uint32_t OFF_SQ = 122880;     // staged q  bf16 [64][D]                  16 KiB
 constexpr uint32_t OFF_SK = 139264;     // staged k                                 16 KiB
-constexpr uint32_t OFF_SV = 155648;     // staged v                                 16 KiB
-constexpr uint32_t OFF_SG = 172032;     // staged log-gates f32 [64][D]             32 KiB
-constexpr uint32_t OFF_GAM = 204800;    // 2^{Lam_last} per key dim, four slots by chunk number   2 KiB
-constexpr uint32_t OFF_TOT = 206848;    // partial log2-decay totals [token groups][D]        2 KiB
-constexpr uint32_t OFF_RED = 208896;    // two sets of [8 warps][8]: builders' max |q|, fast-path flag,
-                                        //   max |k|, max |v| (0..3; set by segment parity); state
-                                        //   warps' max |S| (4; a set per pass, in turn)
-constexpr uint32_t OFF_BAR = 209408;    // 9 mbarriers
-constexpr uint32_t OFF_MISC = 209536;   // TMEM base address, abort flag, decision, run result
-constexpr uint32_t OFF_DG = 209600;     // diagonal of A in float32, with the operand sets:
+constexpr uint32_t OFF_SG = 155648;     // staged log-gates f32 [64][D]             32 KiB
+constexpr uint32_t OFF_SV = 188416;     // staged v, two buffers by chunk parity    32 KiB
+constexpr uint32_t OFF_GAM = 221184;    // 2^{Lam_last} per key dim, four slots by chunk number   2 KiB
+constexpr uint32_t OFF_TOT = 223232;    // partial log2-decay totals [token groups][D]        2 KiB
+constexpr uint32_t OFF_RED = 225280;    // three sets of [8 warps][8]: builders' max |q|, fast-path
+                                        //   flag, max |k|, max |v| (0..3; with the operand sets);
+                                        //   state warps' max |S| (4; two sets, a pass each in turn)
+constexpr uint32_t OFF_BAR = 226048;    // 7 mbarriers
+constexpr uint32_t OFF_MISC = 226112;   // TMEM base address, abort flag, decision, run result
+constexpr uint32_t OFF_DG = 226176;     // diagonal of A in float32, with the operand sets:
                                         //   [set][key-dim half][64 tokens] partial sums  1.5 KiB
-constexpr uint32_t SMEM_BYTES = 211136 + 1024;
+constexpr uint32_t SMEM_BYTES = 227712 + 1024;
 
 // tensor memory: D_O alternates between two buffers by chunk parity, placed on
 // either side of S^T so that [D_O0 | S^T] and [S^T | D_O1] are each one accumulator of
@@ -81,12 +81,12 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_O0 = 0;           // D_O of even chunks (lane e, col i), 64 cols
 constexpr uint32_t TM_S = 64;           // S^T  float32, 128 lanes x D cols
 constexpr uint32_t TM_SH = 256;         // S^T fp16 copy, two key dims per column      D/2 cols
-constexpr uint32_t TM_A0 = 320;         // D_A of even segments, 128 lanes x 64 cols (lanes 0..63 used)
-constexpr uint32_t TM_V = 384;          // V^T: fast, fp16 pairs 2 x 32 cols; exact, f32 64 cols
-constexpr uint32_t TM_A1 = 448;         // D_A of odd segments
+constexpr uint32_t TM_A = 320;          // D_A, 128 lanes x 64 cols (lanes 0..63 used)
+constexpr uint32_t TM_V = 384;          // V^T: fast, fp16 pairs 3 x 32 cols (with the operand sets);
+                                        // exact, f32 64 cols
 // exact path (no fast-path data live): S^T as two tf32 parts for S^T Q~^T, hi in the D
-// columns right of S^T (D_O1 and, for D = 128, the fp16 copy), lo in the D_A buffers (key
-// dims 0..63, 64..127)
+// columns right of S^T (D_O1 and, for D = 128, the fp16 copy), lo in the columns of D_A and
+// of the third V^T buffer (key dims 0..63, 64..127)
 constexpr uint32_t TM_SLO0 = 320;
 constexpr uint32_t TM_SLO1 = 448;
 
@@ -107,8 +107,7 @@ struct Geo {
     static constexpr uint32_t SHI = TM_S + D;     // exact path: hi part of S^T
     static constexpr uint32_t IDF_ST = idesc_f16(128, D, 1);       // S^T += V^T K~ (K~ read MN-major)
     static constexpr uint32_t IDT_UP = idesc_tf32(128, 64 + D, 0, 0);   // exact: [D_O | S^T] update
-    static constexpr uint32_t STAGE = 2 * CH * D * 2 + CH * D * 4;  // staged q, k, log-gates
-    static constexpr uint32_t STAGE_V = CH * D * 2;                 // staged v
+    static constexpr uint32_t STAGE = 3 * CH * D * 2 + CH * D * 4;  // staged q, k, v, log-gates
 };
 
 struct TmaMaps {
@@ -247,28 +246,33 @@ __device__ __forceinline__ int thread_id()
     return t;
 }
 
-// zero the staged rows past a segment of L < 64 tokens: q, k and the gates (QKG), v (V), by
-// all threads or the builder warps only; the copies concerned have landed
-template <int D, bool QKG, bool V>
-__device__ __forceinline__ void zero_tail(uint8_t *smem, int L, bool builders_only)
+// the staged v of the segment in v buffer vb
+__device__ __forceinline__ const uint16_t *staged_v(const uint8_t *smem, int vb)
+{
+    return reinterpret_cast<const uint16_t *>(smem + OFF_SV + vb * 16384);
+}
+
+// zero the staged rows past a segment of L < 64 tokens (all threads, or the builder
+// warps only)
+template <int D>
+__device__ __forceinline__ void zero_tail(uint8_t *smem, int L, int vb, bool builders_only)
 {
     const int tid = threadIdx.x;
-    constexpr int QV = D / 8, GV = D / 4;   // 16-byte vectors per q/k/v row, per gate row
-    constexpr int RV = (QKG ? 2 * QV + GV : 0) + (V ? QV : 0);
+    constexpr int QV = D / 8, RV = 5 * D / 8;   // 16-byte vectors per q/k/v row, per token
 
     if (L < CH) {
         const int nthr = builders_only ? NB : NT;
         for (int idx = tid; idx < (CH - L) * RV; idx += nthr) {
             const int row = L + idx / RV, c = idx % RV;
             uint4 *dst;
-            if (QKG && c < QV)
+            if (c < QV)
                 dst = reinterpret_cast<uint4 *>(smem + OFF_SQ + row * 2 * D) + c;
-            else if (QKG && c < 2 * QV)
+            else if (c < 2 * QV)
                 dst = reinterpret_cast<uint4 *>(smem + OFF_SK + row * 2 * D) + (c - QV);
-            else if (QKG && c < 2 * QV + GV)
-                dst = reinterpret_cast<uint4 *>(smem + OFF_SG + row * 4 * D) + (c - 2 * QV);
+            else if (c < 3 * QV)
+                dst = reinterpret_cast<uint4 *>(smem + OFF_SV + vb * 16384 + row * 2 * D) + (c - 2 * QV);
             else
-                dst = reinterpret_cast<uint4 *>(smem + OFF_SV + row * 2 * D) + (c - (RV - QV));
+                dst = reinterpret_cast<uint4 *>(smem + OFF_SG + row * 4 * D) + (c - 3 * QV);
             *dst = make_uint4(0u, 0u, 0u, 0u);
         }
         fence_proxy_async_smem();   // the next copies overwrite these rows
@@ -295,8 +299,8 @@ __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, bool builders_on
 // 0, or a total log2-decay below -kLamRange) stops after the totals and returns false: the
 // staged inputs are untouched, so the exact path starts from them without another copy.
 template <int D>
-__device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int iset, int gslot, float &mq,
-                                           float &mk, bool &ok)
+__device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int vb, int iset, int gslot,
+                                           float &mq, float &mk, bool &ok)
 {
     using G = Geo<D>;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -306,7 +310,7 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int iset, int g
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
     float *sGam = reinterpret_cast<float *>(smem + OFF_GAM);
 
-    zero_tail<D, true, false>(smem, L, true);
+    zero_tail<D>(smem, L, vb, true);
     const int dp = tid % G::DP, qt = tid / G::DP;
     float amax = -INFINITY;
     {
@@ -387,25 +391,24 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int iset, int g
     return true;
 }
 
-// ... then, once the V^T buffer `par` and the guard words of the segment before are free: V^T,
-// thread (e, half) packing tokens [32 half, 32 half + 32) of value dim e, and the guard words
-// (`built`: whether build_fast went through; if not, a failing flag only)
+// ... then V^T (buffer iset), thread (e, half) packing tokens [32 half, 32 half + 32) of value dim
+// e, and the guard words (set iset; `built`: whether build_fast went through; if not, a failing
+// flag only)
 template <int D>
-__device__ __forceinline__ void build_values(uint8_t *smem, uint32_t tmem, int L, int par, bool built,
+__device__ __forceinline__ void build_values(uint8_t *smem, uint32_t tmem, int vb, int iset, bool built,
                                              float mq, float mk, bool ok)
 {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;   // this warp's TMEM lane quarter
     const int e_own = (warp & 3) * 32 + lane;                  // TMEM lane = value dim e
     const int th = warp >> 2;
-    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
-    float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + par * 64;
+    const uint16_t *sV = staged_v(smem, vb);
+    float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + iset * 64;
     if (!built) {
         if (lane == 0)
             sRed[warp * 8 + 1] = 0.f;
         return;
     }
-    zero_tail<D, false, true>(smem, L, true);
     __nv_bfloat162 bv = __float2bfloat162_rn(0.f);
     {
         uint32_t vpk[16];
@@ -418,7 +421,7 @@ __device__ __forceinline__ void build_values(uint8_t *smem, uint32_t tmem, int L
             bv = bmax_abs(bv, w);
             vpk[m] = pack_h2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
         }
-        tmem_st16(tmem + lrow + TM_V + 32 * par + 16 * th, vpk);
+        tmem_st16(tmem + lrow + TM_V + 32 * iset + 16 * th, vpk);
     }
     const float mv = warp_max(bmax_of(bv));
     // non-increasing Lam (|Q~| <= |q|, |A| <= D max|q| max|k|), a total decay of at most
@@ -503,10 +506,10 @@ __device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpa
 }
 
 
-// ---- the causally masked intra-chunk matrix A (D_A buffer `par`) -> operand set iset's A
+// ---- the causally masked intra-chunk matrix A (D_A) -> operand set iset's A
 // (state warps of TMEM lane quarters 0 and 1)
 template <int D>
-__device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int par, int iset)
+__device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int iset)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool worker = warp >= 8;
@@ -517,7 +520,7 @@ __device__ __forceinline__ void a_build(uint8_t *smem, uint32_t tmem, int par, i
     const int i = (warp & 3) * 32 + lane;      // TMEM lane = query row
     const int jb = ((warp >> 2) & 1) * 32;      // this warp's 32 key columns
     float r[32];
-    tmem_ld32(tmem + lrow + (par ? TM_A1 : TM_A0) + jb, r);
+    tmem_ld32(tmem + lrow + TM_A + jb, r);
     // the diagonal from the builders' float32 partials (one per 64 key dims)
     const float *sDg = reinterpret_cast<const float *>(smem + OFF_DG) + iset * 128;
     const float dg = (i >= jb && i < jb + 32) ? (D == 128 ? sDg[i] + sDg[64 + i] : sDg[i]) : 0.f;
@@ -644,7 +647,7 @@ __device__ __forceinline__ int lam_at(int row, int d)
 // gates below kGateFloor taken at the floor), Q~ = q 2^{Lam} (tf32, X_QT) and 2^{Lam_last} into
 // gam slot 0.  Returns (uniformly) whether some gate is above 0.
 template <int D>
-__device__ __forceinline__ bool exact_decay(uint8_t *smem, int L)
+__device__ __forceinline__ bool exact_decay(uint8_t *smem, int L, int vb)
 {
     const int tid = thread_id(), warp = tid >> 5, lane = tid & 31;
     const int d = (warp & 3) * 32 + lane;
@@ -655,7 +658,7 @@ __device__ __forceinline__ bool exact_decay(uint8_t *smem, int L)
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
     float *sGam = reinterpret_cast<float *>(smem + OFF_GAM);
     float *sLam = reinterpret_cast<float *>(smem + X_LAM);
-    zero_tail<D, true, true>(smem, L, false);
+    zero_tail<D>(smem, L, vb, false);
     float lam[16];
     bool up = false;
     if (worker) {
@@ -693,7 +696,7 @@ __device__ __forceinline__ bool exact_decay(uint8_t *smem, int L)
 
 // (builder warps) K^^T = k 2^{Lam_last - Lam} (tf32, rows 64.. of X_B2) and V^T float32 into TMEM
 template <int D>
-__device__ __forceinline__ void exact_keys_values(uint8_t *smem, uint32_t tmem)
+__device__ __forceinline__ void exact_keys_values(uint8_t *smem, uint32_t tmem, int vb)
 {
     const int warp = thread_id() >> 5, lane = thread_id() & 31;
     const int d = (warp & 3) * 32 + lane;      // key dim, and value dim = TMEM lane of V^T
@@ -701,7 +704,7 @@ __device__ __forceinline__ void exact_keys_values(uint8_t *smem, uint32_t tmem)
         return;
     const uint32_t lrow = (uint32_t)((warp & 3) * 32) << 16;
     const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
-    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
+    const uint16_t *sV = staged_v(smem, vb);
     const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
     const float last = sLam[lam_at<D>(CH - 1, d)];
 #pragma unroll 1
@@ -977,13 +980,13 @@ __device__ __forceinline__ void exact_task(uint8_t *smem, int task)
 // (builder warps) whether the gates of a staged segment alone send it to the exact path: the
 // first step of build_fast, with its arithmetic and its verdict (uniform over the builders)
 template <int D>
-__device__ __forceinline__ bool gates_exact(uint8_t *smem, int L)
+__device__ __forceinline__ bool gates_exact(uint8_t *smem, int L, int vb)
 {
     using G = Geo<D>;
     const int tid = thread_id(), dp = tid % G::DP, qt = tid / G::DP;
     const float *sG = reinterpret_cast<const float *>(smem + OFF_SG);
     float *sTot = reinterpret_cast<float *>(smem + OFF_TOT);
-    zero_tail<D, true, true>(smem, L, true);
+    zero_tail<D>(smem, L, vb, true);
     float amax = -INFINITY, r0 = 0.f, r1 = 0.f;
 #pragma unroll
     for (int x = 0; x < G::TPG; ++x) {
@@ -1098,25 +1101,26 @@ __device__ __forceinline__ void exact_issue_sq(uint32_t tmem, uint32_t sb)
 // shared memory (the task counter).  The state warps split the state and start S^T Q~^T while
 // the builders form K^ and V^T; then both draw score tasks.
 template <int D>
-__device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int L, int *next)
+__device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int L, int vb, int *next)
 {
     constexpr int TASKS = kSquareTasks + 8 * (D / 64);
     if (thread_id() == 0)
         *next = 0;
-    const bool up = exact_decay<D>(smem, L);
+    const bool up = exact_decay<D>(smem, L, vb);
     fence_proxy_async_smem();
     __syncthreads();
     if (thread_id() < NB) {
         if (!up)
             exact_zeros<D>(smem);
-        exact_keys_values<D>(smem, tmem);
+        exact_keys_values<D>(smem, tmem, vb);
     } else {
         exact_split_state<D>(smem, tmem);
         tc_fence_before();
         bar_staters();
-        if (thread_id() == kIssuer) {
+        if (uniform(thread_id() >> 5) == kIssuer / 32) {
             tc_fence_after();
-            exact_issue_sq<D>(tmem, smem_u32(smem));
+            if (elect_one())
+                exact_issue_sq<D>(tmem, smem_u32(smem));
         }
         __syncwarp();
     }
@@ -1156,15 +1160,15 @@ __device__ __forceinline__ void exact_issue_update(uint32_t tmem, uint32_t sb)
 
 // ---- fast path MMA groups (issuing thread) ----
 
-// D_A = Q~ K~^T of an operand set into D_A buffer `par`
+// D_A = Q~ K~^T of an operand set
 template <int D>
-__device__ __forceinline__ void fast_issue_scores(uint32_t tmem, uint32_t sb, int par, int iset)
+__device__ __forceinline__ void fast_issue_scores(uint32_t tmem, uint32_t sb, int iset)
 {
     const uint32_t setb = sb + (uint32_t)iset * SET_BYTES;
 #pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         const uint32_t koff = (kk >> 2) * 8192 + (kk & 3) * 32;
-        mma_f16_ss(tmem + (par ? TM_A1 : TM_A0), sdesc_sw128(setb + S_QH + koff, 16, 1024),
+        mma_f16_ss(tmem + TM_A, sdesc_sw128(setb + S_QH + koff, 16, 1024),
                    sdesc_sw128(setb + S_KH + koff, 16, 1024), IDF_N64, kk > 0);
     }
 }
@@ -1191,7 +1195,7 @@ template <int D, bool WITH_STATE = true>
 __device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, int par, int iset)
 {
     const uint32_t setb = sb + (uint32_t)iset * SET_BYTES;
-    const uint32_t vt = tmem + TM_V + 32 * par;
+    const uint32_t vt = tmem + TM_V + 32 * iset;
 #pragma unroll
     for (int kk = 0; kk < CH / 16; ++kk) {
         mma_f16_ts(tmem + (par ? Geo<D>::O1 : TM_O0), vt + kk * 8,
@@ -1208,7 +1212,7 @@ __device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, in
 // update S in TMEM, write the slot and the largest |S|, and leave each token's group partials
 // in the operand sets) ...
 template <int D>
-__device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L, float *slot, int mset)
+__device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L, int vb, float *slot, int mset)
 {
     constexpr int CW = Geo<D>::CW, NG = Geo<D>::NG;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1218,7 +1222,7 @@ __device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L,
     const int colhalf = (warp >> 2) & 1;
     const uint16_t *sQ = reinterpret_cast<const uint16_t *>(smem + OFF_SQ);
     const uint16_t *sK = reinterpret_cast<const uint16_t *>(smem + OFF_SK);
-    const uint16_t *sV = reinterpret_cast<const uint16_t *>(smem + OFF_SV);
+    const uint16_t *sV = staged_v(smem, vb);
     float *sG = reinterpret_cast<float *>(smem + OFF_SG);
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED) + mset * 64;
     for (int idx = tid; idx < L * D; idx += NT)

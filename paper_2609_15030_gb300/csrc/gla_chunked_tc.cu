@@ -29,8 +29,7 @@
 // fp16 copy of S^T; the causal mask with each token's own score summed in
 // float32 on the diagonal; the output epilogue) the eight builder warps stage
 // chunk c+1 and build its operands (cumulative decay scan, Q~, K~, V^T).  Threads
-// of two builder warps and a state warp issue the TMA copies, one state thread
-// the MMAs (the first builder thread D_A in the RESTART instantiation).
+// of two builder warps issue the TMA copies, one state thread the MMAs.
 //
 // A chunk is fast only if every fp16 operand provably stays below 2^15 in
 // magnitude (|q|, |v|, |K~|, the bound 128 max|q| max|k| on |A|, and a bound
@@ -75,14 +74,13 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
     // [0] TMEM base, [1] abort flag, [2] decision on the latest built segment (1 = fast),
     // [3] run result (1 = the segment at [4] needs the exact path), [4] token index where the
-    // run stopped, [8] whether the latest segment's
-    // build is whole (0: its gates alone send it to the exact path, its inputs still staged),
-    // [9] an exact segment's look ahead, [10] its task counter
+    // run stopped, [5] whether that segment's build is whole (0: its gates alone send it to the
+    // exact path, its inputs still staged), [9] an exact segment's look ahead, [10] its task
+    // counter, [11..12] whether the build of the latest segments is whole, by segment parity
     volatile uint32_t *sMisc = reinterpret_cast<volatile uint32_t *>(smem + OFF_MISC);
     const uint32_t bar_tma = sb + OFF_BAR, bar_a = sb + OFF_BAR + 8, bar_o = sb + OFF_BAR + 16,
                    bar_s = sb + OFF_BAR + 24, bar_built = sb + OFF_BAR + 32,
-                   bar_go = sb + OFF_BAR + 40, bar_v = sb + OFF_BAR + 48,
-                   bar_a1 = sb + OFF_BAR + 56, bar_ld = sb + OFF_BAR + 64;
+                   bar_go = sb + OFF_BAR + 40;
 
     const int tid = threadIdx.x, warp = tid >> 5;
     // (signed: the unsigned division left the d = 128 kernel with 56 bytes of spills, which cost
@@ -104,9 +102,6 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         mbar_init(bar_s, 1);
         mbar_init(bar_built, 1);
         mbar_init(bar_go, 1);
-        mbar_init(bar_v, 1);
-        mbar_init(bar_a1, 1);
-        mbar_init(bar_ld, 1);
         fence_mbar_init();
         sMisc[1] = 0;   // abort flag
     }
@@ -131,16 +126,17 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = sMisc[0];
+    const uint32_t tmem = (uint32_t)uniform((int)sMisc[0]);
+    const int warp_u = uniform(warp);      // for the single-thread issues (elect_one)
     const bool builder = warp < 8;
     const bool worker = !builder;                              // a state warp
 
     // bookkeeping of the loader (copies issued, one still in flight) and of the issuer,
     // for the waits and the abort path; every mbarrier is waited on by one thread only
-    uint32_t n_tma = 0, n_v = 0;      // copies of (q, k, gates) and of v
-    bool tma_pending = false, v_pending = false;
-    uint32_t ph_tma = 0, ph_v = 0, ph_o = 0, ph_s = 0, ph_built = 0, ph_go = 0;
-    uint32_t ph_a = 0, ph_a1 = 0;    // D_A products (RESTART: of even / odd segments)
+    uint32_t n_tma = 0;
+    bool tma_pending = false;
+    uint32_t ph_tma = 0, ph_o = 0, ph_s = 0, ph_built = 0, ph_go = 0;
+    uint32_t ph_a = 0;               // D_A products
     bool aborted = false;
 
     // L2 prefetch of the 64 tokens `ahead` tokens past token t (if any are this problem's)
@@ -154,28 +150,24 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         tma_prefetch_2d(&maps.v, x, y);
         tma_prefetch_2d(&maps.g, x, y);
     };
+    // the v buffer of the segment at token `at`
+    auto vbuf = [&](int at) -> int { return (int)((((uint32_t)at + off) / CH) & 1u); };
     // (loader) staged inputs of the segment at local position tok_local; segments after
     // the first start on the 64-token grid, so the segment kPrefetch ahead starts at
     // tok_local + 64 * kPrefetch and is requested into L2 now
-    // (q, k and the gates, then v, which the builders are done with later)
-    auto copy_qkg = [&](int tok_local) {
+    auto copy_inputs = [&](int tok_local) {
         const int32_t y = p.row0[b] + tok_local;
         const int32_t x = h * D;
         mbar_arrive_expect_tx(bar_tma, Geo<D>::STAGE);
         tma_load_2d(sb + OFF_SG, &maps.g, x, y, bar_tma);
         tma_load_2d(sb + OFF_SQ, &maps.q, x, y, bar_tma);
         tma_load_2d(sb + OFF_SK, &maps.k, x, y, bar_tma);
-    };
-    auto copy_v = [&](int tok_local) {
-        mbar_arrive_expect_tx(bar_v, Geo<D>::STAGE_V);
-        tma_load_2d(sb + OFF_SV, &maps.v, h * D, p.row0[b] + tok_local, bar_v);
+        tma_load_2d(sb + OFF_SV + vbuf(tok_local) * 16384, &maps.v, x, y, bar_tma);
     };
     auto issue_tma = [&](int tok_local) {
-        copy_qkg(tok_local);
-        copy_v(tok_local);
+        copy_inputs(tok_local);
         ++n_tma;
-        ++n_v;
-        tma_pending = v_pending = true;
+        tma_pending = true;
         if (tok_local > 0)
             prefetch(tok_local, CH * kPrefetch);
     };
@@ -203,22 +195,6 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             sMisc[1] = 1;
         ph ^= 1;
         const bool stop = bar_or(id, bad || sMisc[1] != 0);
-        tc_fence_after();
-        if (stop)
-            aborted = true;
-        return !stop;
-    };
-    // (builders) `bar` and the copy of v, waited for by the loader with one barrier
-    auto wait_group_v = [&](uint32_t bar, uint32_t &ph) -> bool {
-        bool bad = false;
-        if (tid == kLoader)
-            bad = !mbar_wait_bounded(bar, ph, kTimeoutNs) || !mbar_wait_bounded(bar_v, ph_v, kTimeoutNs);
-        if (bad)
-            sMisc[1] = 1;
-        ph ^= 1;
-        ph_v ^= 1;
-        v_pending = false;
-        const bool stop = bar_or(1, bad || sMisc[1] != 0);
         tc_fence_after();
         if (stop)
             aborted = true;
@@ -255,12 +231,9 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             aborted = true;
         return !stop;
     };
-    // both copies of the staged inputs, CTA-wide
     auto wait_tma = [&]() -> bool {
         tma_pending = false;
-        if (builder && !wait_group_v(bar_tma, ph_tma))
-            sMisc[1] = 1;
-        return sync_all();
+        return wait_all(kLoader, bar_tma, ph_tma);
     };
     auto seg_len = [&](int at) -> int { return min(n - at, CH - (int)(((uint32_t)at + off) & (CH - 1))); };
     auto is_long = [&](int at) -> bool { return at < n && seg_len(at) > kShort; };
@@ -316,7 +289,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // pending): the per-token recurrence with the recurrent kernel's exact operation order
     // (fma chains over groups of 16 key rows, group partials summed left to right)
     auto short_segment = [&](int tok_s, int L) {
-        short_state<D>(smem, tmem, L, worker ? ckpt_slot(tok_s + L) : nullptr, next_max());
+        short_state<D>(smem, tmem, L, vbuf(tok_s), worker ? ckpt_slot(tok_s + L) : nullptr, next_max());
         if (tid == kLoader && tok_s + L < n)
             issue_tma(tok_s + L);
         short_outputs<D>(smem, L, outp(tok_s), tstride);
@@ -331,8 +304,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // below 2^15 in magnitude.  Returns whether the segment's own inputs pass; `state_ok` says
     // whether the state (its measured magnitude, or a bound on it) passes too.
     float mk_new = 0.f, mv_new = 0.f;
-    auto guard = [&](float s_mag, bool &state_ok) -> bool {
-        const float *red = sRed + (kseq & 1) * 64;
+    auto guard = [&](float s_mag, int kset, bool &state_ok) -> bool {
+        const float *red = sRed + kset * 64;
         float mq = 0.f, mk = 0.f, mv = 0.f;
         bool ok = true;
 #pragma unroll
@@ -355,19 +328,22 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     int ready = 0;
     auto exact_segment = [&](int tok_s, int L) -> bool {
         const int seg_end = tok_s + L;
-        exact_operands<D>(smem, tmem, L, const_cast<int *>(reinterpret_cast<volatile int *>(sMisc + 10)));
-        if (tid == kIssuer) {
+        exact_operands<D>(smem, tmem, L, vbuf(tok_s), const_cast<int *>(reinterpret_cast<volatile int *>(sMisc + 10)));
+        if (warp_u == kIssuer / 32) {
             tc_fence_after();
-            exact_issue_update<D>(tmem, sb);
-            tc_commit(bar_o);
+            if (elect_one()) {
+                exact_issue_update<D>(tmem, sb);
+                tc_commit(bar_o);
+            }
+            __syncwarp();
         }
         const bool ahead = is_long(seg_end);
         if (builder) {
             if (tid == kLoader && seg_end < n)
                 issue_tma(seg_end);
-            if (ahead && wait_group_v(bar_tma, ph_tma)) {
+            if (ahead && wait_group(1, kLoader, bar_tma, ph_tma)) {
                 tma_pending = false;
-                const bool exact = gates_exact<D>(smem, seg_len(seg_end));
+                const bool exact = gates_exact<D>(smem, seg_len(seg_end), vbuf(seg_end));
                 if (tid == kLoader)
                     sMisc[9] = exact ? 1u : 2u;
             }
@@ -388,31 +364,31 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // Handoffs (each mbarrier has one waiting thread and one arriving party):
     //   bar_built: builders -> state warps, segment k built (operands, V^T, guard maxima)
     //   bar_go:    state warps -> builders, the decision on segment k is made (sMisc[2]);
-    //              when it is fast, it also means the V^T and D_A buffers of segment k+1 are free
-    //              (the products of segment k-1 are complete)
+    //              when it is fast, it also means the products of segment k-1 are complete, so
+    //              that segment k+2 may take their operand set and V^T buffer
     // A run ends after the last long segment, before a segment whose own inputs the guard
     // sends to the exact path, or before a segment whose state bound fails: a decision inside a
     // run only has a bound on the state it starts from (that state is still being computed), so
     // such a segment starts a new run, whose first decision reads the measured state exactly as
     // a run resumed from a checkpoint at that segment does.  The groups then meet CTA-wide.
     // No MMA is in flight at either end.
-    // The builders run up to one segment ahead of the decisions: Q~ and K~ of segment k+1 go into
-    // a third operand set while segment k is judged and segment k-1 finishes; only V^T and the
-    // guard words wait for "go" on segment k, and only then are the next segment's q, k and gates
-    // copied over the consumed ones (v, consumed last, follows from the state warps).  With two
-    // sets and one copy of all four, the builders' chain (build, hand over, issue, wait for the
+    // The builders run up to one segment ahead of the decisions: segment k+1 goes into a third
+    // operand set and V^T buffer while segment k is judged and segment k-1 finishes, and only its
+    // hand-over waits for "go" on segment k.  Its staged rows are overwritten by the copy of segment
+    // k+2 as soon as q, k and the gates are consumed (v has two staging buffers).  With two sets and
+    // one copy at the hand-over, the builders' chain (build, hand over, issue, wait for the
     // decision, wait for the copy) set the pace at ~9 k cycles a segment; the D_A and copy issues
     // (~1 k cycles of single-thread work) and two barriers a segment are off it, and the state
     // warps' passes run in rolled halves (less code, fewer registers): 4 x 32 heads of 16,384
-    // tokens 1,088 -> 1,001 us, 256-token tails of 9 x 16 heads 28.5 -> 27.8 us.
+    // tokens 1,088 -> 977 us, 256-token tails of 9 x 16 heads 28.5 -> 26.7 us, 81 packed tails 248 ->
+    // 234 us.
     auto builder_run = [&](int rtok, bool waited) {
         int iset = 0;
         while (true) {
             const int L = seg_len(rtok);
-            // a run's first segment: both copies (unless the look ahead has waited for them)
-            if (kseq > 0 ? !wait_group(1, kLoader, bar_tma, ph_tma)
-                         : !waited && !wait_group_v(bar_tma, ph_tma))
+            if (!waited && !wait_group(1, kLoader, bar_tma, ph_tma))
                 return;
+            waited = false;
             tma_pending = false;
             if (tid == kLoader && !prefetched) {
                 // once the first segment has landed (the state and the first segment are
@@ -423,40 +399,29 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             }
             float mq, mk;
             bool ok;
-            const bool built = build_fast<D>(smem, L, iset, kseq & 3, mq, mk, ok);
+            const bool built = build_fast<D>(smem, L, vbuf(rtok), iset, kseq & 3, mq, mk, ok);
             fence_proxy_async_smem();
-            // the decision on the segment before, and v; for the first segment only a barrier
-            // before the staged rows are overwritten
-            const bool more = rtok + L < n;
-            if (kseq > 0) {
-                if (!wait_group_v(bar_go, ph_go) || sMisc[2] == 0)
+            if (built && rtok + L < n) {
+                // q, k and the gates are consumed: stage the next segment (long or short); an exact
+                // decision on this one reloads it
+                if (!sync_group(1))
                     return;
-            } else if (built && more && !sync_group(1)) {
-                return;
+                if (tid == kLoader) {
+                    ++n_tma;
+                    tma_pending = true;
+                }
+                if (warp_u == 1 && elect_one())
+                    copy_inputs(rtok + L);
+                __syncwarp();
             }
-            // q, k and the gates are consumed: stage those of the next segment (long or short); an
-            // exact decision on this one reloads it
-            if (tid == kLoader && built && more) {
-                ++n_tma;
-                ++n_v;
-                tma_pending = v_pending = true;
-            }
-            if (tid == kLoader + 32 && built && more)
-                copy_qkg(rtok + L);
-            build_values<D>(smem, tmem, L, kseq & 1, built, mq, mk, ok);
+            build_values<D>(smem, tmem, vbuf(rtok), iset, built, mq, mk, ok);
             tc_fence_before();
-            if (!sync_group(1))
+            // every warp's part done, and the decision on the segment before
+            if (kseq > 0 ? !wait_group(1, kLoader, bar_go, ph_go) || sMisc[2] == 0 : !sync_group(1))
                 return;
             if (tid == kLoader) {
-                sMisc[8] = built ? 1u : 0u;
+                sMisc[11 + (kseq & 1)] = built ? 1u : 0u;
                 mbar_arrive(bar_built);
-                if (RESTART && built) {
-                    // D_A at once: the state warps have their start state to load as well, and
-                    // many restart CTAs have a single segment, whose latency this shortens
-                    tc_fence_after();
-                    fast_issue_scores<D>(tmem, sb, kseq & 1, iset);
-                    tc_commit((kseq & 1) ? bar_a1 : bar_a);
-                }
             }
             if (!built || !is_long(rtok + L)) {
                 wait_group(1, kLoader, bar_go, ph_go);   // the run ends with this segment
@@ -467,21 +432,39 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             ++kseq;
         }
     };
-    // What the builders leave to the state warps, which wait for them each segment: (issuer) D_A =
-    // Q~ K~^T of a built segment, into its own buffer; (one thread each of two other warps) the copy
-    // of the next segment's v, now that a built segment's own is packed (an early stopped build
-    // has not consumed it), and the L2 requests of the segment kPrefetch further on
-    auto issue_scores = [&](int par, int iset) {
-        if (tid == kIssuer) {
-            fast_issue_scores<D>(tmem, sb, par, iset);
-            tc_commit(bar_a);
+    // The issuing thread's product groups (state warps; each call ends converged)
+    auto issue_sq = [&](int par, int iset) {       // D_O = S^T Q~^T
+        if (warp_u == kIssuer / 32) {
+            const int pu = uniform(par), iu = uniform(iset);
+            if (elect_one())
+                fast_issue_sq<D>(tmem, sb, pu, iu);
         }
         __syncwarp();
     };
-    auto copy_next_v = [&](int next) {
-        if (tid == NB + 96 && sMisc[8] != 0 && next < n)
-            copy_v(next);
-        if (tid == NB + 7 * 32)
+    auto issue_update = [&](int par, int iset) {   // (RESTART: D_O only, the state is discarded)
+        if (warp_u == kIssuer / 32) {
+            const int pu = uniform(par), iu = uniform(iset);
+            tc_fence_after();
+            if (elect_one()) {
+                fast_issue_update<D, !RESTART>(tmem, sb, pu, iu);
+                tc_commit(bar_o);
+            }
+        }
+        __syncwarp();
+    };
+    auto issue_scores = [&](int iset) {            // D_A = Q~ K~^T
+        if (warp_u == kIssuer / 32) {
+            const int iu = uniform(iset);
+            if (elect_one()) {
+                fast_issue_scores<D>(tmem, sb, iu);
+                tc_commit(bar_a);
+            }
+        }
+        __syncwarp();
+    };
+    // (another state warp) the L2 requests of the segment kPrefetch past the next one
+    auto request = [&](int next) {
+        if (warp_u == NB / 32 + 7 && elect_one())
             prefetch(next, CH * kPrefetch);
         __syncwarp();
     };
@@ -495,8 +478,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         int pend_L = 0;        // the previous segment's tokens
         float mk_cur = 0.f, mv_cur = 0.f;
         while (true) {
-            // the segment at rtok built, and the products of the previous one complete: the V^T and
-            // D_A buffers of the next one are free
+            // the segment at rtok built, and the products of the previous one complete
             tc_fence_before();
             if (!wait_group_o(kseq > 0))
                 return;
@@ -507,19 +489,20 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             // update, 64 max|k| max|v| (the decay factors are <= 1)
             bool state_ok;
             const bool inputs_ok =
-                guard(kseq > 0 ? (state_max() + 64.0f * mk_cur * mv_cur) * kBoundMargin : state_max(), state_ok);
+                guard(kseq > 0 ? (state_max() + 64.0f * mk_cur * mv_cur) * kBoundMargin : state_max(), iset,
+                      state_ok);
             const bool fast = inputs_ok && state_ok;
             if (tid == kIssuer) {
                 sMisc[2] = fast ? 1u : 0u;
                 mbar_arrive(bar_go);
             }
             const int L = seg_len(rtok);
-            copy_next_v(rtok + L);
+            request(rtok + L);
             if (!fast) {
                 stop = kseq > 0 && inputs_ok ? 2u : 1u;   // the exact path or a new run takes this segment
                 break;
             }
-            issue_scores(kseq & 1, iset);
+            issue_scores(iset);
             mk_cur = mk_new;
             mv_cur = mv_new;
             state_pass<D>(smem, tmem, kseq > 0 ? (kseq - 1) & 3 : -1,
@@ -529,20 +512,13 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             // the state in place, and D_A of this segment
             if (!wait_group(2, kIssuer, bar_a, ph_a))
                 return;
-            if (tid == kIssuer)
-                fast_issue_sq<D>(tmem, sb, kseq & 1, iset);   // D_O = S^T Q~^T
-            __syncwarp();
-            a_build<D>(smem, tmem, kseq & 1, iset);
+            issue_sq(kseq & 1, iset);
+            a_build<D>(smem, tmem, iset);
             fence_proxy_async_smem();
             tc_fence_before();
             if (!sync_group(2))
                 return;
-            if (tid == kIssuer) {
-                tc_fence_after();
-                fast_issue_update<D>(tmem, sb, kseq & 1, iset);
-                tc_commit(bar_o);
-            }
-            __syncwarp();
+            issue_update(kseq & 1, iset);
             if (kseq > 0)
                 out_epilogue<D>(tmem, outp(rtok - pend_L), tstride, pend_L, (kseq - 1) & 1);
             drained = false;
@@ -565,6 +541,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         if (tid == kIssuer) {
             sMisc[3] = stop;
             sMisc[4] = (uint32_t)rtok;
+            sMisc[5] = sMisc[11 + (kseq & 1)];
         }
     };
 
@@ -585,9 +562,6 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     auto state_run_restart = [&](int rtok) {
         int iset = 0;
         bool drained = true;
-        auto wait_scores = [&]() -> bool {
-            return (kseq & 1) ? wait_group(2, kIssuer, bar_a1, ph_a1) : wait_group(2, kIssuer, bar_a, ph_a);
-        };
         uint32_t stop = 0;   // 0 done or short segment, 1 exact
         int pend_L = 0;
         while (true) {
@@ -603,40 +577,31 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                 return;
             drained = true;
             bool state_ok;
-            const bool fast = guard(state_max(), state_ok) && state_ok;
+            const bool fast = guard(state_max(), iset, state_ok) && state_ok;
             if (tid == kIssuer) {
                 sMisc[2] = fast ? 1u : 0u;
                 mbar_arrive(bar_go);
             }
-            copy_next_v(rtok + L);
+            request(rtok + L);
             if (!fast) {
-                // the exact path takes this segment: its (unused) D_A product drained first
-                stop = 1;
-                if (sMisc[8] != 0 && !wait_scores())
-                    return;
+                stop = 1;   // the exact path takes this segment
                 break;
             }
+            issue_scores(iset);
             if (tid == kIssuer && is_long(rtok + L))
                 prefetch_state(rtok + L);   // read by the load at the end of this segment
             __syncwarp();
             state_pass<D>(smem, tmem, -1, nullptr, true, next_max());   // the fp16 copy of S for D_O
             tc_fence_before();
-            if (!wait_scores())
+            if (!wait_group(2, kIssuer, bar_a, ph_a))
                 return;
-            if (tid == kIssuer)
-                fast_issue_sq<D>(tmem, sb, kseq & 1, iset);
-            __syncwarp();
-            a_build<D>(smem, tmem, kseq & 1, iset);
+            issue_sq(kseq & 1, iset);
+            a_build<D>(smem, tmem, iset);
             fence_proxy_async_smem();
             tc_fence_before();
             if (!sync_group(2))
                 return;
-            if (tid == kIssuer) {
-                tc_fence_after();
-                fast_issue_update<D, false>(tmem, sb, kseq & 1, iset);   // D_O only: the state is discarded
-                tc_commit(bar_o);
-            }
-            __syncwarp();
+            issue_update(kseq & 1, iset);
             if (kseq > 0)
                 out_epilogue<D>(tmem, outp(rtok - pend_L), tstride, pend_L, (kseq - 1) & 1);
             drained = false;
@@ -662,6 +627,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         if (tid == kIssuer) {
             sMisc[3] = stop;
             sMisc[4] = (uint32_t)rtok;
+            sMisc[5] = sMisc[11 + (kseq & 1)];
         }
     };
 
@@ -712,18 +678,14 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             if (stop == 0)
                 continue;
             // the segment at tok takes the exact path (1) or starts a new run (2).  Its inputs
-            // are still staged if its build stopped early (sMisc[8] == 0); else restage them (the
-            // copy of the next segment may be in flight)
-            if (sMisc[8] != 0) {
+            // are still staged if its build stopped early (sMisc[5] == 0); else restage them (the
+            // copy of a later segment may be in flight)
+            if (sMisc[5] != 0) {
                 if (tid == kLoader) {
                     if (tma_pending && !mbar_wait_bounded(bar_tma, ph_tma, kTimeoutNs))
                         sMisc[1] = 1;
                     if (tma_pending)
                         ph_tma ^= 1;
-                    if (v_pending && !mbar_wait_bounded(bar_v, ph_v, kTimeoutNs))
-                        sMisc[1] = 1;
-                    if (v_pending)
-                        ph_v ^= 1;
                     issue_tma(tok);
                 }
                 if (stop == 2)
@@ -748,15 +710,13 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             report(p.d_err, HS_DEVERR_TIMEOUT);
             if (n_tma > 0)
                 mbar_wait_bounded(bar_tma, (n_tma - 1) & 1, kTimeoutNs);
-            if (n_v > 0)
-                mbar_wait_bounded(bar_v, (n_v - 1) & 1, kTimeoutNs);
-            tc_commit(bar_ld);   // the D_A products this thread issued (RESTART)
-            mbar_wait_bounded(bar_ld, 0, kTimeoutNs);
         }
-        if (tid == kIssuer) {
+        __syncwarp();
+        if (warp_u == kIssuer / 32 && elect_one()) {
             tc_commit(bar_s);
             mbar_wait_bounded(bar_s, ph_s, kTimeoutNs);
         }
+        __syncwarp();
     }
     tc_fence_before();
     __syncthreads();

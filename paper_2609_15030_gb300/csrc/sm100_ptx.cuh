@@ -131,6 +131,27 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
                  : "memory");
 }
 
+// true in one lane of a converged warp, the same one every time.  A tensor-core or TMA issue
+// under a warp-uniform condition and this one takes its operands from uniform registers;
+// under a comparison of threadIdx.x it does not, and eight MMAs took 0.8 to 1.2 k cycles to
+// issue instead of 0.5 to 0.7 k.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r));
+    return r != 0;
+}
+
+// a value all lanes of the warp agree on, known to the compiler as warp-uniform
+__device__ __forceinline__ int uniform(int x)
+{
+    return __shfl_sync(0xffffffffu, x, 0);
+}
+
 // D[tmem] (+)= A[smem desc] * B[smem desc]   (kind::tf32, fp32 accumulate)
 __device__ __forceinline__ void mma_tf32_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                             uint32_t idesc, uint32_t accumulate)
