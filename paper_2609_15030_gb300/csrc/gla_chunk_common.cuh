@@ -457,10 +457,13 @@ __device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpa
         return;
     float m = 0.f;
     if (e_own < D) {
-        // 32 columns at a time
+        // 32 columns at a time; at d = 128 the issuing warp, which also issues D_A meanwhile, takes
+        // a quarter of its lanes' columns and its partner three
+        const int d0 = D == 128 && warp == kIssuer / 32 + 4 ? 32 : colhalf * CW;
+        const int d1 = D == 128 && warp == kIssuer / 32 ? 32 : colhalf * CW + CW;
         __half2 hm = __float2half2_rn(0.f);
 #pragma unroll 1
-        for (int db = colhalf * CW; db < colhalf * CW + CW; db += 32) {
+        for (int db = d0; db < d1; db += 32) {
             float r[32];
             tmem_ld32(tmem + lrow + TM_S + db, r);
             tmem_wait_ld();
