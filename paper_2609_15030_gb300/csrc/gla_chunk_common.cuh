@@ -45,7 +45,11 @@ constexpr float kBoundMargin = 1.00390625f; // 1 + 2^-8
 constexpr float kLamRange = 10.0f;          // fast path: a segment's total log2-decay >= -10, so
                                             // Q~ = q 2^Lam stays far from fp16's subnormals
 constexpr uint64_t kTimeoutNs = 1000000000ull;
-constexpr int kPrefetch = 2;                // segments requested into L2 ahead of the staged one
+// segments requested into L2 ahead of the staged one.  One, since a segment is staged while the
+// one two before it is still in work: two cost 256-token tails 26.6 us instead of 25.3 (their
+// last segments competed with the first), three cost 4 x 32 heads of 16,384 tokens 992 us
+// instead of 960, none 1,037.
+constexpr int kPrefetch = 1;
 
 // shared memory map (offsets from a 1024-byte aligned base), sized for the head width
 // D = d_k = d_v = 128 (a D = 64 head uses the first part of each region).  Operands are
