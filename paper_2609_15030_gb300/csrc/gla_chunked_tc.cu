@@ -105,8 +105,20 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         fence_mbar_init();
         sMisc[1] = 0;   // abort flag
     }
-    if (warp == 0)
+    if (warp == NB / 32)   // not the loader's warp: the first copy does not wait for it
         tmem_alloc(sb + OFF_MISC, TMEM_COLS);
+    // the v buffer of the segment at token `at`
+    auto vbuf = [&](int at) -> int { return (int)((((uint32_t)at + off) / CH) & 1u); };
+    // (one thread) the inputs of the segment at token tok_local into the staging buffers
+    auto copy_inputs = [&](int tok_local) {
+        const int32_t y = p.row0[b] + tok_local;
+        const int32_t x = h * D;
+        mbar_arrive_expect_tx(bar_tma, Geo<D>::STAGE);
+        tma_load_2d(sb + OFF_SG, &maps.g, x, y, bar_tma);
+        tma_load_2d(sb + OFF_SQ, &maps.q, x, y, bar_tma);
+        tma_load_2d(sb + OFF_SK, &maps.k, x, y, bar_tma);
+        tma_load_2d(sb + OFF_SV + vbuf(tok_local) * 16384, &maps.v, x, y, bar_tma);
+    };
     if (tid == kLoader) {
         // the first segment's inputs into L2 while the previous kernel finishes: a
         // prefetch moves no data into this SM, and L2 holds the only copy any later write
@@ -123,6 +135,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // build at once, and the state warps wait below, before they load a state
     if (!RESTART)
         pdl_wait();
+    if (tid == kLoader)
+        copy_inputs(0);   // the barriers are this thread's own work so far: no CTA barrier needed
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -133,8 +147,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
 
     // bookkeeping of the loader (copies issued, one still in flight) and of the issuer,
     // for the waits and the abort path; every mbarrier is waited on by one thread only
-    uint32_t n_tma = 0;
-    bool tma_pending = false;
+    uint32_t n_tma = 1;
+    bool tma_pending = true;
     uint32_t ph_tma = 0, ph_o = 0, ph_s = 0, ph_built = 0, ph_go = 0;
     uint32_t ph_a = 0;               // D_A products
     bool aborted = false;
@@ -150,26 +164,13 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         tma_prefetch_2d(&maps.v, x, y);
         tma_prefetch_2d(&maps.g, x, y);
     };
-    // the v buffer of the segment at token `at`
-    auto vbuf = [&](int at) -> int { return (int)((((uint32_t)at + off) / CH) & 1u); };
-    // (loader) staged inputs of the segment at local position tok_local; segments after
-    // the first start on the 64-token grid, so the segment kPrefetch ahead starts at
-    // tok_local + 64 * kPrefetch and is requested into L2 now
-    auto copy_inputs = [&](int tok_local) {
-        const int32_t y = p.row0[b] + tok_local;
-        const int32_t x = h * D;
-        mbar_arrive_expect_tx(bar_tma, Geo<D>::STAGE);
-        tma_load_2d(sb + OFF_SG, &maps.g, x, y, bar_tma);
-        tma_load_2d(sb + OFF_SQ, &maps.q, x, y, bar_tma);
-        tma_load_2d(sb + OFF_SK, &maps.k, x, y, bar_tma);
-        tma_load_2d(sb + OFF_SV + vbuf(tok_local) * 16384, &maps.v, x, y, bar_tma);
-    };
+    // (loader) the same with its bookkeeping; segments after the first start on the 64-token grid,
+    // so the segment kPrefetch ahead starts at tok_local + 64 * kPrefetch and is requested into L2
     auto issue_tma = [&](int tok_local) {
         copy_inputs(tok_local);
         ++n_tma;
         tma_pending = true;
-        if (tok_local > 0)
-            prefetch(tok_local, CH * kPrefetch);
+        prefetch(tok_local, CH * kPrefetch);
     };
     // one thread (`who`) waits on an mbarrier; false (for every thread) if that wait ran
     // out or another thread raised the abort flag.  CTA-wide, or within the builder (id 1)
@@ -266,8 +267,6 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // reading the last
     auto next_max = [&]() -> int { return smax ^= 1; };
 
-    if (tid == kLoader)
-        issue_tma(0);
     bool prefetched = false;   // (loader) the segments after the first requested into L2
 
     // incoming state -> TMEM (state warps), transposed: S^T[e][d] = state[d][e]; its
@@ -720,7 +719,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == NB / 32) {
         tc_fence_after();
         tmem_dealloc(tmem, TMEM_COLS);
     }

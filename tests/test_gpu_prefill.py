@@ -277,6 +277,41 @@ def test_exact_segment_scores(d, p0, n, gate_above_0):
     _check(*got, *ref, [p0], [n], "exact scores")
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("p0,tail", [(0, 64), (37, 3), (5, 40)])
+def test_fast_runs_of_every_length(d, p0, tail):
+    """Fast runs of 1 to 7 segments, each ended by one exact segment, so that runs start and
+    stop at every phase of the three operand sets and two v buffers, with a build running
+    ahead of the decision that stops it; from on- and off-grid starts, the last segment whole,
+    short (token by token) or ragged.  The resume from every other checkpoint gives the
+    recomputation bit for bit."""
+    dev = device()
+    nH = 2
+    first = 64 - p0 % 64
+    segs = sum(r + 1 for r in range(1, 8))
+    n = first + 64 * (segs - 1) + tail
+    inp = gen_linear(31 + p0 + d, 0, 1, n, nH, d, d)
+    at, k = 0, 0
+    for run in range(1, 8):            # segment k (of the call) is exact after `run` fast ones
+        k += run
+        at = 0 if k == 0 else first + 64 * (k - 1)
+        inp.a[0, at:at + 64] = -0.5
+        k += 1
+    S0 = gen_state(3, 0, 1, nH, d, d)
+    o, S, cks = run_prefill(inp, [p0], [n], S0, 64, dev, hs.HS_LINATTN_CHUNKED_TC)
+    ref = oracle.gla(inp.q, inp.k, inp.v, inp.a, [p0], [n], S0=S0, C_=64)
+    _check(o, S, cks, *ref, [p0], [n], "runs")
+    for m in range(1, len(cks[0]), 2):
+        c = (p0 // 64 + 1 + m) * 64 - p0           # tokens up to that checkpoint
+        if c >= n:
+            continue
+        sub = type(inp)(*(x[:, c:].copy() for x in (inp.q, inp.k, inp.v, inp.a)))
+        o1, S1, _ = run_prefill(sub, [p0 + c], [n - c], cks[0][m][None], 64, dev,
+                                hs.HS_LINATTN_CHUNKED_TC)
+        assert np.array_equal(o1[0].view(np.uint32), o[0, c:].view(np.uint32)), m
+        assert np.array_equal(S1.view(np.uint32), S.view(np.uint32)), m
+
+
 @pytest.mark.parametrize("where", ["short_call", "full_segment"])
 def test_zero_gate_inside_an_exact_segment(where):
     """A zero gate (a = -1e4) followed, in the same segment, by growing gates (the exact
