@@ -26,7 +26,8 @@ constexpr int CH = 64;    // chunk length (absolute grid)
 constexpr int NB = 256;   // operand builders (warps 0..7): cumulative gates, Q~, K~, K~^T, V^T
 constexpr int NW = 256;   // state warps (warps 8..15): state passes, masks, epilogues
 constexpr int NT = NB + NW;
-constexpr int kLoader = 0;   // the first builder thread issues every TMA copy
+constexpr int kLoader = 0;   // the first builder thread issues the copies outside a run of fast
+                             // segments; inside one a lane of warp 1 does
 constexpr int kIssuer = NB + 64;  // the state thread that issues every MMA but D_A: in a warp of
                                   // TMEM lane quarter 2, which has no part in the masking of A
 constexpr int kShort = 8; // segments of at most this many tokens run token by token
@@ -785,9 +786,11 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 // are taken pair by pair.  The tasks (one warp each, drawn from a shared counter, the long ones
 // first) are halves of the key dims of four 16 x 16 units (a square of H = 16, or two of H = 8),
 // quarters of those of each half of the 32 x 32 square, and 64 key dims of a triangle.  Meanwhile the
-// issuing thread's warp feeds S^T Q~^T to the tensor core, about 6 k cycles of dependent products,
-// which the tasks about fill.  Segments with a gate above 0 keep the pairwise form
-// (exact_scores_pairs).
+// issuing thread's warp feeds S^T Q~^T to the tensor core, a chain of dependent products under the
+// tasks.  Tails of 475 tokens of 9 x 16 heads with every segment on this path: 507 us taken pair
+// by pair, 125 us with the squares' products on CUDA cores, 94 us as tf32 fragments, 87 us with
+// the builders looking one segment ahead, now bound by the exponentials: ~2,300 warp instructions a
+// segment.  Segments with a gate above 0 keep the pairwise form (exact_scores_pairs).
 
 // a 16 x 16 unit's rows: query rows r0.. and r1.. (8 each), key rows c0.. and c1.., and the
 // tokens R that (r0, c0) and (r1, c1) factor at; units 2 and 3 hold two squares of H = 8, in
@@ -1295,7 +1298,7 @@ __device__ __forceinline__ void short_outputs(const uint8_t *smem, int L, float 
 }
 
 // ---- operands of a segment's state from the zero state, dS = sum_j K^_j^T v_j with K^_j =
-// k_j 2^{Lam_last - Lam_j} (gla_dstate_kernel and the cluster prefill, same bits in both).  A
+// k_j 2^{Lam_last - Lam_j} (gla_dstate_kernel).  A
 // thread of NWARPS warps owns key dim and value dim (warp mod 4) * 32 + lane and 64 / NWARPS * 4
 // tokens, in groups of 16: Lam_last - Lam_j is the sum of the later groups' log2-decay and a
 // running sum backwards through the group, so strong decay costs no precision.  K^ (tf32)

@@ -15,7 +15,9 @@ namespace hs {
 // scheduled while this one runs.  Each kernel waits for its predecessors to
 // complete (and their memory to be visible) before it touches global memory
 // (L2 prefetches aside), then releases its own dependents; the tensor-core
-// prefill only waits (see pdl_wait).
+// prefill only waits (see pdl_wait), and as the output pass of the
+// segment-parallel prefill it waits only in the warps that read or write what
+// the kernel before it touches.
 __device__ __forceinline__ void pdl_wait_and_release()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
