@@ -12,7 +12,7 @@
 // so a run resumed at a checkpoint on the grid repeats the same operations from there:
 // resumed and full computations agree bit for bit.
 //
-// One CTA per (problem, head, block of 512 state elements); thread i owns four consecutive
+// One CTA per (problem, head, block of 256 state elements); thread i owns four consecutive
 // elements (d, e..e+3) of one key row d (a float4), and the D/4 lanes of a row (a warp at
 // D = 128, a half-warp at D = 64) are consecutive.  The first pass leaves G_n of row d at
 // element (d, 0) of segment n's start-state block: the row's first lane, which owns that
@@ -21,20 +21,39 @@
 // of dS_n (the first lane also G_n) for the next kStages segments into its own slots of
 // shared-memory rings with cp.async (one commit group per segment, so that waiting for the
 // oldest group never waits for a newer copy), applies the oldest and refills its slots.
+//
+// The pass is bound by memory: per segment and head 64 KiB of dS in, 64 KiB of start state out.
+// What it needs is the same number of bytes in flight on every SM: small CTAs whose rings let
+// seven of them on an SM give 16 heads at d = 128 (1,024 CTAs) 6.7 per SM on all 152, while with
+// CTAs of 128 threads and a 40 KiB ring the first 512 / 5 SMs to be free took five each.  dS is
+// read for the last time here, so its lines go first when L2 needs room for the start states, which
+// the output pass reads next.  4,608 tokens of 16 heads, the whole call: 99.3 us with five CTAs of
+// 128 threads, 94.6 with four, 93.1 as it is (1 us of it the L2 policy).
 #include "hs_internal.cuh"
 
 namespace hs {
 namespace {
 
-constexpr int kThreads = 128;        // float4 per thread: 512 state elements per CTA
+constexpr int kThreads = 64;         // a float4 per thread: 256 state elements per CTA
 constexpr int kChunk = 64;           // segments on the 64-token absolute grid
-constexpr int kStages = 16;          // segments whose dS and G are in flight
+constexpr int kStages = 28;          // segments whose dS and G are in flight: 28.4 KiB of rings, so
+                                     // that seven CTAs fit on an SM
+constexpr int kRows = kThreads / 16;  // key rows of a CTA (d = 64; half as many at d = 128)
+constexpr uint32_t kSmemBytes = kStages * (16 * kThreads + 4 * kRows);   // the rings
 
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
+// the L2 policy of lines read for the last time
+__device__ __forceinline__ uint64_t policy_evict_first()
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+    uint64_t p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src, uint64_t policy)
+{
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(
                      (uint32_t)__cvta_generic_to_shared(smem_dst)),
-                 "l"(gmem_src)
+                 "l"(gmem_src), "l"(policy)
                  : "memory");
 }
 
@@ -62,9 +81,11 @@ __global__ void __launch_bounds__(kThreads)
 gla_scan_kernel(const __grid_constant__ ScanParams p)
 {
     constexpr int BLOCKS = D * D / (4 * kThreads);   // CTAs per (problem, head)
-    __shared__ float4 sRing[kStages][kThreads];      // dS of the segments in flight
-    __shared__ float sGate[kStages][kThreads];       // their G (in a row's first lane)
     constexpr int W = D / 4;                         // lanes per key row
+    extern __shared__ float4 smem[];
+    // dS of the segments in flight and their G, one per key row
+    float4 (*sRing)[kThreads] = reinterpret_cast<float4 (*)[kThreads]>(smem);
+    float (*sGate)[kRows] = reinterpret_cast<float (*)[kRows]>(smem + kStages * kThreads);
     const int lane = threadIdx.x & 31;
     const bool row_lead = (lane & (W - 1)) == 0;
     const int bh = blockIdx.x / BLOCKS;
@@ -80,47 +101,59 @@ gla_scan_kernel(const __grid_constant__ ScanParams p)
     float4 *st = reinterpret_cast<float4 *>(p.state + (int64_t)b * sstride + hs_);
     pdl_wait_and_release();
     float4 S = *st;
-    auto seg_end_of = [&](int64_t at) -> int64_t { return min(end, (at / kChunk + 1) * kChunk); };
-    // the rings: one commit group per segment (empty past the last), kStages in flight
-    int64_t ld_at = pos0;             // start of the next segment to copy
-    int32_t ld_seg = p.seg_base[b];
+    const uint64_t last_read = policy_evict_first();
+    // the rings: one commit group per segment (empty past the last), kStages in flight.  Segments
+    // are counted and addresses stepped: with 64-bit positions divided and compared for each, 4,608
+    // tokens of 16 heads took 1 us more
+    const int n_seg = end > pos0 ? (int)((end + kChunk - 1) / kChunk - pos0 / kChunk) : 0;
+    const float *ld_dS = p.dS + (int64_t)p.seg_base[b] * sstride + hs_;   // the next segment to copy
+    float *Sn = p.Sn + (int64_t)p.seg_base[b] * sstride + hs_;            // the current segment
+    const float *ld_G = Sn;
+    int to_load = n_seg;
     auto refill = [&](int slot) {
-        if (ld_at < end) {
-            const int64_t o = (int64_t)ld_seg * sstride + hs_;
-            cp_async16(&sRing[slot][threadIdx.x], p.dS + o);
+        if (to_load > 0) {
+            cp_async16(&sRing[slot][threadIdx.x], ld_dS, last_read);
             if (row_lead)
-                cp_async4(&sGate[slot][threadIdx.x], p.Sn + o);
-            ld_at = seg_end_of(ld_at);
-            ++ld_seg;
+                cp_async4(&sGate[slot][threadIdx.x / W], ld_G);
+            ld_dS += sstride;
+            ld_G += sstride;
+            --to_load;
         }
         cp_async_commit();
     };
     for (int j = 0; j < kStages; ++j)
         refill(j);
-    int64_t at = pos0;
-    int32_t seg = p.seg_base[b];
-    // the next checkpoint position on the grid and its slot pointer, read one checkpoint
-    // ahead (only for positions within the call: the pointer array ends there)
-    int64_t next_ck = (C > 0 && p.ckpt_slots != nullptr) ? (pos0 / C + 1) * C : INT64_MAX;
+    // the segment that ends at the next checkpoint position (-1: none within the call) and its
+    // slot pointer, read one checkpoint ahead (the pointer array ends with the call)
+    const int per_ck = C / kChunk;
+    const int last_ck = (int)(end / kChunk - 1 - pos0 / kChunk);   // the last segment that ends on the grid
+    int ck_seg = -1;
     int32_t ck = p.ck_base[b];
-    float *cs_next = next_ck <= end ? p.ckpt_slots[ck] : nullptr;
+    float *cs_next = nullptr;
+    if (C > 0 && p.ckpt_slots != nullptr && (pos0 / C + 1) * C <= end) {
+        ck_seg = (int)((pos0 / C + 1) * per_ck - 1 - pos0 / kChunk);
+        cs_next = p.ckpt_slots[ck];
+    }
     int slot = 0;
-    while (at < end) {
-        const int64_t e = seg_end_of(at);
+#pragma unroll 1
+    for (int i = 0; i < n_seg; ++i) {
         cp_async_wait_oldest();
         const float4 dq = sRing[slot][threadIdx.x];
-        const float G = __shfl_sync(0xffffffffu, row_lead ? sGate[slot][threadIdx.x] : 0.f,
+        const float G = __shfl_sync(0xffffffffu, row_lead ? sGate[slot][threadIdx.x / W] : 0.f,
                                     lane & ~(W - 1));
         // the start state replaces the gate the first pass left in the row's first float4
-        *reinterpret_cast<float4 *>(p.Sn + (int64_t)seg * sstride + hs_) = S;
+        *reinterpret_cast<float4 *>(Sn) = S;
+        Sn += sstride;
         S.x = fmaf(G, S.x, dq.x);
         S.y = fmaf(G, S.y, dq.y);
         S.z = fmaf(G, S.z, dq.z);
         S.w = fmaf(G, S.w, dq.w);
-        if (e == next_ck) {
+        refill(slot);     // after the slot is consumed: its next copies cannot overtake the reads
+        slot = slot + 1 == kStages ? 0 : slot + 1;
+        if (i == ck_seg) {
             float *cs = cs_next;
-            next_ck += C;
-            if (next_ck <= end)
+            ck_seg = ck_seg + per_ck <= last_ck ? ck_seg + per_ck : -1;
+            if (ck_seg >= 0)
                 cs_next = p.ckpt_slots[++ck];
             if (cs == nullptr || (reinterpret_cast<uintptr_t>(cs) & 15u) != 0) {
                 if (threadIdx.x == 0 && blk == 0 && h == 0)
@@ -129,10 +162,6 @@ gla_scan_kernel(const __grid_constant__ ScanParams p)
                 *reinterpret_cast<float4 *>(cs + hs_) = S;
             }
         }
-        refill(slot);     // after the slot is consumed: its next copies cannot overtake the reads
-        slot = slot + 1 == kStages ? 0 : slot + 1;
-        at = e;
-        ++seg;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     *st = S;
@@ -145,12 +174,13 @@ cudaError_t launch_gla_scan(const ScanParams &p, int d, cudaStream_t s)
     const unsigned bh = (unsigned)p.batch * (unsigned)p.n_heads;
     if (bh == 0)
         return cudaSuccess;
+    static std::atomic<uint64_t> smem_set[2];
     if (d == 128)
-        return launch_pdl(gla_scan_kernel<128>, dim3(bh * (128 * 128 / (4 * kThreads))),
-                          dim3(kThreads), 0, s, p);
+        return launch_pdl_big_smem(gla_scan_kernel<128>, dim3(bh * (128 * 128 / (4 * kThreads))),
+                                   dim3(kThreads), kSmemBytes, s, smem_set[0], p);
     if (d == 64)
-        return launch_pdl(gla_scan_kernel<64>, dim3(bh * (64 * 64 / (4 * kThreads))),
-                          dim3(kThreads), 0, s, p);
+        return launch_pdl_big_smem(gla_scan_kernel<64>, dim3(bh * (64 * 64 / (4 * kThreads))),
+                                   dim3(kThreads), kSmemBytes, s, smem_set[1], p);
     return cudaErrorNotSupported;
 }
 
