@@ -789,8 +789,10 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 // issuing thread's warp feeds S^T Q~^T to the tensor core, a chain of dependent products under the
 // tasks.  Tails of 475 tokens of 9 x 16 heads with every segment on this path: 507 us taken pair
 // by pair, 125 us with the squares' products on CUDA cores, 94 us as tf32 fragments, 87 us with
-// the builders looking one segment ahead, now bound by the exponentials: ~2,300 warp instructions a
-// segment.  Segments with a gate above 0 keep the pairwise form (exact_scores_pairs).
+// the builders looking one segment ahead: 22 k cycles a segment, the decays, operands, scores,
+// update and outputs one after another (a segment's exponentials alone are ~2,300 warp
+// instructions, 4.6 k cycles of the special-function units).
+// Segments with a gate above 0 keep the pairwise form (exact_scores_pairs).
 
 // a 16 x 16 unit's rows: query rows r0.. and r1.. (8 each), key rows c0.. and c1.., and the
 // tokens R that (r0, c0) and (r1, c1) factor at; units 2 and 3 hold two squares of H = 8, in
