@@ -10,9 +10,11 @@
 // call reads and writes 64 KiB per head and computes a few tokens in between), so what matters
 // is that the loads of one CTA overlap the arithmetic and stores of others: 256 threads of 64
 // registers over 32 KiB of state put four CTAs on an SM.  72 problems of 16 heads and 2-8
-// tokens (160 MB): 36.6 us = 4.4 TB/s, against 38.2 us with whole heads (16 x 4 blocks, 125
+// tokens (160 MB): 35.1 us = 4.6 TB/s, against 38.2 us with whole heads (16 x 4 blocks, 125
 // registers, two CTAs per SM).  Tokens are staged eight at a time in shared memory, and their rows
-// of q, k and g are read back 16 bytes at a time, one broadcast per four rows.
+// of q, k and g are read back 16 bytes at a time, one broadcast per four rows.  A thread's two
+// columns go through one f32x2 instruction (scalar instructions: 36.4 us; with each value stored
+// twice in shared memory, so that a load gives the pair: 38.9 us, from the 43 KiB it takes).
 //
 // Per token the arithmetic is fixed: g = expf(a); every element becomes
 // fmaf(g_d, S[d][e], k_d * v_e); partial dot products over each group of 16
@@ -23,9 +25,12 @@
 // only on each token's inputs and the incoming state, so resuming from any
 // checkpoint reproduces a full recomputation bit for bit.
 #include "hs_internal.cuh"
+#include "sm100_ptx.cuh"
 
 namespace hs {
 namespace {
+
+using namespace ptx;
 
 constexpr int kTokBlock = 8;
 
@@ -70,10 +75,10 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
     // this thread's first element of a state
     const int64_t elem = (int64_t)h * D * D + 16 * rg * D + e0 + 2 * cg;
     float *st = p.state + (int64_t)b * p.n_heads * D * D + elem;
-    float2 S[16];   // S[r] = state row 16*rg + r, columns e0 + 2*cg, + 1
+    uint64_t S[16];   // S[r] = state row 16*rg + r, columns e0 + 2*cg, + 1
 #pragma unroll
     for (int r = 0; r < 16; ++r)
-        S[r] = *reinterpret_cast<const float2 *>(st + r * D);
+        S[r] = *reinterpret_cast<const uint64_t *>(st + r * D);
 
     for (int t0 = 0; t0 < n; t0 += kTokBlock) {
         const int tb = min(kTokBlock, n - t0);
@@ -94,8 +99,8 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
         __syncthreads();
 #pragma unroll 1
         for (int tt = 0; tt < tb; ++tt) {
-            const float2 v2 = *reinterpret_cast<const float2 *>(&sv[tt][2 * cg]);
-            float2 acc = make_float2(0.f, 0.f);
+            const uint64_t v2 = *reinterpret_cast<const uint64_t *>(&sv[tt][2 * cg]);
+            uint64_t acc = 0;
 #pragma unroll
             for (int r4 = 0; r4 < 16; r4 += 4) {
                 const int i = 16 * rg + r4;
@@ -106,14 +111,12 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
                             qq[4] = {q4.x, q4.y, q4.z, q4.w};
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                    float2 &s = S[r4 + x];
-                    s.x = fmaf(g[x], s.x, kk[x] * v2.x);
-                    s.y = fmaf(g[x], s.y, kk[x] * v2.y);
-                    acc.x = fmaf(qq[x], s.x, acc.x);
-                    acc.y = fmaf(qq[x], s.y, acc.y);
+                    uint64_t &s = S[r4 + x];
+                    s = fma2(pair(g[x], g[x]), s, mul2(pair(kk[x], kk[x]), v2));
+                    acc = fma2(pair(qq[x], qq[x]), s, acc);
                 }
             }
-            *reinterpret_cast<float2 *>(&spart[tt][rg][2 * cg]) = acc;
+            *reinterpret_cast<uint64_t *>(&spart[tt][rg][2 * cg]) = acc;
             if (t0 + tt + 1 == next_ck) {
                 float *slot = p.ckpt_slots[ck++];
                 next_ck = next_ck <= n - p.ckpt_interval ? next_ck + p.ckpt_interval : 0;
@@ -127,7 +130,7 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
                     slot += elem;
 #pragma unroll
                     for (int r = 0; r < 16; ++r)
-                        *reinterpret_cast<float2 *>(slot + r * D) = S[r];
+                        *reinterpret_cast<uint64_t *>(slot + r * D) = S[r];
                 }
             }
         }
@@ -135,7 +138,7 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
             // final state out before the output reduction, so the store drains behind it
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                *reinterpret_cast<float2 *>(st + r * D) = S[r];
+                *reinterpret_cast<uint64_t *>(st + r * D) = S[r];
         }
         __syncthreads();
         for (int idx = tid; idx < tb * kCols; idx += NTH) {

@@ -146,6 +146,28 @@ __device__ __forceinline__ bool elect_one()
     return r != 0;
 }
 
+// two float32 operations in one instruction, each rounded as its scalar form
+__device__ __forceinline__ uint64_t pair(float x, float y)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // a value all lanes of the warp agree on, known to the compiler as warp-uniform
 __device__ __forceinline__ int uniform(int x)
 {
