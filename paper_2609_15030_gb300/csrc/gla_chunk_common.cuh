@@ -23,7 +23,7 @@ namespace gck {
 using namespace ptx;
 
 constexpr int CH = 64;    // chunk length (absolute grid)
-constexpr int NB = 256;   // operand builders (warps 0..7): cumulative gates, Q~, K~, K~^T, V^T
+constexpr int NB = 256;   // operand builders (warps 0..7): cumulative gates, Q~, K~, V^T
 constexpr int NW = 256;   // state warps (warps 8..15): state passes, masks, epilogues
 constexpr int NT = NB + NW;
 constexpr int kLoader = 0;   // the first builder thread issues the copies outside a run of fast
@@ -78,9 +78,8 @@ constexpr uint32_t OFF_DG = 226176;     // diagonal of A in float32, with the op
 constexpr uint32_t SMEM_BYTES = 227712 + 1024;
 
 // tensor memory: D_O alternates between two buffers by chunk parity, placed on
-// either side of S^T so that [D_O0 | S^T] and [S^T | D_O1] are each one accumulator of
-// N = 64 + D; even chunks order the (64 + D)-row operand as [A ; K~^T], odd ones as
-// [K~^T ; A].  Every MMA has M = 128 (TMEM lanes = value dim e, or query row i for D_A):
+// either side of S^T; the exact path takes [D_O0 | S^T] as one accumulator of N = 64 + D
+// columns.  Every MMA has M = 128 (TMEM lanes = value dim e, or query row i for D_A):
 // with D = 64 the lanes 64..127 of the state-side products are computed and never read.
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_O0 = 0;           // D_O of even chunks (lane e, col i), 64 cols
@@ -293,9 +292,10 @@ __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, int vb, bool bui
 // (dp, qt) owns key dims 2dp, 2dp+1 for the TPG tokens of group qt (16 tokens x 4 groups at
 // D = 128, 8 x 8 at D = 64): it sums their log2-gates, then runs the cumulative sum again
 // from the earlier groups' totals (shared memory; 2^{Lam_last} into gam slot `gslot`) while
-// it writes Q~ and K~ (token-major, the d-contractions' operands) and K~^T (rows of
-// [A ; K~^T]), fp16, with 4- and 16-byte stores.  Per warp: max |q|, |k| and per thread
-// whether its operands fit fp16 (for the guard).  The diagonal A_ii = q_i . k_i (no decay between a token and itself)
+// it writes Q~ and K~ (token-major), fp16, with 4-byte stores.  Its two key dims are a register
+// pair: their sums and products are f32x2 instructions, the roundings those of the scalar ones
+// (with the state pass's decay: 4 x 32 heads of 16,384 tokens 957.5 us, now 950).  Per warp:
+// max |q|, |k| and per thread whether its operands fit fp16 (for the guard).  The diagonal A_ii = q_i . k_i (no decay between a token and itself)
 // is summed in float32 from the bf16 inputs, each warp's 64 key dims by a butterfly, into
 // the set's diagonal partials: fp16 Q~ and K~ would round the terms of that dot product to
 // 11 bits, which a token whose own q . k cancels cannot afford.
@@ -320,15 +320,14 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int vb, int ise
     float amax = -INFINITY;
     {
         // group totals
-        float r0 = 0.f, r1 = 0.f;
+        uint64_t r = 0;
 #pragma unroll
         for (int x = 0; x < G::TPG; ++x) {
-            const float2 a = *reinterpret_cast<const float2 *>(sG + (G::TPG * qt + x) * D + 2 * dp);
-            amax = fmaxf(amax, fmaxf(a.x, a.y));
-            r0 = fmaf(a.x, kLog2e, r0);
-            r1 = fmaf(a.y, kLog2e, r1);
+            const uint64_t a = *reinterpret_cast<const uint64_t *>(sG + (G::TPG * qt + x) * D + 2 * dp);
+            amax = fmaxf(amax, fmaxf(unpair(a).x, unpair(a).y));
+            r = fma2(a, pair(kLog2e, kLog2e), r);
         }
-        *reinterpret_cast<float2 *>(sTot + qt * D + 2 * dp) = make_float2(r0, r1);
+        *reinterpret_cast<uint64_t *>(sTot + qt * D + 2 * dp) = r;
     }
     bar_builders();
     // the running sums start from the earlier groups' totals
@@ -357,27 +356,30 @@ __device__ __forceinline__ bool build_fast(uint8_t *smem, int L, int vb, int ise
     __half2 hq = __float2half2_rn(0.f), hk = hq;                 // max |Q~|, |K~| (fp16)
     // runs of 8 tokens; within a run, token pairs: Q~ and K~ as fp16 pairs of key dims
     float *sDg = reinterpret_cast<float *>(smem + OFF_DG) + iset * 128 + (dp >> 5) * 64;
+    uint64_t run = pair(run0, run1);
 #pragma unroll 1
     for (int grp = 0; grp < G::TPG / 8; ++grp) {
         const int j0 = G::TPG * qt + 8 * grp;
         // the eight tokens' inputs first: the compiler cannot move a load over the operand stores
-        float2 a[8];
+        uint64_t a[8];
         uint32_t q2[8], k2[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            a[t] = *reinterpret_cast<const float2 *>(sG + (j0 + t) * D + 2 * dp);
+            a[t] = *reinterpret_cast<const uint64_t *>(sG + (j0 + t) * D + 2 * dp);
             q2[t] = *reinterpret_cast<const uint32_t *>(sQ + (j0 + t) * D + 2 * dp);
             k2[t] = *reinterpret_cast<const uint32_t *>(sK + (j0 + t) * D + 2 * dp);
         }
         float pd[8];   // q . k over this thread's two key dims, tokens 8 grp + 0..7 of its group
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-            run0 = fmaf(a[t].x, kLog2e, run0);
-            run1 = fmaf(a[t].y, kLog2e, run1);
+            run = fma2(a[t], pair(kLog2e, kLog2e), run);
+            const float2 lam = unpair(run);
             const float q0 = __uint_as_float(q2[t] << 16), q1 = __uint_as_float(q2[t] & 0xFFFF0000u);
             const float k0 = __uint_as_float(k2[t] << 16), k1 = __uint_as_float(k2[t] & 0xFFFF0000u);
-            const uint32_t qp = pack_h2(q0 * ex2(run0), q1 * ex2(run1));
-            const uint32_t kp = pack_h2(k0 * ex2(-run0), k1 * ex2(-run1));
+            const float2 qs = unpair(mul2(pair(q0, q1), pair(ex2(lam.x), ex2(lam.y))));
+            const float2 ks = unpair(mul2(pair(k0, k1), pair(ex2(-lam.x), ex2(-lam.y))));
+            const uint32_t qp = pack_h2(qs.x, qs.y);
+            const uint32_t kp = pack_h2(ks.x, ks.y);
             pd[t] = fmaf(q1, k1, q0 * k0);
             *reinterpret_cast<uint32_t *>(set + S_QH + h_off(64, j0 + t, 2 * dp)) = qp;
             *reinterpret_cast<uint32_t *>(set + S_KH + h_off(64, j0 + t, 2 * dp)) = kp;
@@ -477,10 +479,12 @@ __device__ __forceinline__ void state_pass(uint8_t *smem, uint32_t tmem, int gpa
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const float4 g4 = *reinterpret_cast<const float4 *>(gam + 4 * c);
-                    r[4 * c] *= g4.x;
-                    r[4 * c + 1] *= g4.y;
-                    r[4 * c + 2] *= g4.z;
-                    r[4 * c + 3] *= g4.w;
+                    const float2 x = unpair(mul2(pair(r[4 * c], r[4 * c + 1]), pair(g4.x, g4.y)));
+                    const float2 y = unpair(mul2(pair(r[4 * c + 2], r[4 * c + 3]), pair(g4.z, g4.w)));
+                    r[4 * c] = x.x;
+                    r[4 * c + 1] = x.y;
+                    r[4 * c + 2] = y.x;
+                    r[4 * c + 3] = y.y;
                 }
                 tmem_st32(tmem + lrow + TM_S + db, r);
             }

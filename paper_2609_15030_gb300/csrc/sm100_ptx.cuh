@@ -154,6 +154,13 @@ __device__ __forceinline__ uint64_t pair(float x, float y)
     return r;
 }
 
+__device__ __forceinline__ float2 unpair(uint64_t a)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
 {
     uint64_t r;
