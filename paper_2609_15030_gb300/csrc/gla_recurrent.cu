@@ -10,11 +10,12 @@
 // call reads and writes 64 KiB per head and computes a few tokens in between), so what matters
 // is that the loads of one CTA overlap the arithmetic and stores of others: 256 threads of 64
 // registers over 32 KiB of state put four CTAs on an SM.  72 problems of 16 heads and 2-8
-// tokens (160 MB): 35.1 us = 4.6 TB/s, against 38.2 us with whole heads (16 x 4 blocks, 125
-// registers, two CTAs per SM).  Tokens are staged eight at a time in shared memory, and their rows
+// tokens (160 MB): 31.7 us = 5.1 TB/s, against 35.1 us before its lines were requested into L2 first
+// (the tokens alone: 32.9) and 38.2 us with whole heads (16 x 4 blocks, 125 registers, two CTAs per SM).  Tokens are staged eight at a time in shared memory, and their rows
 // of q, k and g are read back 16 bytes at a time, one broadcast per four rows.  A thread's two
-// columns go through one f32x2 instruction (scalar instructions: 36.4 us; with each value stored
-// twice in shared memory, so that a load gives the pair: 38.9 us, from the 43 KiB it takes).
+// columns go through one f32x2 instruction (scalar instructions cost 1.3 us more; with each value
+// stored twice in shared memory, so that a load gives the pair, 3.7 us more, from the 43 KiB it
+// takes).
 //
 // Per token the arithmetic is fixed: g = expf(a); every element becomes
 // fmaf(g_d, S[d][e], k_d * v_e); partial dot products over each group of 16
@@ -65,8 +66,28 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
     const int n = p.n_tokens[b];
     if (n <= 0)
         return;
-    pdl_wait_and_release();
     const int tid = threadIdx.x;
+    {
+        // the first tokens' rows and the state into L2, while the kernel before finishes and ahead of
+        // the loads below (a prefetch moves no data into this SM, so it is safe even if that kernel
+        // writes them): the tokens' loads, needed first, are issued last, and waited a whole trip to
+        // memory behind the state's
+        constexpr int LB = D / 64;   // 128-byte lines of one bf16 row (a float row is 2 LB)
+        const int t = tid / (5 * LB), l = tid % (5 * LB);
+        if (t < min(n, kTokBlock)) {
+            const int64_t at = (((int64_t)p.row0[b] + t) * p.n_heads + h) * D;
+            const char *src = l < LB       ? reinterpret_cast<const char *>(p.q + at) + 128 * l
+                              : l < 2 * LB ? reinterpret_cast<const char *>(p.k + at) + 128 * (l - LB)
+                              : l < 3 * LB ? reinterpret_cast<const char *>(p.v + at) + 128 * (l - 2 * LB)
+                                           : reinterpret_cast<const char *>(p.log_g + at) + 128 * (l - 3 * LB);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+        }
+    }
+    // the CTA's 64 columns of a state row are two lines
+    if (tid < 2 * D)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(p.state + ((int64_t)b * p.n_heads + h) * D * D +
+                                                      (tid >> 1) * D + e0 + (tid & 1) * 32));
+    pdl_wait_and_release();
     const int cg = tid % NCG;
     const int rg = tid / NCG;
     int next_ck = p.first_ck[b];      // tokens up to the next checkpoint, and its slot
