@@ -10,12 +10,13 @@
 // call reads and writes 64 KiB per head and computes a few tokens in between), so what matters
 // is that the loads of one CTA overlap the arithmetic and stores of others: 256 threads of 64
 // registers over 32 KiB of state put four CTAs on an SM.  72 problems of 16 heads and 2-8
-// tokens (160 MB): 31.7 us = 5.1 TB/s, against 35.1 us before its lines were requested into L2 first
-// (the tokens alone: 32.9) and 38.2 us with whole heads (16 x 4 blocks, 125 registers, two CTAs per SM).  Tokens are staged eight at a time in shared memory, and their rows
-// of q, k and g are read back 16 bytes at a time, one broadcast per four rows.  A thread's two
-// columns go through one f32x2 instruction (scalar instructions cost 1.3 us more; with each value
-// stored twice in shared memory, so that a load gives the pair, 3.7 us more, from the 43 KiB it
-// takes).
+// tokens (160 MB): 29.5 us = 5.4 TB/s; 31.7 without the later CTAs' states requested into L2, 35.1
+// without the CTA's own lines requested first either (its tokens' alone: 32.9), and 38.2 us with
+// whole heads (16 x 4 blocks, 125 registers, two CTAs per SM) then.  Tokens are staged eight at a
+// time in shared memory, and their rows of q, k and g are read back 16 bytes at a time, one
+// broadcast per four rows.  A thread's two columns go through one f32x2 instruction (scalar
+// instructions cost 1.3 us more; with each value stored twice in shared memory, so that a load
+// gives the pair, 3.7 us more, from the 43 KiB it takes).
 //
 // Per token the arithmetic is fixed: g = expf(a); every element becomes
 // fmaf(g_d, S[d][e], k_d * v_e); partial dot products over each group of 16
@@ -49,7 +50,7 @@ constexpr int kCols = 64;             // value columns of a CTA
 // the CTA's columns 2*cg, 2*cg+1.
 template <int D>
 __global__ void __launch_bounds__((kCols / 2) * (D / 16), D == 128 ? 4 : 7)
-gla_recurrent_kernel(const __grid_constant__ GlaParams p)
+gla_recurrent_kernel(const __grid_constant__ GlaParams p, unsigned ahead)
 {
     constexpr int NCG = kCols / 2;    // column pairs (lanes)
     constexpr int NRG = D / 16;       // row groups of 16
@@ -88,6 +89,14 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(p.state + ((int64_t)b * p.n_heads + h) * D * D +
                                                       (tid >> 1) * D + e0 + (tid & 1) * 32));
     pdl_wait_and_release();
+    // the state of a CTA that starts about when this one ends (see the launch)
+    const unsigned nx = blockIdx.x + ahead;
+    if (tid < 2 * D && nx < gridDim.x) {
+        const unsigned nbh = nx / NCB;
+        if (p.n_tokens[nbh / p.n_heads] > 0)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.state + (int64_t)nbh * D * D + (tid >> 1) * D +
+                                                          (nx - nbh * NCB) * kCols + (tid & 1) * 32));
+    }
     const int cg = tid % NCG;
     const int rg = tid / NCG;
     int next_ck = p.first_ck[b];      // tokens up to the next checkpoint, and its slot
@@ -176,12 +185,15 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p)
 
 }  // namespace
 
-cudaError_t launch_gla_recurrent(const GlaParams &p, int d, cudaStream_t s)
+cudaError_t launch_gla_recurrent(const GlaParams &p, int d, int sm_count, cudaStream_t s)
 {
     const unsigned grid = (unsigned)p.batch * (unsigned)p.n_heads * (unsigned)(d / kCols);
+    // each CTA requests the state three CTAs per SM further on (an SM holds four at d = 128, seven at
+    // d = 64).  72 problems of 16 heads, 2-8 tokens: 31.7 us without, 29.9 two, 29.5 three, 30.2 four,
+    // 31.7 five, 32.6 eight further; 32 problems of 32 heads, 1-2 tokens: 24.6, 22.7, 22.7, 22.8, 23.3, 24.1
     if (d == 128)
-        return launch_pdl(gla_recurrent_kernel<128>, dim3(grid), dim3(256), 0, s, p);
-    return launch_pdl(gla_recurrent_kernel<64>, dim3(grid), dim3(128), 0, s, p);
+        return launch_pdl(gla_recurrent_kernel<128>, dim3(grid), dim3(256), 0, s, p, 3u * sm_count);
+    return launch_pdl(gla_recurrent_kernel<64>, dim3(grid), dim3(128), 0, s, p, 5u * sm_count);
 }
 
 }  // namespace hs

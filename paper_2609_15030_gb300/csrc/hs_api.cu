@@ -375,7 +375,11 @@ static hs_status prefill(const hs_linattn_shape *shp, const uint16_t *q, const u
         return cuda_status(hs::launch_gla_chunked_tc(p, s.d_k, stream));
     if (s.kernel == HS_LINATTN_SINGLE_TOKEN || (s.kernel == HS_LINATTN_AUTO && max_n == 1))
         return cuda_status(hs::launch_gla_decode(p, s.d_k, stream));
-    return cuda_status(hs::launch_gla_recurrent(p, s.d_k, stream));
+    int sms = 0;
+    const hs_status sm_st = sm_count(&sms);
+    if (sm_st != HS_OK)
+        return sm_st;
+    return cuda_status(hs::launch_gla_recurrent(p, s.d_k, sms, stream));
 }
 
 hs_status hs_linattn_prefill_from_state(const hs_linattn_shape *shp, const uint16_t *q,

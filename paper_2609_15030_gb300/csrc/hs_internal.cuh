@@ -155,7 +155,7 @@ struct ScanParams {
     int32_t seg_base[HS_MAX_BATCH];   // index of the problem's first segment in dS / Sn
 };
 cudaError_t launch_gla_scan(const ScanParams &p, int d, cudaStream_t s);
-cudaError_t launch_gla_recurrent(const GlaParams &p, int d, cudaStream_t s);
+cudaError_t launch_gla_recurrent(const GlaParams &p, int d, int sm_count, cudaStream_t s);
 cudaError_t launch_gla_decode(const GlaParams &p, int d, cudaStream_t s);
 cudaError_t launch_gla_chunked_tc(const GlaParams &p, int d, cudaStream_t s);
 // every segment from its own start state (see the kernel); ckpt_slots must be nullptr
