@@ -46,6 +46,11 @@ constexpr float kBoundMargin = 1.00390625f; // 1 + 2^-8
 constexpr float kLamRange = 10.0f;          // fast path: a segment's total log2-decay >= -10, so
                                             // Q~ = q 2^Lam stays far from fp16's subnormals
 constexpr uint64_t kTimeoutNs = 1000000000ull;
+// decision words of a run (fast path or not), in turn by segment.  Two: builder threads read the
+// one of segment k - 1 after the barrier that follows its wait, and the first of them may already
+// hand segment k over, whose decision must not land in the word the others are still to read; the
+// decision after that needs a hand-over which comes after every builder thread passed its next wait.
+constexpr int kDecisions = 2;
 // segments requested into L2 ahead of the staged one.  One, since a segment is staged while the
 // one two before it is still in work: two cost 256-token tails 26.6 us instead of 25.3 (their
 // last segments competed with the first), three cost 4 x 32 heads of 16,384 tokens 992 us

@@ -72,11 +72,10 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const uint32_t sb = smem_u32(smem);
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
-    // [0] TMEM base, [1] abort flag, [2] decision on the latest built segment (1 = fast),
-    // [3] run result (1 = the segment at [4] needs the exact path), [4] token index where the
+    // [0] TMEM base, [1] abort flag, [3] run result (1 = the segment at [4] needs the exact path), [4] token index where the
     // run stopped, [5] whether that segment's build is whole (0: its gates alone send it to the
-    // exact path, its inputs still staged), [9] an exact segment's look ahead, [10] its task
-    // counter, [11..12] whether the build of the latest segments is whole, by segment parity
+    // exact path, its inputs still staged), [6..7] decisions on the latest segments (1 = fast),
+    // by segment, [9] an exact segment's look ahead, [10] its task counter, [11..12] whether the build of the latest segments is whole, by segment parity
     volatile uint32_t *sMisc = reinterpret_cast<volatile uint32_t *>(smem + OFF_MISC);
     const uint32_t bar_tma = sb + OFF_BAR, bar_a = sb + OFF_BAR + 8, bar_o = sb + OFF_BAR + 16,
                    bar_s = sb + OFF_BAR + 24, bar_built = sb + OFF_BAR + 32,
@@ -298,6 +297,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     };
 
     int kseq = 0;   // long segments of the current run so far (slot of 2^{Lam_last}: kseq mod 4)
+    // the decision word of the run's segment k
+    auto decision = [&](int k) -> volatile uint32_t & { return sMisc[6 + (k & (kDecisions - 1))]; };
     // the guard of a built fast segment (state warps, after the wait for the builders): log-gates
     // <= 0, and every fp16 operand (Q~, K~, V, A, the fp16 copy of the state it starts from)
     // below 2^15 in magnitude.  Returns whether the segment's own inputs pass; `state_ok` says
@@ -362,7 +363,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     // the builders stage and build segment k+1 while the state warps finish segment k.
     // Handoffs (each mbarrier has one waiting thread and one arriving party):
     //   bar_built: builders -> state warps, segment k built (operands, V^T, guard maxima)
-    //   bar_go:    state warps -> builders, the decision on segment k is made (sMisc[2]);
+    //   bar_go:    state warps -> builders, the decision on segment k is made (see kDecisions);
     //              when it is fast, it also means the products of segment k-1 are complete, so
     //              that segment k+2 may take their operand set and V^T buffer
     // A run ends after the last long segment, before a segment whose own inputs the guard
@@ -416,7 +417,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             build_values<D>(smem, tmem, vbuf(rtok), iset, built, mq, mk, ok);
             tc_fence_before();
             // every warp's part done, and the decision on the segment before
-            if (kseq > 0 ? !wait_group(1, kLoader, bar_go, ph_go) || sMisc[2] == 0 : !sync_group(1))
+            if (kseq > 0 ? !wait_group(1, kLoader, bar_go, ph_go) || decision(kseq - 1) == 0 : !sync_group(1))
                 return;
             if (tid == kLoader) {
                 sMisc[11 + (kseq & 1)] = built ? 1u : 0u;
@@ -492,7 +493,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                       state_ok);
             const bool fast = inputs_ok && state_ok;
             if (tid == kIssuer) {
-                sMisc[2] = fast ? 1u : 0u;
+                decision(kseq) = fast ? 1u : 0u;
                 mbar_arrive(bar_go);
             }
             const int L = seg_len(rtok);
@@ -578,7 +579,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             bool state_ok;
             const bool fast = guard(state_max(), iset, state_ok) && state_ok;
             if (tid == kIssuer) {
-                sMisc[2] = fast ? 1u : 0u;
+                decision(kseq) = fast ? 1u : 0u;
                 mbar_arrive(bar_go);
             }
             request(rtok + L);

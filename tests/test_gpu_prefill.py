@@ -312,6 +312,42 @@ def test_fast_runs_of_every_length(d, p0, tail):
         assert np.array_equal(S1.view(np.uint32), S.view(np.uint32)), m
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("p0,tail", [(0, 64), (5, 40)])
+def test_fast_runs_ended_by_magnitude(d, p0, tail):
+    """As above, but the segment that ends a run has ordinary gates and fails the bound on
+    |q| |k|: its build is whole, the builders are a segment past it with one more copy in flight,
+    and its inputs are staged again, at every phase of the operand sets and v buffers.  12 heads
+    of two problems, so that the threads of a group meet the decision at many different times."""
+    dev = device()
+    nH = 12
+    first = 64 - p0 % 64
+    segs = sum(r + 1 for r in range(1, 8))
+    n = first + 64 * (segs - 1) + tail
+    inp = gen_linear(53 + p0 + d, 0, 2, n, nH, d, d)
+    k = 0
+    for run in range(1, 8):
+        k += run
+        x = slice(0 if k == 0 else first + 64 * (k - 1), first + 64 * k)
+        for y in (inp.q, inp.k):
+            y[:, x] = _scaled(y[:, x], 64.0)
+            assert np.abs(bf16_bits_to_f32(y[:, x])).max(axis=(1, 3)).min() > (2.0 ** 15 / d) ** 0.5
+        k += 1
+    S0 = gen_state(3, 0, 2, nH, d, d)
+    o, S, cks = run_prefill(inp, [p0] * 2, [n] * 2, S0, 64, dev, hs.HS_LINATTN_CHUNKED_TC)
+    ref = oracle.gla(inp.q, inp.k, inp.v, inp.a, [p0] * 2, [n] * 2, S0=S0, C_=64, threads=16)
+    _check(o, S, cks, *ref, [p0] * 2, [n] * 2, "runs")
+    for m in range(1, len(cks[0]), 3):
+        c = (p0 // 64 + 1 + m) * 64 - p0
+        if c >= n:
+            continue
+        sub = type(inp)(*(x[:, c:].copy() for x in (inp.q, inp.k, inp.v, inp.a)))
+        o1, S1, _ = run_prefill(sub, [p0 + c] * 2, [n - c] * 2, np.stack([x[m] for x in cks]), 64, dev,
+                                hs.HS_LINATTN_CHUNKED_TC)
+        assert np.array_equal(o1.view(np.uint32), o[:, c:].view(np.uint32)), m
+        assert np.array_equal(S1.view(np.uint32), S.view(np.uint32)), m
+
+
 @pytest.mark.parametrize("where", ["short_call", "full_segment"])
 def test_zero_gate_inside_an_exact_segment(where):
     """A zero gate (a = -1e4) followed, in the same segment, by growing gates (the exact
