@@ -83,8 +83,7 @@ constexpr uint32_t OFF_DG = 226176;     // diagonal of A in float32, with the op
 constexpr uint32_t SMEM_BYTES = 227712 + 1024;
 
 // tensor memory: D_O alternates between two buffers by chunk parity, placed on
-// either side of S^T; the exact path takes [D_O0 | S^T] as one accumulator of N = 64 + D
-// columns.  Every MMA has M = 128 (TMEM lanes = value dim e, or query row i for D_A):
+// either side of S^T.  Every MMA has M = 128 (TMEM lanes = value dim e, or query row i for D_A):
 // with D = 64 the lanes 64..127 of the state-side products are computed and never read.
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_O0 = 0;           // D_O of even chunks (lane e, col i), 64 cols
@@ -115,7 +114,7 @@ struct Geo {
     static constexpr uint32_t O1 = TM_S + D;      // D_O of odd chunks, right of S^T
     static constexpr uint32_t SHI = TM_S + D;     // exact path: hi part of S^T
     static constexpr uint32_t IDF_ST = idesc_f16(128, D, 1);       // S^T += V^T K~ (K~ read MN-major)
-    static constexpr uint32_t IDT_UP = idesc_tf32(128, 64 + D, 0, 0);   // exact: [D_O | S^T] update
+    static constexpr uint32_t IDT_ST = idesc_tf32(128, D, 0, 0);   // exact: S^T += V^T K^
     static constexpr uint32_t STAGE = 3 * CH * D * 2 + CH * D * 4;  // staged q, k, v, log-gates
 };
 
@@ -1165,17 +1164,20 @@ __device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int
     __syncthreads();
 }
 
-// (issuing thread) [D_O | S^T] += V^T [A ; K^^T]^T (S^T decayed before), 8 tokens per step: one
-// accumulator of N = 64 + D columns, since D_O (TM_O0) and S^T (TM_S) are adjacent
+// (issuing thread) D_O += V^T A^T and S^T += V^T K^ (S^T decayed before), 8 tokens per step.  Two
+// accumulators of N = 64 and N = D columns: S^T Q~^T is not waited for, and products execute in
+// issue order only on the same accumulator with the same shape.  (As one accumulator [D_O | S^T] of
+// N = 64 + D after a wait for S^T Q~^T: tails of 475 tokens of 9 x 16 heads 87.8 us, one segment of
+// two d = 64 heads 11.0 us; so 86.5 and 10.5.)
 template <int D>
 __device__ __forceinline__ void exact_issue_update(uint32_t tmem, uint32_t sb)
 {
-    static_assert(TM_S == TM_O0 + 64, "D_O and S^T adjacent");
 #pragma unroll 1
     for (int kk = 0; kk < CH / 8; ++kk) {
         const uint32_t koff = (kk >> 2) * (Geo<D>::ROWS * 128) + (kk & 3) * 32;
-        mma_tf32_ts(tmem + TM_O0, tmem + TM_V + kk * 8, sdesc_sw128(sb + X_B2 + koff, 16, 1024),
-                    Geo<D>::IDT_UP, 1);
+        mma_tf32_ts(tmem + TM_O0, tmem + TM_V + kk * 8, sdesc_sw128(sb + X_B2 + koff, 16, 1024), IDT_N64, 1);
+        mma_tf32_ts(tmem + TM_S, tmem + TM_V + kk * 8, sdesc_sw128(sb + X_B2 + 8192 + koff, 16, 1024),
+                    Geo<D>::IDT_ST, 1);
     }
 }
 

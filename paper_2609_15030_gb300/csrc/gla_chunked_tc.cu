@@ -328,7 +328,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
     int ready = 0;
     auto exact_segment = [&](int tok_s, int L) -> bool {
         const int seg_end = tok_s + L;
-        exact_operands<D>(smem, tmem, L, vbuf(tok_s), const_cast<int *>(reinterpret_cast<volatile int *>(sMisc + 10)));
+        exact_operands<D>(smem, tmem, L, vbuf(tok_s),
+                          const_cast<int *>(reinterpret_cast<volatile int *>(sMisc + 10)));
         if (warp_u == kIssuer / 32) {
             tc_fence_after();
             if (elect_one()) {

@@ -1,7 +1,8 @@
-"""The hand-over between the two warp groups of the tensor-core prefill, on the CPU: every
-interleaving of a small model of a run of fast segments.
+"""Orders that the tensor-core prefill's warps must keep, on the CPU: every interleaving of a
+small model of the hand-over in a run of fast segments, and the order of two tensor-core
+products on the same columns.
 
-Two builder threads (the loader, which waits and arrives for its group, and any other) and the
+The hand-over: two builder threads (the loader, which waits and arrives for its group, and any other) and the
 issuing state thread pass the segments on as the kernel's builder_run and state_run do: built ->
 decision -> go.  Both builder threads read the decision on the segment before, after a barrier of
 their group; a thread that reads another answer than its partner goes to the CTA-wide barrier
@@ -85,3 +86,26 @@ def test_every_builder_thread_reads_the_same_decision(stop):
         assert _stuck(words, fast) == []
     if stop > 1:                                       # the model sees the fault of a single word
         assert _stuck(1, (1,) * (stop - 1) + (0, 1))
+
+
+def _body(src, name):
+    """The text of a function from its name to the closing brace in column 0."""
+    at = src.index(f" {name}(")
+    return src[at:src.index("\n}", at)]
+
+
+def test_products_on_the_same_columns_have_one_shape():
+    """Tensor-core products execute in issue order only on the same accumulator with the same
+    shape.  The exact path's update accumulates onto D_O while S^T Q~^T may still run: the
+    accumulators both write have one instruction descriptor, and no other overlaps them (S^T
+    starts where D_O's 64 columns end)."""
+    src = _source("gla_chunk_common.cuh")
+    product = re.compile(r"mma_tf32_ts\(tmem \+ (\w+),.*?((?:Geo<D>::)?IDT_\w+)", re.S)
+    first = dict(product.findall(_body(src, "exact_issue_sq")))
+    second = dict(product.findall(_body(src, "exact_issue_update")))
+    assert first.keys() & second.keys() == {"TM_O0"}
+    assert first["TM_O0"] == second["TM_O0"] == "IDT_N64"
+    assert re.search(r"IDT_N64 = idesc_tf32\(128, 64, ", src)
+    assert second == {"TM_O0": "IDT_N64", "TM_S": "Geo<D>::IDT_ST"}
+    column = lambda name: int(re.search(rf"constexpr uint32_t {name} = (\d+);", src).group(1))
+    assert column("TM_O0") + 64 <= column("TM_S")
