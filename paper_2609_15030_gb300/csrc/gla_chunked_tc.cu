@@ -225,6 +225,14 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             aborted = true;
         return !stop;
     };
+    // (builder warps) the next decision.  In the output pass it waits for the state warps, and they
+    // for the kernel before: the loader waits for that kernel itself first, so that the time limit
+    // covers this kernel's own work alone
+    auto wait_go = [&]() -> bool {
+        if (RESTART && tid == kLoader)
+            pdl_wait();
+        return wait_group(1, kLoader, bar_go, ph_go);
+    };
     auto sync_all = [&]() -> bool {
         const bool stop = __syncthreads_or(sMisc[1] != 0) != 0;
         if (stop)
@@ -418,14 +426,14 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
             build_values<D>(smem, tmem, vbuf(rtok), iset, built, mq, mk, ok);
             tc_fence_before();
             // every warp's part done, and the decision on the segment before
-            if (kseq > 0 ? !wait_group(1, kLoader, bar_go, ph_go) || decision(kseq - 1) == 0 : !sync_group(1))
+            if (kseq > 0 ? !wait_go() || decision(kseq - 1) == 0 : !sync_group(1))
                 return;
             if (tid == kLoader) {
                 sMisc[11 + (kseq & 1)] = built ? 1u : 0u;
                 mbar_arrive(bar_built);
             }
             if (!built || !is_long(rtok + L)) {
-                wait_group(1, kLoader, bar_go, ph_go);   // the run ends with this segment
+                wait_go();   // the run ends with this segment
                 return;
             }
             rtok += L;

@@ -17,7 +17,7 @@ namespace hs {
 // (L2 prefetches aside), then releases its own dependents; the tensor-core
 // prefill only waits (see pdl_wait), and as the output pass of the
 // segment-parallel prefill it waits only in the warps that read or write what
-// the kernel before it touches.
+// the kernel before it touches, and in the thread whose bounded wait depends on them.
 __device__ __forceinline__ void pdl_wait_and_release()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -1,6 +1,6 @@
 """Orders that the tensor-core prefill's warps must keep, on the CPU: every interleaving of a
-small model of the hand-over in a run of fast segments, and the order of two tensor-core
-products on the same columns.
+small model of the hand-over in a run of fast segments, the order of two tensor-core products on
+the same columns, and where the time limit of a wait starts.
 
 The hand-over: two builder threads (the loader, which waits and arrives for its group, and any other) and the
 issuing state thread pass the segments on as the kernel's builder_run and state_run do: built ->
@@ -109,3 +109,16 @@ def test_products_on_the_same_columns_have_one_shape():
     assert second == {"TM_O0": "IDT_N64", "TM_S": "Geo<D>::IDT_ST"}
     column = lambda name: int(re.search(rf"constexpr uint32_t {name} = (\d+);", src).group(1))
     assert column("TM_O0") + 64 <= column("TM_S")
+
+
+def test_output_pass_time_limit_starts_after_the_kernel_before():
+    """In the output pass the state warps wait, without a limit, for the scan, while the builders
+    already work.  Every bounded wait of theirs on the state warps (bar_go) follows the loader's own
+    wait for the scan: a slow scan is not reported as a wait that ran out."""
+    kernel = _source("gla_chunked_tc.cu")
+    waits = re.findall(r"(\w+)\(\w+, (?:\w+, )?bar_go, (\w+)\)", kernel)
+    assert sorted(waits) == [("wait_all", "ph_stall"), ("wait_group", "ph_go")]   # the first: a test hook
+    go = kernel[kernel.index("auto wait_go = "):]
+    go = go[:go.index("};")]
+    assert re.search(r"if \(RESTART && tid == kLoader\)\s*pdl_wait\(\);\s*return wait_group\(1, kLoader, bar_go", go)
+    assert kernel.count("wait_go()") == 2
