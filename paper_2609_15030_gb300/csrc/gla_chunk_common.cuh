@@ -237,10 +237,11 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
-// round to tf32 (nearest, ties away from zero) with integer ops; low 13 bits cleared
+// round to tf32 (nearest, ties away from zero) with integer ops; low 13 bits cleared.  A NaN stays
+// one: CUDA's, 0x7FFFFFFF, would carry into the sign and become -0, hiding what the inputs did
 __device__ __forceinline__ float rna_tf32(float x)
 {
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+    return x == x ? __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u) : x;
 }
 
 

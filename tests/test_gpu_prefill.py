@@ -348,6 +348,30 @@ def test_fast_runs_ended_by_magnitude(d, p0, tail):
         assert np.array_equal(S1.view(np.uint32), S.view(np.uint32)), m
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("at", [3, 20, 37])
+@pytest.mark.parametrize("which,bad", [("q", np.nan), ("k", np.nan), ("q", np.inf), ("k", np.inf)])
+def test_exact_segment_shows_non_finite_inputs(which, bad, at, d):
+    """One NaN or infinite element of q or k in an exact segment (head 1): the outputs that the
+    recurrence makes non-finite are not finite (that query's; every one from that key on), and all
+    others follow the oracle.  The key's scores lie in its own 8 x 8 triangle and in squares of
+    every size."""
+    dev = device()
+    n, nH = 64, 2
+    inp = gen_linear(91 + d, 0, 1, n, nH, d, d)
+    inp.a[0, :, :, ::3] = -0.3                       # 64 tokens: far past the fast path's decay
+    S0 = gen_state(5, 0, 1, nH, d, d)
+    ro, _, _ = oracle.gla(inp.q, inp.k, inp.v, inp.a, [0], [n], S0=S0)
+    getattr(inp, which)[0, at, 1, 17:18] = f32_to_bf16_bits(np.array([bad]))
+    o, S, _ = run_prefill(inp, [0], [n], S0, 0, dev, hs.HS_LINATTN_CHUNKED_TC)
+    hit = np.zeros((n, nH), bool)
+    hit[slice(at, at + 1) if which == "q" else slice(at, None), 1] = True
+    assert not np.isfinite(o[0][hit]).any()
+    want, got = np.where(hit[..., None], 0, ro[0]), np.where(hit[..., None], 0, o[0])
+    assert maxnorm_err(got, want, axes=(0, 2)) <= TOL
+    assert np.isfinite(S[0, 0]).all() and np.isfinite(S[0, 1]).all() == (which == "q")
+
+
 @pytest.mark.parametrize("where", ["short_call", "full_segment"])
 def test_zero_gate_inside_an_exact_segment(where):
     """A zero gate (a = -1e4) followed, in the same segment, by growing gates (the exact
