@@ -801,7 +801,8 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 // the builders looking one segment ahead: 22 k cycles a segment, the decays, operands, scores,
 // update and outputs one after another (a segment's exponentials alone are ~2,300 warp
 // instructions, 4.6 k cycles of the special-function units).
-// Segments with a gate above 0 keep the pairwise form (exact_scores_pairs).
+// Segments with a gate above 0 keep the pairwise form (exact_scores_pairs), and segments with a
+// score that comes out infinite or NaN fall back to it.
 
 // a 16 x 16 unit's rows: query rows r0.. and r1.. (8 each), key rows c0.. and c1.., and the
 // tokens R that (r0, c0) and (r1, c1) factor at; units 2 and 3 hold two squares of H = 8, in
@@ -1043,12 +1044,15 @@ __device__ __forceinline__ void exact_zeros(uint8_t *smem)
     }
 }
 
-// the partial sums added up: every score on and below the diagonal, and the triangles' zeros
+// the partial sums added up: every score on and below the diagonal, and the triangles' zeros.
+// Returns whether one of this thread's scores is infinite or NaN.
 template <int D>
-__device__ __forceinline__ void exact_scores_sum(uint8_t *smem)
+__device__ __forceinline__ bool exact_scores_sum(uint8_t *smem)
 {
     const int tid = thread_id();
+    bool bad = false;
     auto put = [&](int i, int j, float a) {
+        bad = bad || !(fabsf(a) < INFINITY);
         *reinterpret_cast<float *>(smem + X_B2 + t_off(Geo<D>::ROWS, i, j)) = rna_tf32(a);
     };
 #pragma unroll
@@ -1077,9 +1081,10 @@ __device__ __forceinline__ void exact_scores_sum(uint8_t *smem)
         }
         put(8 * blk + i, 8 * blk + j, a);
     }
+    return bad;
 }
 
-// pair by pair, for segments with a gate above 0
+// pair by pair, for segments with a gate above 0 or a score that is not finite
 template <int D>
 __device__ __forceinline__ void exact_scores_pairs(uint8_t *smem, int L)
 {
@@ -1145,9 +1150,8 @@ __device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int
         }
         __syncwarp();
     }
-    if (up) {
-        exact_scores_pairs<D>(smem, L);
-    } else {
+    bool pairs = up;
+    if (!up) {
         while (true) {
             int task = 0;
             if ((thread_id() & 31) == 0)
@@ -1158,11 +1162,18 @@ __device__ __forceinline__ void exact_operands(uint8_t *smem, uint32_t tmem, int
             exact_task<D>(smem, task);
         }
         __syncthreads();
-        exact_scores_sum<D>(smem);
+        const bool bad = exact_scores_sum<D>(smem);
+        fence_proxy_async_smem();
+        tc_fence_before();
+        // an infinite q or k has no split into two parts (an infinity less itself is NaN)
+        pairs = __syncthreads_or(bad) != 0;
     }
-    fence_proxy_async_smem();
-    tc_fence_before();
-    __syncthreads();
+    if (pairs) {
+        exact_scores_pairs<D>(smem, L);
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+    }
 }
 
 // (issuing thread) D_O += V^T A^T and S^T += V^T K^ (S^T decayed before), 8 tokens per step.  Two

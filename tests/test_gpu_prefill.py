@@ -355,7 +355,7 @@ def test_exact_segment_shows_non_finite_inputs(which, bad, at, d):
     """One NaN or infinite element of q or k in an exact segment (head 1): the outputs that the
     recurrence makes non-finite are not finite (that query's; every one from that key on), and all
     others follow the oracle.  The key's scores lie in its own 8 x 8 triangle and in squares of
-    every size."""
+    every size.  Where the recurrence gives an infinity, an infinite key gives that one, not NaN."""
     dev = device()
     n, nH = 64, 2
     inp = gen_linear(91 + d, 0, 1, n, nH, d, d)
@@ -367,6 +367,10 @@ def test_exact_segment_shows_non_finite_inputs(which, bad, at, d):
     hit = np.zeros((n, nH), bool)
     hit[slice(at, at + 1) if which == "q" else slice(at, None), 1] = True
     assert not np.isfinite(o[0][hit]).any()
+    if (which, bad) == ("k", np.inf):
+        bad_o, _, _ = oracle.gla(inp.q, inp.k, inp.v, inp.a, [0], [n], S0=S0)
+        assert np.isinf(bad_o[0][hit]).all()
+        assert np.array_equal(o[0][hit], bad_o[0][hit].astype(np.float32))
     want, got = np.where(hit[..., None], 0, ro[0]), np.where(hit[..., None], 0, o[0])
     assert maxnorm_err(got, want, axes=(0, 2)) <= TOL
     assert np.isfinite(S[0, 0]).all() and np.isfinite(S[0, 1]).all() == (which == "q")
