@@ -790,8 +790,8 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 // factors at the token R that ends the block's first half, 2^{Lam_i - Lam_j} =
 // 2^{Lam_i - Lam_R} 2^{Lam_R - Lam_j} with j <= R < i, so both exponents are <= 0: no overflow,
 // and a factor that underflows stands for a product that does.  The factors are formed in
-// registers as matrix fragments and split into two tf32 parts each, so that a product keeps
-// ~2^-21 (three tf32 products, float32 sums).  The eight 8 x 8 triangles left on the diagonal
+// registers as matrix fragments and split into two tf32 parts each, three tf32 products for one
+// (see squares_mma).  The eight 8 x 8 triangles left on the diagonal
 // are taken pair by pair.  The tasks (one warp each, drawn from a shared counter, the long ones
 // first) are halves of the key dims of four 16 x 16 units (a square of H = 16, or two of H = 8),
 // quarters of those of each half of the 32 x 32 square, and 64 key dims of a triangle.  Meanwhile the
@@ -828,19 +828,26 @@ constexpr uint32_t X_P32 = OFF_SG;             // 32 x 32 square [4 quarters][32
 constexpr uint32_t X_P16 = OFF_SG + 16384;     // units [4][2 halves][16][16]              8 KiB
 constexpr uint32_t X_PTR = OFF_SG + 24576;     // triangles [8][d / 64][40]              2.5 KiB
 
-// four factors x 2^{+-(l - lr)} of one row (key dims kk..kk+3), x in bf16, lr given
+// four factors x 2^{+-(l - lr)} of one row (key dims kk..kk+3): x in bf16 and the powers, lr given
+struct Factors {
+    uint2 w;
+    float e[4];
+
+    __device__ __forceinline__ float x(int i) const
+    {
+        const uint32_t u = i < 2 ? w.x : w.y;
+        return __uint_as_float((i & 1) ? u & 0xFFFF0000u : u << 16);
+    }
+};
+
 template <int D, int SIGN>
-__device__ __forceinline__ void factors4(const uint8_t *smem, uint32_t off, int row, const float4 &r,
-                                         int kk, float *y)
+__device__ __forceinline__ Factors factors4(const uint8_t *smem, uint32_t off, int row, const float4 &r, int kk)
 {
     const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
-    const uint2 w = *reinterpret_cast<const uint2 *>(smem + off + (row * D + kk) * 2);
     const float4 l = *reinterpret_cast<const float4 *>(sLam + lam_at<D>(row, kk));
     const float s = (float)SIGN;
-    y[0] = __uint_as_float(w.x << 16) * ex2(s * (l.x - r.x));
-    y[1] = __uint_as_float(w.x & 0xFFFF0000u) * ex2(s * (l.y - r.y));
-    y[2] = __uint_as_float(w.y << 16) * ex2(s * (l.z - r.z));
-    y[3] = __uint_as_float(w.y & 0xFFFF0000u) * ex2(s * (l.w - r.w));
+    return {*reinterpret_cast<const uint2 *>(smem + off + (row * D + kk) * 2),
+            {ex2(s * (l.x - r.x)), ex2(s * (l.y - r.y)), ex2(s * (l.z - r.z)), ex2(s * (l.w - r.w))}};
 }
 
 template <int D>
@@ -850,38 +857,45 @@ __device__ __forceinline__ float4 lam4(const uint8_t *smem, int row, int kk)
                                              lam_at<D>(row, kk));
 }
 
-// MT x NT tiles of 16 x 8 scores += fragments a (rows g and g + 8 of each tile) and b, each four
-// consecutive key dims per lane: a k step of the products takes two of them (any assignment
-// of key dims to k will do, as long as both operands share it)
-template <int MT, int NT8>
-__device__ __forceinline__ void squares_mma(float (&acc)[MT][NT8][4], const float (&a)[2 * MT][4],
-                                            const float (&b)[NT8][4])
+// NT8 tiles of 16 x 8 scores += fragments a (rows g and g + 8) and b, each four consecutive key dims
+// per lane: a k step of the products takes two of them (any assignment of key dims to k will
+// do, as long as both operands share it).  The matrix instruction truncates its sums, so each
+// step's three products have an accumulator of their own, which float32 additions (to nearest)
+// collect.  Root mean square error of cancelling scores relative to the sum of their terms'
+// magnitudes: 1.7e-8 at d = 128 and 2.3e-8 at d = 64 (taken pair by pair 2.0e-8 and 2.3e-8); with
+// parts split by truncation and one accumulator throughout 4.1e-8 and 4.9e-8, at 87.5 us instead of
+// 90.6 for tails of 475 tokens of 9 x 16 heads.
+template <int NT8>
+__device__ __forceinline__ void squares_mma(float (&acc)[NT8][4], const Factors (&a)[2],
+                                            const Factors (&b)[NT8])
 {
 #pragma unroll
     for (int x = 0; x < 4; x += 2) {
-        uint32_t bh[NT8][2], bl[NT8][2];
+        uint32_t ah[4], al[4], bh[NT8][2], bl[NT8][2];
+        float c[NT8][4];
 #pragma unroll
         for (int n = 0; n < NT8; ++n) {
-            split_tf32(b[n][x], bh[n][0], bl[n][0]);
-            split_tf32(b[n][x + 1], bh[n][1], bl[n][1]);
+            split_tf32(b[n].x(x), b[n].e[x], bh[n][0], bl[n][0]);
+            split_tf32(b[n].x(x + 1), b[n].e[x + 1], bh[n][1], bl[n][1]);
         }
+        split_tf32(a[0].x(x), a[0].e[x], ah[0], al[0]);
+        split_tf32(a[1].x(x), a[1].e[x], ah[1], al[1]);
+        split_tf32(a[0].x(x + 1), a[0].e[x + 1], ah[2], al[2]);
+        split_tf32(a[1].x(x + 1), a[1].e[x + 1], ah[3], al[3]);
 #pragma unroll
-        for (int m = 0; m < MT; ++m) {
-            uint32_t ah[4], al[4];
-            split_tf32(a[2 * m][x], ah[0], al[0]);
-            split_tf32(a[2 * m + 1][x], ah[1], al[1]);
-            split_tf32(a[2 * m][x + 1], ah[2], al[2]);
-            split_tf32(a[2 * m + 1][x + 1], ah[3], al[3]);
+        for (int n = 0; n < NT8; ++n)
+            mma_m16n8k8_tf32_new(c[n], al, bh[n]);
 #pragma unroll
-            for (int n = 0; n < NT8; ++n)
-                mma_m16n8k8_tf32(acc[m][n], al, bh[n]);
+        for (int n = 0; n < NT8; ++n)
+            mma_m16n8k8_tf32(c[n], ah, bl[n]);
 #pragma unroll
-            for (int n = 0; n < NT8; ++n)
-                mma_m16n8k8_tf32(acc[m][n], ah, bl[n]);
+        for (int n = 0; n < NT8; ++n)
+            mma_m16n8k8_tf32(c[n], ah, bh[n]);
 #pragma unroll
-            for (int n = 0; n < NT8; ++n)
-                mma_m16n8k8_tf32(acc[m][n], ah, bh[n]);
-        }
+        for (int n = 0; n < NT8; ++n)
+#pragma unroll
+            for (int y = 0; y < 4; ++y)
+                acc[n][y] += c[n][y];
     }
 }
 
@@ -891,25 +905,25 @@ template <int D>
 __device__ __forceinline__ void exact_square32(uint8_t *smem, int mh, int quarter)
 {
     const int lane = thread_id() & 31, g = lane >> 2, t = lane & 3;
-    float acc[1][4][4] = {};
+    float acc[4][4] = {};
 #pragma unroll 1
     for (int k0 = quarter * (D / 4); k0 < (quarter + 1) * (D / 4); k0 += 16) {
         const int kk = k0 + 4 * t;
         const float4 r = lam4<D>(smem, 31, kk);
-        float a[2][4], b[4][4];
+        Factors a[2], b[4];
 #pragma unroll
         for (int x = 0; x < 2; ++x)
-            factors4<D, 1>(smem, OFF_SQ, 32 + 16 * mh + 8 * x + g, r, kk, a[x]);
+            a[x] = factors4<D, 1>(smem, OFF_SQ, 32 + 16 * mh + 8 * x + g, r, kk);
 #pragma unroll
         for (int x = 0; x < 4; ++x)
-            factors4<D, -1>(smem, OFF_SK, 8 * x + g, r, kk, b[x]);
-        squares_mma<1, 4>(acc, a, b);
+            b[x] = factors4<D, -1>(smem, OFF_SK, 8 * x + g, r, kk);
+        squares_mma<4>(acc, a, b);
     }
     float *dst = reinterpret_cast<float *>(smem + X_P32) + quarter * 1024 + (16 * mh + g) * 32 + 2 * t;
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-        *reinterpret_cast<float2 *>(dst + 8 * n) = make_float2(acc[0][n][0], acc[0][n][1]);
-        *reinterpret_cast<float2 *>(dst + 8 * 32 + 8 * n) = make_float2(acc[0][n][2], acc[0][n][3]);
+        *reinterpret_cast<float2 *>(dst + 8 * n) = make_float2(acc[n][0], acc[n][1]);
+        *reinterpret_cast<float2 *>(dst + 8 * 32 + 8 * n) = make_float2(acc[n][2], acc[n][3]);
     }
 }
 
@@ -919,28 +933,28 @@ __device__ __forceinline__ void exact_square16(uint8_t *smem, int u, int half)
 {
     const int lane = thread_id() & 31, g = lane >> 2, t = lane & 3;
     const SquareUnit m = square_unit(u);
-    float acc[1][2][4] = {};
+    float acc[2][4] = {};
 #pragma unroll 1
     for (int k0 = half * (D / 2); k0 < (half + 1) * (D / 2); k0 += 32) {
-        float a[2][2][4], b[2][2][4];
+        Factors a[2][2], b[2][2];
 #pragma unroll
         for (int y = 0; y < 2; ++y) {
             const int kk = k0 + 16 * y + 4 * t;
             const float4 ra = lam4<D>(smem, m.ref0, kk), rb = lam4<D>(smem, m.ref1, kk);
-            factors4<D, 1>(smem, OFF_SQ, m.r0 + g, ra, kk, a[y][0]);
-            factors4<D, 1>(smem, OFF_SQ, m.r1 + g, rb, kk, a[y][1]);
-            factors4<D, -1>(smem, OFF_SK, m.c0 + g, ra, kk, b[y][0]);
-            factors4<D, -1>(smem, OFF_SK, m.c1 + g, rb, kk, b[y][1]);
+            a[y][0] = factors4<D, 1>(smem, OFF_SQ, m.r0 + g, ra, kk);
+            a[y][1] = factors4<D, 1>(smem, OFF_SQ, m.r1 + g, rb, kk);
+            b[y][0] = factors4<D, -1>(smem, OFF_SK, m.c0 + g, ra, kk);
+            b[y][1] = factors4<D, -1>(smem, OFF_SK, m.c1 + g, rb, kk);
         }
-        squares_mma<1, 2>(acc, a[0], b[0]);
-        squares_mma<1, 2>(acc, a[1], b[1]);
+        squares_mma<2>(acc, a[0], b[0]);
+        squares_mma<2>(acc, a[1], b[1]);
     }
     float *dst = reinterpret_cast<float *>(smem + X_P16) + (2 * u + half) * 256;
 #pragma unroll
     for (int n = 0; n < 2; ++n) {
         float *p = dst + g * 16 + 8 * n + 2 * t;
-        *reinterpret_cast<float2 *>(p) = make_float2(acc[0][n][0], acc[0][n][1]);
-        *reinterpret_cast<float2 *>(p + 8 * 16) = make_float2(acc[0][n][2], acc[0][n][3]);
+        *reinterpret_cast<float2 *>(p) = make_float2(acc[n][0], acc[n][1]);
+        *reinterpret_cast<float2 *>(p + 8 * 16) = make_float2(acc[n][2], acc[n][3]);
     }
 }
 

@@ -306,12 +306,20 @@ __device__ __forceinline__ void tmem_wait_st()
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-// x as two tf32 parts: hi = x with the low 13 mantissa bits cleared (exact), lo = x - hi
-// (exact in fp32; the products read its leading 11 bits)
-__device__ __forceinline__ void split_tf32(float x, uint32_t &hi, uint32_t &lo)
+// round to tf32 (nearest, ties away from zero; infinities and NaN stay)
+__device__ __forceinline__ uint32_t cvt_tf32(float x)
 {
-    hi = __float_as_uint(x) & 0xFFFFE000u;
-    lo = __float_as_uint(x - __uint_as_float(hi));
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return r;
+}
+
+// x * y as two tf32 parts, each rounded to nearest: hi, and lo = x y - hi (one fma), so that hi + lo
+// is x y to 2^-24.  Of an infinity or a NaN lo is NaN, and so is every product with it.
+__device__ __forceinline__ void split_tf32(float x, float y, uint32_t &hi, uint32_t &lo)
+{
+    hi = cvt_tf32(x * y);
+    lo = cvt_tf32(fmaf(x, y, -__uint_as_float(hi)));
 }
 
 // c += a * b on one warp, 16 x 8 x 8, tf32 operands, fp32 accumulators (lane = 4 g + t:
@@ -325,6 +333,17 @@ __device__ __forceinline__ void mma_m16n8k8_tf32(float (&c)[4], const uint32_t (
         "{%0,%1,%2,%3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// c = a * b, the same
+__device__ __forceinline__ void mma_m16n8k8_tf32_new(float (&c)[4], const uint32_t (&a)[4],
+                                                     const uint32_t (&b)[2])
+{
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%10,%10,%10,%10};"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
 }
 
 }  // namespace ptx

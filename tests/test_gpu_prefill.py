@@ -348,6 +348,66 @@ def test_fast_runs_ended_by_magnitude(d, p0, tail):
         assert np.array_equal(S1.view(np.uint32), S.view(np.uint32)), m
 
 
+def _cancelling_scores(d, seed=0):
+    """One 64-token exact segment of 62 heads: head h has a value (1 in every column) at token h
+    only, so that its later outputs are its scores A_ih themselves; every later query is moved
+    until that score cancels to less than 2^-13 of the sum of its terms' magnitudes.  Returns the
+    inputs, the scores in float64 and those sums (zeros up to the key)."""
+    nH, n = 62, 64
+    inp = gen_linear(7 + d, seed, 1, n, nH, d, d)
+    rng = np.random.default_rng([d, seed])
+    inp.a[0] = rng.uniform(-0.05, 0.0, size=(n, nH, d))
+    inp.a[0, 63] = -8.0                              # past the fast path's total decay
+    inp.v[:] = 0
+    lam = np.cumsum(inp.a[0].astype(np.float64), axis=0)
+    ref, mag = np.zeros((n, nH)), np.zeros((n, nH))
+    for h in range(nH):
+        inp.v[0, h, h] = f32_to_bf16_bits(np.ones(d))
+        k = bf16_bits_to_f32(inp.k[0, h, h]).astype(np.float64)
+        kw = k * np.exp(lam[h + 1:, h] - lam[h, h])
+        q = bf16_bits_to_f32(inp.q[0, h + 1:, h]).astype(np.float64)
+        q -= ((q * kw).sum(-1) / (kw * kw).sum(-1))[:, None] * kw
+        bits, rows, unit = f32_to_bf16_bits(q), np.arange(63 - h), np.array([1, 65535], np.uint16)
+        for _ in range(12):                          # one unit in the last place of one element a step
+            val = lambda b: bf16_bits_to_f32(b).astype(np.float64) * kw
+            left = val(bits).sum(-1)
+            moved = np.stack([left[:, None] + val(bits + u) - val(bits) for u in unit])
+            pick = np.abs(moved).transpose(1, 2, 0).reshape(63 - h, -1).argmin(-1)
+            better = np.abs(moved[pick % 2, rows, pick // 2]) < np.abs(left)
+            bits[rows, pick // 2] += np.where(better, unit[pick % 2], 0).astype(np.uint16)
+        inp.q[0, h + 1:, h] = bits
+        ref[h + 1:, h], mag[h + 1:, h] = val(bits).sum(-1), np.abs(val(bits)).sum(-1)
+    assert (np.abs(ref) <= 2.0 ** -13 * mag).all()
+    return inp, ref, mag
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_factored_scores_are_as_exact_as_pairwise_ones(d):
+    """The exact path's scores off the 8 x 8 triangles are products of two scaled factors, each in
+    two tf32 parts; with a gate above 0 they are float32 sums pair by pair instead.  On scores that
+    cancel (their rounding to tf32 afterwards is below 2^-25 of the terms' magnitudes) the root
+    mean square error of the first must not exceed that of the second, in the squares of each
+    size: a ratio of 1.2 is three standard deviations of the smallest sample (1,024 scores, 0.06)
+    above equality.  One tf32 product per term would be 3,000 times off, parts split by truncation
+    twice.  A positive gate at token 0 decays no pair: it only chooses the form."""
+    dev = device()
+    err = {}
+    for seed in range(4):
+        inp, ref, mag = _cancelling_scores(d, seed)
+        i, j = np.indices(ref.shape)
+        for form, gate in (("factored", -0.01), ("pairwise", 0.01)):
+            inp.a[0, 0] = gate
+            o, _, _ = run_prefill(inp, [0], [64], None, 0, dev, hs.HS_LINATTN_CHUNKED_TC)
+            assert np.array_equal(o[0], np.broadcast_to(o[0][..., :1], o[0].shape))
+            e = (o[0, ..., 0] - ref) / np.where(mag == 0, 1, mag)
+            for half in (32, 16, 8):                 # the squares of this size
+                at = (i > j) & (i // half != j // half) & (i // (2 * half) == j // (2 * half))
+                err.setdefault((half, form), []).append((e[at] ** 2).mean())
+    for half in (32, 16, 8):
+        rms = [np.sqrt(np.mean(err[half, form])) for form in ("factored", "pairwise")]
+        assert 0 < rms[0] <= 1.2 * rms[1], (half, rms)
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("at", [3, 20, 37])
 @pytest.mark.parametrize("which,bad", [("q", np.nan), ("k", np.nan), ("q", np.inf), ("k", np.inf)])
