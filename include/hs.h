@@ -262,8 +262,8 @@ typedef enum hs_linattn_kernel {
     HS_LINATTN_CHUNKED_TC = 2, /* chunked form on tcgen05 tensor cores (d_k == d_v, 64 or
                                   128; at 64 the M = 128 products leave half their TMEM lanes
                                   unused) */
-    HS_LINATTN_SINGLE_TOKEN = 3 /* one decode step per problem, state in registers, no
-                                  shared memory (HS_ERR_UNSUPPORTED if some n_tokens > 1) */
+    HS_LINATTN_SINGLE_TOKEN = 3 /* one decode step per problem, state in registers
+                                  (HS_ERR_UNSUPPORTED if some n_tokens > 1) */
 } hs_linattn_kernel;
 
 typedef struct hs_linattn_shape {
@@ -321,10 +321,11 @@ typedef struct hs_linattn_shape {
  * token.  The tensor-core kernel runs a chunk on fp16 operands (11 significant
  * bits, float32 accumulation and state) when its log-gates are <= 0, its total
  * log2-decay stays >= -10 in every key dimension and every operand provably fits
- * fp16; any other chunk runs on tf32 operands with the intra-chunk scores computed
- * in float32.  On both paths a token's own score A_ii = q_i . k_i is summed in
- * float32 from the bf16 inputs, so operand rounding enters only through the
- * products of different tokens and through the state.  Per output element,
+ * fp16; any other chunk runs on tf32 operands with the intra-chunk scores as exact
+ * as float32 sums before their rounding to tf32.  On both paths a token's own score
+ * A_ii = q_i . k_i is summed in float32 from the bf16 inputs, so operand rounding
+ * enters only through the products of different tokens and through the state.  Per
+ * output element,
  * with eps = 2^-11 and Q~ = q 2^Lam, K~ = k 2^-Lam the decayed operands of the
  * chunk, the error is at most about
  *   2 eps (sum_d |Q~_id| |S_de| + sum_{j<i} |v_je| sum_d |Q~_id K~_jd|)
@@ -334,6 +335,10 @@ typedef struct hs_linattn_shape {
  * magnitudes are within about 1,000 times of it: over 3,000 seeded stress calls
  * (tails up to 600 tokens, v scaled by 2^17, q and k by 64, gates of -30, -1.2,
  * -1e4 and +0.02, states up to 2^16) the largest max-normalised error was 5.6e-4.
+ * Inputs should be finite.  Where a NaN or an infinity in q or k makes an output of
+ * the recurrence non-finite, that output is not finite here either (NaN possibly in
+ * place of an infinity); one in v may also reach earlier outputs of its chunk in its
+ * own column, and a NaN log-gate may act as a zero gate.
  * All of q, k, v, log_g, o, state must be 16-byte aligned.  q/k/v/log_g are only
  * read; o, state and the slots must not overlap the inputs or each other.
  * Token rows are 32-bit: b*max_tokens + n_tokens[b] must stay below 2^31.

@@ -196,69 +196,70 @@ def hs_align_prefix(N: int, hit_len: int, avail, page_size: int):
     """Strict-prefix alignment; returns (c, n_pages, tail)."""
     av = (C.c_int64 * len(avail))(*[int(a) for a in avail]) if len(avail) else None
     c, npg, tail = C.c_int64(), C.c_int64(), C.c_int64()
-    rc = (_lib or load()).hs_align_prefix(int(N), int(hit_len), C.cast(av, C.c_void_p) if av else None,
-                                len(avail), int(page_size), C.addressof(c), C.addressof(npg),
-                                C.addressof(tail))
+    rc = (_lib or load()).hs_align_prefix(
+        int(N), int(hit_len), C.cast(av, C.c_void_p) if av else None, len(avail), int(page_size),
+        C.addressof(c), C.addressof(npg), C.addressof(tail))
     _check(rc, "hs_align_prefix")
     return c.value, npg.value, tail.value
 
 
 def hs_restore_kv_pages(staging_layers, cache_layers, n_layers: int, block_table, n_pages: int,
                         page_bytes: int, num_blocks: int, d_err=None, stream=None):
-    rc = (_lib or load()).hs_restore_kv_pages(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
-                                    _ptr(block_table), int(n_pages), int(page_bytes),
-                                    int(num_blocks), _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_restore_kv_pages(
+        _ptr(staging_layers), _ptr(cache_layers), int(n_layers), _ptr(block_table), int(n_pages),
+        int(page_bytes), int(num_blocks), _ptr(d_err), _stream(stream))
     _check(rc, "hs_restore_kv_pages")
 
 
 def hs_restore_request(staging_layers, cache_layers, n_layers: int, block_table, n_pages: int,
                        page_bytes: int, num_blocks: int, src_slots, dst_slots, n_slots: int,
                        floats_each: int, d_err=None, stream=None):
-    rc = (_lib or load()).hs_restore_request(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
-                                   _ptr(block_table), int(n_pages), int(page_bytes),
-                                   int(num_blocks), _ptr(src_slots), _ptr(dst_slots), int(n_slots),
-                                   int(floats_each), _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_restore_request(
+        _ptr(staging_layers), _ptr(cache_layers), int(n_layers), _ptr(block_table), int(n_pages),
+        int(page_bytes), int(num_blocks), _ptr(src_slots), _ptr(dst_slots), int(n_slots),
+        int(floats_each), _ptr(d_err), _stream(stream))
     _check(rc, "hs_restore_request")
 
 
 def hs_save_kv_pages(cache_layers, staging_layers, n_layers: int, block_table, n_pages: int,
                      page_bytes: int, num_blocks: int, d_err=None, stream=None):
-    rc = (_lib or load()).hs_save_kv_pages(_ptr(cache_layers), _ptr(staging_layers), int(n_layers),
-                                 _ptr(block_table), int(n_pages), int(page_bytes),
-                                 int(num_blocks), _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_save_kv_pages(
+        _ptr(cache_layers), _ptr(staging_layers), int(n_layers), _ptr(block_table), int(n_pages),
+        int(page_bytes), int(num_blocks), _ptr(d_err), _stream(stream))
     _check(rc, "hs_save_kv_pages")
 
 
 def hs_restore_kv_page_slices(staging_layers, cache_layers, n_layers: int, block_table,
                               n_pages: int, page_bytes: int, rows: int, col_off: int,
                               col_bytes: int, num_blocks: int, d_err=None, stream=None):
-    rc = (_lib or load()).hs_restore_kv_page_slices(_ptr(staging_layers), _ptr(cache_layers), int(n_layers),
-                                          _ptr(block_table), int(n_pages), int(page_bytes),
-                                          int(rows), int(col_off), int(col_bytes), int(num_blocks),
-                                          _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_restore_kv_page_slices(
+        _ptr(staging_layers), _ptr(cache_layers), int(n_layers), _ptr(block_table), int(n_pages),
+        int(page_bytes), int(rows), int(col_off), int(col_bytes), int(num_blocks), _ptr(d_err),
+        _stream(stream))
     _check(rc, "hs_restore_kv_page_slices")
 
 
 def hs_save_kv_page_slices(cache_layers, staging_layers, n_layers: int, block_table, n_pages: int,
                            page_bytes: int, rows: int, col_off: int, col_bytes: int,
                            num_blocks: int, d_err=None, stream=None):
-    rc = (_lib or load()).hs_save_kv_page_slices(_ptr(cache_layers), _ptr(staging_layers), int(n_layers),
-                                       _ptr(block_table), int(n_pages), int(page_bytes),
-                                       int(rows), int(col_off), int(col_bytes), int(num_blocks),
-                                       _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_save_kv_page_slices(
+        _ptr(cache_layers), _ptr(staging_layers), int(n_layers), _ptr(block_table), int(n_pages),
+        int(page_bytes), int(rows), int(col_off), int(col_bytes), int(num_blocks), _ptr(d_err),
+        _stream(stream))
     _check(rc, "hs_save_kv_page_slices")
 
 
 def hs_restore_state(src_slots, dst_slots, n: int, floats_each: int, d_err=None, stream=None):
-    rc = (_lib or load()).hs_restore_state(_ptr(src_slots), _ptr(dst_slots), int(n), int(floats_each),
-                                 _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_restore_state(
+        _ptr(src_slots), _ptr(dst_slots), int(n), int(floats_each), _ptr(d_err), _stream(stream))
     _check(rc, "hs_restore_state")
 
 
 def hs_checkpoint_states(live_states, ckpt_slots, n: int, floats_each: int, d_err=None,
                          stream=None):
-    rc = (_lib or load()).hs_checkpoint_states(_ptr(live_states), _ptr(ckpt_slots), int(n),
-                                     int(floats_each), _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_checkpoint_states(
+        _ptr(live_states), _ptr(ckpt_slots), int(n), int(floats_each), _ptr(d_err),
+        _stream(stream))
     _check(rc, "hs_checkpoint_states")
 
 
@@ -272,9 +273,9 @@ def _prefill_call(name, shape, q, k, v, log_g, o, state, pos0, n_tokens, ckpt_in
     B = int(shape.batch)
     p0, keep_p0 = _i64(pos0, B)
     nt, keep_nt = _i32(n_tokens, B)
-    rc = getattr(_lib or load(), name)(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o),
-                               _ptr(state), p0, nt, int(ckpt_interval),
-                               _ptr(ckpt_slots), _ptr(d_err), _stream(stream))
+    rc = getattr(_lib or load(), name)(
+        C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o), _ptr(state), p0, nt,
+        int(ckpt_interval), _ptr(ckpt_slots), _ptr(d_err), _stream(stream))
     _check(rc, name)
 
 
@@ -300,8 +301,8 @@ def hs_linattn_scan_workspace_bytes(shape: hs_linattn_shape, pos0, n_tokens) -> 
     p0, keep_p0 = _i64(pos0, B)
     nt, keep_nt = _i32(n_tokens, B)
     out = C.c_int64()
-    rc = (_lib or load()).hs_linattn_scan_workspace_bytes(C.byref(shape), p0, nt,
-                                                C.addressof(out))
+    rc = (_lib or load()).hs_linattn_scan_workspace_bytes(
+        C.byref(shape), p0, nt, C.addressof(out))
     _check(rc, "hs_linattn_scan_workspace_bytes")
     return out.value
 
@@ -314,10 +315,10 @@ def hs_linattn_prefill_scan(shape: hs_linattn_shape, q, k, v, log_g, o, state, p
     B = int(shape.batch)
     p0, keep_p0 = _i64(pos0, B)
     nt, keep_nt = _i32(n_tokens, B)
-    rc = (_lib or load()).hs_linattn_prefill_scan(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g),
-                                        _ptr(o), _ptr(state), p0, nt,
-                                        int(ckpt_interval), _ptr(ckpt_slots), _ptr(workspace),
-                                        int(workspace_bytes), _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_linattn_prefill_scan(
+        C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o), _ptr(state), p0, nt,
+        int(ckpt_interval), _ptr(ckpt_slots), _ptr(workspace), int(workspace_bytes), _ptr(d_err),
+        _stream(stream))
     _check(rc, "hs_linattn_prefill_scan")
 
 
@@ -333,11 +334,9 @@ def hs_linattn_prefill_scan_noalloc(shape: hs_linattn_shape, q, k, v, log_g, o, 
     B = int(shape.batch)
     p0, keep_p0 = _i64(pos0, B)
     nt, keep_nt = _i32(n_tokens, B)
-    rc = (_lib or load()).hs_linattn_prefill_scan_noalloc(C.byref(shape), _ptr(q), _ptr(k), _ptr(v),
-                                                _ptr(log_g), _ptr(o), _ptr(state),
-                                                p0, nt,
-                                                int(ckpt_interval), _ptr(ckpt_slots),
-                                                _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_linattn_prefill_scan_noalloc(
+        C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o), _ptr(state), p0, nt,
+        int(ckpt_interval), _ptr(ckpt_slots), _ptr(d_err), _stream(stream))
     _check(rc, "hs_linattn_prefill_scan_noalloc")
 
 
@@ -350,10 +349,9 @@ def hs_linattn_prefill_packed(shape: hs_linattn_shape, q, k, v, log_g, o, state,
     p0, keep_p0 = _i64(pos0, B)
     nt, keep_nt = _i32(n_tokens, B)
     cu, keep_cu = _i64(cu_rows, B + 1)
-    rc = (_lib or load()).hs_linattn_prefill_packed(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g),
-                                          _ptr(o), _ptr(state), p0, nt,
-                                          cu, int(ckpt_interval), _ptr(ckpt_slots),
-                                          _ptr(d_err), _stream(stream))
+    rc = (_lib or load()).hs_linattn_prefill_packed(
+        C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(log_g), _ptr(o), _ptr(state), p0, nt, cu,
+        int(ckpt_interval), _ptr(ckpt_slots), _ptr(d_err), _stream(stream))
     _check(rc, "hs_linattn_prefill_packed")
 
 
@@ -362,7 +360,7 @@ def hs_linattn_num_checkpoints(pos0, n_tokens, ckpt_interval: int) -> int:
     p0, keep_p0 = _i64(pos0, B)
     nt, keep_nt = _i32(n_tokens, B)
     tot = C.c_int64()
-    rc = (_lib or load()).hs_linattn_num_checkpoints(B, p0, nt, int(ckpt_interval),
-                                           C.addressof(tot))
+    rc = (_lib or load()).hs_linattn_num_checkpoints(
+        B, p0, nt, int(ckpt_interval), C.addressof(tot))
     _check(rc, "hs_linattn_num_checkpoints")
     return tot.value

@@ -28,8 +28,9 @@ constexpr int NW = 256;   // state warps (warps 8..15): state passes, masks, epi
 constexpr int NT = NB + NW;
 constexpr int kLoader = 0;   // the first builder thread issues the copies outside a run of fast
                              // segments; inside one a lane of warp 1 does
-constexpr int kIssuer = NB + 64;  // the state thread that issues every MMA but D_A: in a warp of
-                                  // TMEM lane quarter 2, which has no part in the masking of A
+constexpr int kIssuer = NB + 64;  // the state thread that waits and arrives for its group; its warp's
+                                  // elected lane issues every MMA.  In TMEM lane quarter 2, which
+                                  // has no part in the masking of A
 constexpr int kShort = 8; // segments of at most this many tokens run token by token
 constexpr float kLog2e = 1.4426950408889634f;
 // exact path: log-gates below this are taken at this value.  2^(kGateFloor * log2 e) = 2^-144
@@ -65,7 +66,7 @@ constexpr uint32_t S_QH = 0;            //   Q~  fp16 [64 tok i][D]             
 constexpr uint32_t S_KH = 16384;        //   K~  fp16 [64 tok j][D]                     16 KiB
 constexpr uint32_t S_AH = 32768;        //   A   fp16 [64 tok i][64 tok j]                8 KiB
 constexpr uint32_t X_QT = 0;            // exact path (over the sets): Q~ tf32 [64][D]         32 KiB
-constexpr uint32_t X_LAM = 32768;       //   Lam f32 [64 tok][D], row-major                     32 KiB
+constexpr uint32_t X_LAM = 32768;       //   Lam f32 [64 tok][D] (see lam_at)                    32 KiB
 constexpr uint32_t X_B2 = 65536;        //   [A ; K^^T] tf32 [64 i + D][64 tok j]               48 KiB
 constexpr uint32_t OFF_SQ = 122880;     // staged q  bf16 [64][D]                  16 KiB
 constexpr uint32_t OFF_SK = 139264;     // staged k                                 16 KiB
@@ -76,7 +77,7 @@ constexpr uint32_t OFF_TOT = 223232;    // partial log2-decay totals [token grou
 constexpr uint32_t OFF_RED = 225280;    // three sets of [8 warps][8]: builders' max |q|, fast-path
                                         //   flag, max |k|, max |v| (0..3; with the operand sets);
                                         //   state warps' max |S| (4; two sets, a pass each in turn)
-constexpr uint32_t OFF_BAR = 226048;    // 7 mbarriers
+constexpr uint32_t OFF_BAR = 226048;    // 6 mbarriers
 constexpr uint32_t OFF_MISC = 226112;   // TMEM base address, abort flag, decision, run result
 constexpr uint32_t OFF_DG = 226176;     // diagonal of A in float32, with the operand sets:
                                         //   [set][key-dim half][64 tokens] partial sums  1.5 KiB
@@ -300,10 +301,11 @@ __device__ __forceinline__ void zero_tail(uint8_t *smem, int L, int vb, bool bui
 // it writes Q~ and K~ (token-major), fp16, with 4-byte stores.  Its two key dims are a register
 // pair: their sums and products are f32x2 instructions, the roundings those of the scalar ones
 // (with the state pass's decay: 4 x 32 heads of 16,384 tokens 957.5 us, now 950).  Per warp:
-// max |q|, |k| and per thread whether its operands fit fp16 (for the guard).  The diagonal A_ii = q_i . k_i (no decay between a token and itself)
-// is summed in float32 from the bf16 inputs, each warp's 64 key dims by a butterfly, into
-// the set's diagonal partials: fp16 Q~ and K~ would round the terms of that dot product to
-// 11 bits, which a token whose own q . k cancels cannot afford.
+// max |q|, |k| and per thread whether its operands fit fp16 (for the guard).  The diagonal
+// A_ii = q_i . k_i (no decay between a token and itself) is summed in float32 from the bf16
+// inputs, each warp's 64 key dims by a butterfly, into the set's diagonal partials: fp16 Q~ and K~
+// would round the terms of that dot product to 11 bits, which a token whose own q . k cancels
+// cannot afford.
 //
 // A segment that the guard is sure to send to the exact path for its gates alone (one above
 // 0, or a total log2-decay below -kLamRange) stops after the totals and returns false: the
@@ -781,15 +783,15 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
     tmem_wait_st();
 }
 
-// ---- exact path: A_ij = sum_d q_id k_jd 2^{Lam_id - Lam_jd}, j <= i < L, in float32, rounded
-// to tf32 into rows 0..63 of X_B2 (zeros above the diagonal).
+// ---- exact path: A_ij = sum_d q_id k_jd 2^{Lam_id - Lam_jd}, j <= i < L, as exact as float32 sums
+// over pairs, then rounded to tf32 into rows 0..63 of X_B2 (zeros above the diagonal).
 //
 // Taken pair by pair that is 262,144 exponentials at d = 128 and, with one thread per pair, a
 // 32-way bank conflict on every operand.  When no gate is above 0 the 64 x 64 triangle is cut
 // in halves instead: the lower left H x H square of every block of 2 H tokens (H = 32, 16, 8)
 // factors at the token R that ends the block's first half, 2^{Lam_i - Lam_j} =
 // 2^{Lam_i - Lam_R} 2^{Lam_R - Lam_j} with j <= R < i, so both exponents are <= 0: no overflow,
-// and a factor that underflows stands for a product that does.  The factors are formed in
+// and a power that underflows stands for a power 2^{Lam_i - Lam_j} that does.  The factors are formed in
 // registers as matrix fragments and split into two tf32 parts each, three tf32 products for one
 // (see squares_mma).  The eight 8 x 8 triangles left on the diagonal
 // are taken pair by pair.  The tasks (one warp each, drawn from a shared counter, the long ones
@@ -798,8 +800,9 @@ __device__ __forceinline__ void exact_split_state(const uint8_t *smem, uint32_t 
 // issuing thread's warp feeds S^T Q~^T to the tensor core, a chain of dependent products under the
 // tasks.  Tails of 475 tokens of 9 x 16 heads with every segment on this path: 507 us taken pair
 // by pair, 125 us with the squares' products on CUDA cores, 94 us as tf32 fragments, 87 us with
-// the builders looking one segment ahead: 22 k cycles a segment, the decays, operands, scores,
-// update and outputs one after another (a segment's exponentials alone are ~2,300 warp
+// the builders looking one segment ahead, and 90.7 us since the fragments are rounded and summed
+// as exactly as pairs and infinities and NaN are kept: ~23 k cycles a segment, the decays, operands,
+// scores, update and outputs one after another (a segment's exponentials alone are ~2,300 warp
 // instructions, 4.6 k cycles of the special-function units).
 // Segments with a gate above 0 keep the pairwise form (exact_scores_pairs), and segments with a
 // score that comes out infinite or NaN fall back to it.
@@ -841,7 +844,8 @@ struct Factors {
 };
 
 template <int D, int SIGN>
-__device__ __forceinline__ Factors factors4(const uint8_t *smem, uint32_t off, int row, const float4 &r, int kk)
+__device__ __forceinline__ Factors factors4(const uint8_t *smem, uint32_t off, int row, const float4 &r,
+                                            int kk)
 {
     const float *sLam = reinterpret_cast<const float *>(smem + X_LAM);
     const float4 l = *reinterpret_cast<const float4 *>(sLam + lam_at<D>(row, kk));
@@ -1261,7 +1265,8 @@ __device__ __forceinline__ void fast_issue_update(uint32_t tmem, uint32_t sb, in
 // update S in TMEM, write the slot and the largest |S|, and leave each token's group partials
 // in the operand sets) ...
 template <int D>
-__device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L, int vb, float *slot, int mset)
+__device__ __forceinline__ void short_state(uint8_t *smem, uint32_t tmem, int L, int vb, float *slot,
+                                            int mset)
 {
     constexpr int CW = Geo<D>::CW, NG = Geo<D>::NG;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;

@@ -37,8 +37,8 @@
 // 2^{Lam_last} stays >= 2^-10 in every key dim (so Q~ never nears fp16's
 // subnormals).  Any other chunk (strong decay, huge values) runs the exact
 // path: tf32 operands (the state split into two exact tf32 parts), the
-// intra-chunk matrix computed in float32 from factors 2^{Lam_i - Lam_j} <= 1,
-// and the state updated as
+// intra-chunk matrix formed as exactly as float32 sums from factors
+// 2^{Lam_i - Lam_j} <= 1 before it is rounded to tf32, and the state updated as
 // diag(2^{Lam_last}) S + K^^T V with K^_j = k_j 2^{Lam_last - Lam_j}.  The
 // choice depends only on the chunk's inputs and on the state it starts from,
 // as does every operation order, so a resumed run reproduces a full
@@ -72,10 +72,11 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const uint32_t sb = smem_u32(smem);
     float *sRed = reinterpret_cast<float *>(smem + OFF_RED);
-    // [0] TMEM base, [1] abort flag, [3] run result (1 = the segment at [4] needs the exact path), [4] token index where the
-    // run stopped, [5] whether that segment's build is whole (0: its gates alone send it to the
-    // exact path, its inputs still staged), [6..7] decisions on the latest segments (1 = fast),
-    // by segment, [9] an exact segment's look ahead, [10] its task counter, [11..12] whether the build of the latest segments is whole, by segment parity
+    // [0] TMEM base, [1] abort flag, [3] run result (1 = the segment at [4] needs the exact path),
+    // [4] token index where the run stopped, [5] whether that segment's build is whole (0: its gates
+    // alone send it to the exact path, its inputs still staged), [6..7] decisions on the latest
+    // segments (1 = fast), by segment, [9] an exact segment's look ahead, [10] its task counter,
+    // [11..12] whether the build of the latest segments is whole, by segment parity
     volatile uint32_t *sMisc = reinterpret_cast<volatile uint32_t *>(smem + OFF_MISC);
     const uint32_t bar_tma = sb + OFF_BAR, bar_a = sb + OFF_BAR + 8, bar_o = sb + OFF_BAR + 16,
                    bar_s = sb + OFF_BAR + 24, bar_built = sb + OFF_BAR + 32,
@@ -83,7 +84,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
 
     const int tid = threadIdx.x, warp = tid >> 5;
     // (signed: the unsigned division left the d = 128 kernel with 56 bytes of spills, which cost
-    // 4 to 5 % of every tail: 29.8 us, now 28.5, for 256 tokens of 9 x 16 heads)
+    // 4 to 5 % of every tail: 29.8 us instead of 28.5 for 256 tokens of 9 x 16 heads; now it has
+    // none, the output pass at d = 128 20 bytes)
     const int bh = blockIdx.x;
     const int b = bh / p.n_heads;
     const int h = bh - b * p.n_heads;
@@ -357,7 +359,8 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
                     sMisc[9] = exact ? 1u : 2u;
             }
         } else if (wait_group(2, kIssuer, bar_o, ph_o)) {
-            state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false, next_max());   // checkpoint and |S| of the final state
+            // checkpoint and |S| of the final state
+            state_pass<D>(smem, tmem, -1, ckpt_slot(seg_end), false, next_max());
             out_epilogue<D>(tmem, outp(tok_s), tstride, L, 0);
         }
         tc_fence_before();

@@ -34,7 +34,8 @@ constexpr int kChunk = 64;
 constexpr uint32_t kTmemCols = 256;
 constexpr uint32_t kTmV = 128;                // V^T: column = token
 // shared memory (from a 1024-byte aligned base): the K^ operand (d x 64 tf32) and the
-// staged segment; 97 KiB with the alignment slack, so at most two CTAs fit on an SM
+// staged segment; 97 KiB with the alignment slack (99 KiB with the decay totals), so at most two
+// CTAs fit on an SM
 constexpr uint32_t OFF_OP = 0;                // K^ operand, K-major, 128-byte swizzle  32 KiB
 constexpr uint32_t OFF_K = 32768;             // k  bf16 [64 tokens][d]                 16 KiB
 constexpr uint32_t OFF_V = 49152;             // v  bf16 [64][d]                        16 KiB

@@ -9,7 +9,7 @@
 // warp is 256 contiguous bytes of one row.  The kernel is bound by the state's bytes (a short
 // call reads and writes 64 KiB per head and computes a few tokens in between), so what matters
 // is that the loads of one CTA overlap the arithmetic and stores of others: 256 threads of 64
-// registers over 32 KiB of state put four CTAs on an SM.  72 problems of 16 heads and 2-8
+// registers (8 bytes spilled) over 32 KiB of state put four CTAs on an SM.  72 problems of 16 heads and 2-8
 // tokens (160 MB): 29.5 us = 5.4 TB/s; 31.7 without the later CTAs' states requested into L2, 35.1
 // without the CTA's own lines requested first either (its tokens' alone: 32.9), and 38.2 us with
 // whole heads (16 x 4 blocks, 125 registers, two CTAs per SM) then.  Tokens are staged eight at a
@@ -188,9 +188,12 @@ gla_recurrent_kernel(const __grid_constant__ GlaParams p, unsigned ahead)
 cudaError_t launch_gla_recurrent(const GlaParams &p, int d, int sm_count, cudaStream_t s)
 {
     const unsigned grid = (unsigned)p.batch * (unsigned)p.n_heads * (unsigned)(d / kCols);
-    // each CTA requests the state three CTAs per SM further on (an SM holds four at d = 128, seven at
-    // d = 64).  72 problems of 16 heads, 2-8 tokens: 31.7 us without, 29.9 two, 29.5 three, 30.2 four,
-    // 31.7 five, 32.6 eight further; 32 problems of 32 heads, 1-2 tokens: 24.6, 22.7, 22.7, 22.8, 23.3, 24.1
+    // each CTA requests the state three CTAs per SM further on at d = 128 (an SM holds four), five at
+    // d = 64 (seven).  d = 128, 72 problems of 16 heads, 2-8 tokens: 31.7 us without, 29.9 two, 29.5
+    // three, 30.2 four, 31.7 five, 32.6 eight further; 32 problems of 32 heads, 1-2 tokens: 24.6, 22.7,
+    // 22.7, 22.8, 23.3, 24.1.  d = 64, 72 problems of 16 heads, 2-8 tokens: 10.24 us without, 9.98 two,
+    // 9.95 three, 9.92 four, 9.92 five, 9.88 six, 10.25 eight; 128 of 32 heads, 1-2 tokens: 22.6, 21.6,
+    // 21.2, 20.9, 20.7, 20.7, 20.8; 384 of 32 heads, 2-4 tokens: 64.9, 63.8, 63.6, 63.4, 63.3, 63.6, 65.4
     if (d == 128)
         return launch_pdl(gla_recurrent_kernel<128>, dim3(grid), dim3(256), 0, s, p, 3u * sm_count);
     return launch_pdl(gla_recurrent_kernel<64>, dim3(grid), dim3(128), 0, s, p, 5u * sm_count);

@@ -52,7 +52,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// First detected device-side problem wins; kernels never clear the word.
 // Launch a kernel that needs more than 48 KiB of dynamic shared memory.  Its limit is set
 // with cudaFuncSetAttribute on the first launch on each device (bit `dev` of `done`) instead
 // of on every call; if a launch still fails (the device's context was reset since), the
@@ -86,6 +85,7 @@ inline cudaError_t launch_pdl_big_smem(void (*kernel)(KArgs...), dim3 grid, dim3
     return launch_pdl(kernel, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
+// First detected device-side problem wins; kernels never clear the word.
 __device__ __forceinline__ void report(int32_t *d_err, int32_t code)
 {
     if (d_err != nullptr)
@@ -105,7 +105,8 @@ struct GlaParams {
     int32_t batch;
     int32_t n_heads;
     int32_t ckpt_interval;     // 0: none
-    int32_t stall_for_test;    // tensor-core kernel only: one wait that nothing completes (failure-detection tests)
+    int32_t stall_for_test;    // tensor-core kernel only: one wait that nothing completes
+                               // (failure-detection tests)
     int32_t off[HS_MAX_BATCH];      // absolute position of the first token within its chunk
     int32_t first_ck[HS_MAX_BATCH]; // tokens up to the problem's first checkpoint position (which
                                     // may lie past n_tokens); 0: no checkpoints
