@@ -1105,9 +1105,10 @@ __device__ __forceinline__ bool exact_scores_sum(uint8_t *smem)
 // pair by pair, for segments with a gate above 0 or a score that is not finite: one float32 chain per
 // score, a thread each.  Four key dims a step, since a warp's 32 keys lie in as many rows of the same
 // banks: by single elements tails of 512 tokens of 9 x 16 heads, every segment here, took 928 us, now
-// 511 (same bits).
+// 517 (same bits).  A call, not inlined: inlined it left the output pass at d = 128 with 28 bytes of
+// spills (4,608 tokens of 16 heads 93.5 us instead of 92.45).
 template <int D>
-__device__ __forceinline__ void exact_scores_pairs(uint8_t *smem, int L)
+__device__ __noinline__ void exact_scores_pairs(uint8_t *smem, int L)
 {
     const int tid = thread_id();
     const float *lg = reinterpret_cast<const float *>(smem + X_LAM);

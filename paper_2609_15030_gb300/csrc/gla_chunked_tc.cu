@@ -84,8 +84,7 @@ gla_chunked_tc_kernel(const __grid_constant__ GlaParams p, const __grid_constant
 
     const int tid = threadIdx.x, warp = tid >> 5;
     // (signed: the unsigned division left the d = 128 kernel with 56 bytes of spills, which cost
-    // 4 to 5 % of every tail: 29.8 us instead of 28.5 for 256 tokens of 9 x 16 heads; now it has
-    // none, the output pass at d = 128 20 bytes)
+    // 4 to 5 % of every tail: 29.8 us instead of 28.5 for 256 tokens of 9 x 16 heads)
     const int bh = blockIdx.x;
     const int b = bh / p.n_heads;
     const int h = bh - b * p.n_heads;
