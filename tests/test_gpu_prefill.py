@@ -14,7 +14,7 @@ import oracle
 import paper_2609_15030_gb300 as hs
 from hs_inputs import (LONG24, LONG_LENGTHS, SWEEP, SWEEP_LENGTHS, TINY, bf16_bits_to_f32,
                        f32_to_bf16_bits, gen_linear, gen_state)
-from tests.gpu_helpers import TOL, device, maxnorm_err, run_prefill, to_dev
+from tests.gpu_helpers import TOL, device, maxnorm_err, run_prefill, run_scan_prefill, to_dev
 
 pytestmark = pytest.mark.gpu
 KERNELS = [pytest.param(hs.HS_LINATTN_RECURRENT, id="recurrent"),
@@ -337,6 +337,8 @@ def test_fast_runs_ended_by_magnitude(d, p0, tail):
     o, S, cks = run_prefill(inp, [p0] * 2, [n] * 2, S0, 64, dev, hs.HS_LINATTN_CHUNKED_TC)
     ref = oracle.gla(inp.q, inp.k, inp.v, inp.a, [p0] * 2, [n] * 2, S0=S0, C_=64, threads=16)
     _check(o, S, cks, *ref, [p0] * 2, [n] * 2, "runs")
+    # the output pass of the segment-parallel form, several segments to a CTA
+    _check(*run_scan_prefill(inp, [p0] * 2, [n] * 2, S0, 64, dev), *ref, [p0] * 2, [n] * 2, "spans")
     for m in range(1, len(cks[0]), 3):
         c = (p0 // 64 + 1 + m) * 64 - p0
         if c >= n:
